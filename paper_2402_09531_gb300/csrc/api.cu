@@ -65,6 +65,19 @@ void Plan::free_tree() {
   bq32.release();
   bqm32.release();
   near_parts64.release();
+  fx_state = -1;
+  fx_sym = -1;
+  fx_chunks = 0;
+  fx_parts = false;
+  fx_chunk_t.release();
+  fx_chunk_ptr.release();
+  h_upcount.clear();
+  fx_pts.release();
+  fx_nodes.release();
+  fx_q.release();
+  fx_qm.release();
+  fx_qs.release();
+  fx_qms.release();
   sym_t.release();
   sym_s.release();
   sym_uprow.release();
@@ -125,6 +138,10 @@ void Plan::free_all() {
   far_vexp.release();
   far_vt_ok = false;
   d_err.release();
+  fx_table.release();
+  fx_flag.release();
+  fx_colmax.release();
+  fx_colscale.release();
   stage_in.release();
   stage_out.release();
   for (auto& r : tm.recs) {
@@ -311,14 +328,10 @@ dwfmm_status dwfmm_tree_build(dwfmm_plan plan, const double* pts, int64_t n, int
     P.gauss_fact = false;
     P.gauss_bound = 0.0;
     if (P.kernel == DWFMM_K_GAUSS && n > 0) {
-      std::vector<double> lo(P.d), hi(P.d);
-      DW_CUDA(cudaMemcpyAsync(lo.data(), P.d_lo.p, sizeof(double) * P.d, cudaMemcpyDeviceToHost, P.stream));
-      DW_CUDA(cudaMemcpyAsync(hi.data(), P.d_hi.p, sizeof(double) * P.d, cudaMemcpyDeviceToHost, P.stream));
-      DW_CUDA(cudaStreamSynchronize(P.stream));
       const double s2 = 1.4426950408889634 / (2.0 * P.sigma * P.sigma);
       double b = 0.0;
       for (int k = 0; k < P.d; ++k) {
-        const double m = std::max(std::fabs(lo[k]), std::fabs(hi[k]));
+        const double m = std::max(std::fabs(P.h_lo0[k]), std::fabs(P.h_hi0[k]));
         b += m * m * s2;
       }
       P.gauss_fact = b <= 30.0;

@@ -186,6 +186,81 @@ struct PersistArgs {
 };
 
 
+namespace ks {
+// Rows of one side of a sum (ksum.cuh).
+struct Side {
+  int64_t gstride;   // elements between groups
+  int ld;            // elements between coordinate rows (or rhs rows)
+  const int32_t* count;
+  int count_off;
+  int count_const;   // used when count == nullptr
+};
+}  // namespace ks
+
+// Fixed-point float64 kernel summation (fix64.cuh, sum_fix.cuh).
+namespace fx {
+
+struct Consts {
+  unsigned long long K;   // scale of w: sqrt(T) (exp, Matern) or T (Gaussian) -> w 2^57
+};
+
+struct FixArgs {
+  const int4* rec;               // point records [group][ld][2 DM], targets and sources
+  const int2* q;                 // charge limbs [group][ld][RC]
+  const double* qscale;          // [group][16]
+  const unsigned long long* table;
+  Consts c;
+  const int32_t* rowptr;
+  const int32_t* col;
+  int first, ld, Rc;
+  int passes, tp, nsub;          // passes of tp targets, threads per target
+  int group_entries;             // source groups per stage (short groups), 0: chunks of one group
+  int splits;                    // parts of each list; part p writes at out + p * split_stride
+  int64_t split_stride;
+  double* out;                   // [group][16][ld]
+  int64_t o_gstride;
+  const int* flag;               // != 0: a charge is not finite or below 2^-960, sum in float64
+  // the float64 path's view of the same data; side also holds the group sizes
+  int d;
+  double inv_sigma;
+  const double* coord;
+  ks::Side side;
+  const double* charge;
+  int64_t q_gstride;
+};
+
+// Symmetric form: each unordered pair of near leaves once (sum_fix.cuh).
+struct FixSymArgs {
+  const int4* rec;               // leaf records [leaf][ld][2 DM]
+  const int2* q;                 // charge limbs [leaf][ld][RC], one scale per column
+  const double* qscale;          // [16]
+  const unsigned long long* table;
+  Consts c;
+  const int32_t* count;          // [leaf]
+  const int32_t* chunk_t;        // [chunk] target leaf
+  const int32_t* chunk_ptr;      // [leaf + 1] first chunk of a leaf's row
+  const int32_t* uprow;          // [leaf + 1] upper entries (t, s >= t)
+  const int32_t* up_s;
+  int ld, Rc, cmax;              // slots, right-hand sides, largest leaf
+  int batches;                   // batches of 64 sources per warp
+  double* pf;                    // [chunk][Rc][ld] sums for the row's targets
+  double* pt;                    // [entry][Rc][ld] sums for the entry's sources
+  const int* flag;
+  int d;
+  double inv_sigma;
+  const double* coord;           // [leaf][d][ld]
+  const double* charge;          // [leaf][16][ld]
+};
+
+void launch_fix_exp(int d, int RC, const FixArgs& a, int ctas, cudaStream_t s);
+void launch_fix_matern(int d, int RC, const FixArgs& a, int ctas, cudaStream_t s);
+void launch_fix_gauss(int d, int RC, const FixArgs& a, int ctas, cudaStream_t s);
+void launch_fix_sym_exp(int d, int RC, const FixSymArgs& a, int chunks, cudaStream_t s);
+void launch_fix_sym_matern(int d, int RC, const FixSymArgs& a, int chunks, cudaStream_t s);
+void launch_fix_sym_gauss(int d, int RC, const FixSymArgs& a, int chunks, cudaStream_t s);
+
+}  // namespace fx
+
 struct TreeDev {
   int64_t N;
   int J;
@@ -312,6 +387,25 @@ struct Plan {
   // solve workspace
   DBuf<double> cg_r, cg_p, cg_ap, cg_c, cg_f, cg_dot, cg_tmp;
 
+  // fixed-point float64 sums (sum_fix.cu): -1 = not looked at for this tree,
+  // 0 = the box or the kernel's range does not fit, 1 = records are built
+  int fx_state = -1;
+  int fx_F = 0;
+  fx::Consts fx_c{};
+  double h_lo0[kMaxDim] = {0}, h_hi0[kMaxDim] = {0};   // root box
+  DBuf<int> fx_pts, fx_nodes, fx_q, fx_qm;
+  DBuf<double> fx_qs, fx_qms;
+  DBuf<unsigned long long> fx_table;
+  DBuf<int> fx_flag;   // near field, couplings: sum in float64 (cleared by the scatter)
+  DBuf<unsigned long long> fx_colmax;   // [16] largest |x| of each column, as bits (cleared by the scatter)
+  DBuf<double> fx_colscale;             // [16]
+  // symmetric form: row chunks of the upper near entries (batches of 64
+  // sources per warp), built for the tree
+  int fx_sym = -1, fx_chunks = 0, fx_batches = 0, fx_cmax = 0;
+  DBuf<int32_t> fx_chunk_t, fx_chunk_ptr;
+  bool fx_parts = false;   // the last near field left its sums in sym_pf / sym_pt
+  std::vector<int> h_upcount;   // upper near entries per leaf
+
   // scratch for tree build
   DBuf<unsigned char> scratch;
 
@@ -394,7 +488,9 @@ void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy
 void ensure_workspace(Plan& P, bool fp64);
 void farfield_set_smem_limits(Plan& P);
 size_t farfield_smem_need(const Plan& P, bool fp64);
-void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64);
+// colmax: also the columns' largest magnitudes (float64 sums in fixed point;
+// the scatter of the same pass clears them)
+void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64, bool colmax = false);
 void launch_scatter(Plan& P, double* y, int64_t ldy, int r0, int Rc, bool fp64);
 void launch_farfield(Plan& P, int Rc, bool fp64);
 bool farfield_tc_eligible(const Plan& P);   // farfield_tc.cu
@@ -411,6 +507,9 @@ void m2l_autotune(Plan& P, int Rc);                         // p2p_f32.cu
 void build_far_sym_lists(Plan& P);                          // nearfield.cu
 bool near_sym_tc(Plan& P, int D, int Rc, cudaStream_t s);   // symmetric tensor-core P2P (MIXED, 9..16 RHS)
 int sm_count();
+bool fix_ready(Plan& P);                    // sum_fix.cu: fixed-point float64 sums
+bool near_fix(Plan& P, int Rc, cudaStream_t s);
+bool m2l_fix(Plan& P, int Rc);
 bool p2p_f32_tuned(Plan& P, int Rc, cudaStream_t s);
 bool m2l_f32_tuned(Plan& P, int Rc);
 void check_device_error(Plan& P);

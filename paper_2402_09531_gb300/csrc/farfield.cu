@@ -562,7 +562,8 @@ __global__ void __launch_bounds__(kPersistThreads, 3) k_batch_persistent(const _
 // x (caller order, column-major) -> xb[leaf][r][m_pad] for r in [r0, r0+Rc).
 template <typename T>
 __global__ void k_gather(const double* x, int64_t ldx, int r0, int Rc, const int32_t* perm,
-                         const int32_t* begin, const int32_t* count, int L, int m_pad, T* xb) {
+                         const int32_t* begin, const int32_t* count, int L, int m_pad, T* xb,
+                         unsigned long long* colmax) {
   const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const int64_t total = static_cast<int64_t>(L) * kRC * m_pad;
   if (t >= total) return;
@@ -574,13 +575,60 @@ __global__ void k_gather(const double* x, int64_t ldx, int r0, int Rc, const int
   T v = T(0);
   if (r < Rc && i < count[c]) v = static_cast<T>(x[static_cast<int64_t>(r0 + r) * ldx + perm[begin[c] + i]]);
   xb[t] = v;
+  if (colmax && r < Rc) {
+    // largest magnitude of each column; lanes of a warp may lie in two rows
+    const unsigned act = __activemask();
+    unsigned long long m = static_cast<unsigned long long>(__double_as_longlong(fabs(static_cast<double>(v))));
+    const unsigned same = __match_any_sync(act, r);
+    const unsigned hi = __reduce_max_sync(same, static_cast<unsigned>(m >> 32));
+    const unsigned lo = __reduce_max_sync(same, static_cast<unsigned>(m >> 32) == hi ? static_cast<unsigned>(m) : 0u);
+    m = (static_cast<unsigned long long>(hi) << 32) | lo;
+    if ((threadIdx.x & 31) == __ffs(same) - 1 && m > colmax[r]) atomicMax(colmax + r, m);
+  }
+}
+
+// Scatter of the symmetric fixed-point near field: y = the row's chunk sums,
+// then the transposed sums of its lower entries, each in list order, plus the
+// far field.
+__global__ void k_scatter_parts(double* y, int64_t ldy, int r0, int Rc, const int32_t* perm, const int32_t* begin,
+                                const int32_t* count, int L, int m_pad, const int32_t* chunk_ptr, const int32_t* lorow,
+                                const int32_t* lo_slot, const double* pf, const double* pt, const double* yfar,
+                                int has_far, int* flags, unsigned long long* colmax) {
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t < 2) flags[t] = 0;   // every sum that reads them is done
+  if (t < kRC) colmax[t] = 0;
+  if (t >= static_cast<int64_t>(L) * Rc * m_pad) return;
+  const int i = static_cast<int>(t % m_pad);
+  const int64_t lr = t / m_pad;
+  const int r = static_cast<int>(lr % Rc);
+  const int leaf = static_cast<int>(lr / Rc);
+  const int c = L - 1 + leaf;
+  if (i >= count[c]) return;
+  const int64_t at = static_cast<int64_t>(r) * m_pad + i, step = static_cast<int64_t>(Rc) * m_pad;
+  double v = 0.0;
+  for (int e = chunk_ptr[leaf]; e < chunk_ptr[leaf + 1]; ++e) v += pf[e * step + at];
+  const int ke = lorow[leaf + 1];
+  int k = lorow[leaf];
+  for (; k + 8 <= ke; k += 8) {   // independent loads, sums in list order
+    double w[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) w[u] = pt[lo_slot[k + u] * step + at];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v += w[u];
+  }
+  for (; k < ke; ++k) v += pt[lo_slot[k] * step + at];
+  if (has_far) v += yfar[(static_cast<int64_t>(leaf) * kRC + r) * m_pad + i];
+  y[static_cast<int64_t>(r0 + r) * ldy + perm[begin[c] + i]] = v;
 }
 
 template <typename T>
 __global__ void k_scatter(double* y, int64_t ldy, int r0, int Rc, const int32_t* perm,
                           const int32_t* begin, const int32_t* count, int L, int m_pad,
-                          const T* ynear, const T* yfar, int has_far) {
+                          const T* ynear, const T* yfar, int has_far, int* flags,
+                          unsigned long long* colmax) {
   const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (flags && t < 2) flags[t] = 0;   // every sum that reads them is done
+  if (colmax && t < kRC) colmax[t] = 0;
   const int64_t total = static_cast<int64_t>(L) * kRC * m_pad;
   if (t >= total) return;
   const int i = static_cast<int>(t % m_pad);
@@ -678,28 +726,34 @@ size_t farfield_smem_need(const Plan& P, bool fp64) {
   return std::max(a, b);
 }
 
-void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64) {
+void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64, bool colmax) {
   const int64_t total = static_cast<int64_t>(P.L) * kRC * P.m_pad;
   if (fp64)
     k_gather<double><<<ceil_div(total, 256), 256, 0, P.stream>>>(x, ldx, r0, Rc, P.d_perm.p, P.d_begin.p,
-                                                                 P.d_count.p, P.L, P.m_pad, P.xb64.p);
+                                                                 P.d_count.p, P.L, P.m_pad, P.xb64.p,
+                                                                 colmax ? P.fx_colmax.p : nullptr);
   else
     k_gather<float><<<ceil_div(total, 256), 256, 0, P.stream>>>(x, ldx, r0, Rc, P.d_perm.p, P.d_begin.p,
-                                                                P.d_count.p, P.L, P.m_pad, P.xb32.p);
+                                                                P.d_count.p, P.L, P.m_pad, P.xb32.p, nullptr);
   DW_CUDA(cudaGetLastError());
 }
 
 void launch_scatter(Plan& P, double* y, int64_t ldy, int r0, int Rc, bool fp64) {
   const int64_t total = static_cast<int64_t>(P.L) * kRC * P.m_pad;
   const int has_far = P.jmin <= P.J;
-  if (fp64)
+  if (fp64 && P.fx_parts)
+    k_scatter_parts<<<ceil_div(static_cast<int64_t>(P.L) * Rc * P.m_pad, 256), 256, 0, P.stream>>>(
+        y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad, P.fx_chunk_ptr.p, P.sym_lorow.p,
+        P.sym_loslot.p, P.sym_pf.p, P.sym_pt.p, P.yfar64.p, has_far, P.fx_flag.p, P.fx_colmax.p);
+  else if (fp64)
     k_scatter<double><<<ceil_div(total, 256), 256, 0, P.stream>>>(y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p,
                                                                   P.d_count.p, P.L, P.m_pad, P.ynear64.p,
-                                                                  P.yfar64.p, has_far);
+                                                                  P.yfar64.p, has_far, P.fx_flag.p,
+                                                                  P.fx_colmax.p);
   else
     k_scatter<float><<<ceil_div(total, 256), 256, 0, P.stream>>>(y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p,
                                                                  P.d_count.p, P.L, P.m_pad, P.ynear32.p,
-                                                                 P.yfar32.p, has_far);
+                                                                 P.yfar32.p, has_far, nullptr, nullptr);
   DW_CUDA(cudaGetLastError());
 }
 

@@ -64,12 +64,13 @@ void ensure_workspace(Plan& P, bool fp64) {
 void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy, int R, bool fp64) {
   if (P.N == 0 || R == 0) return;
   ensure_workspace(P, fp64);
+  const bool fix = fp64 && fix_ready(P);   // the tree's records, before the side stream forks
   cudaStream_t s = P.stream;
   timer_begin(P, 6, s);
   for (int r0 = 0; r0 < R; r0 += kRC) {
     const int Rc = std::min(kRC, R - r0);
     timer_begin(P, 0, s);
-    launch_gather(P, x, ldx, r0, Rc, fp64);
+    launch_gather(P, x, ldx, r0, Rc, fp64, fix);
     timer_end(P, 0, s, 1);
     if (!fp64) m2l_autotune(P, Rc);   // once per tree, before the near field starts
     if (P.tm.on && P.tm.serialize) {  // every phase alone on the caller's stream

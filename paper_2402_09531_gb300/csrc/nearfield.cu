@@ -6,8 +6,10 @@
 //        of every s with (c, s) in the farfield F, charges = m_s; this is
 //        l_c = sum_s S_{c,s} m_s with the coupling matrices of Sec. 5.2.
 // One CTA per target group, one thread per target, sources staged through
-// shared memory in chunks.  This generic kernel serves float64 (parity) and
-// the fallback float32 shapes; the tuned float32 P2P lives in p2p_f32.cu.
+// shared memory in chunks.  This generic kernel serves the fallback float32
+// shapes (the tuned float32 P2P lives in p2p_f32.cu) and the float64 sums that
+// the fixed-point kernels (sum_fix.cu) do not take: d > 16, boxes beyond about
+// 22 length scales.
 //
 // The float64 P2P has a symmetric form as well: phi is symmetric and so is
 // the near relation, so each unordered pair of near leaves (T, S) is
@@ -23,6 +25,7 @@
 #include <vector>
 
 #include "dwfmm_internal.cuh"
+#include "ksum.cuh"
 
 namespace dw {
 
@@ -40,29 +43,8 @@ int sm_count() {
 
 namespace {
 
-constexpr int kThreads = 128;
-constexpr int kSrcChunk = 128;
+using namespace ks;
 
-template <typename T, int KER>
-__device__ __forceinline__ T phi_r2(T r2, T inv_sigma) {
-  if (KER == DWFMM_K_GAUSS) return exp(T(-0.5) * r2 * inv_sigma * inv_sigma);
-  const T s = sqrt(r2) * inv_sigma;
-  if (KER == DWFMM_K_EXP) return exp(-s);
-  const T t = T(1.7320508075688772) * s;
-  return (T(1) + t) * exp(-t);
-}
-
-struct Side {
-  int64_t gstride;   // elements between groups
-  int ld;            // elements between coordinate rows (or rhs rows)
-  const int32_t* count;
-  int count_off;
-  int count_const;   // used when count == nullptr
-};
-
-// DM: compile-time bound on d (coordinates beyond d are zero, so the extra
-// terms of the squared distance are exactly 0); RC: right-hand sides held in
-// registers (rows beyond Rc are zero charges).
 // splits > 1: CTA blockIdx.x handles part (blockIdx.x % splits) of group
 // blockIdx.x / splits's list and writes its partial sums to out + part *
 // split_stride (the caller adds the parts in a fixed order).
@@ -78,51 +60,10 @@ k_ksum(int first_group, const int32_t* rowptr, const int32_t* col, int d, T inv_
   const int r0 = rowptr[g], len = rowptr[g + 1] - r0;
   const int rb = r0 + static_cast<int>((static_cast<int64_t>(len) * part) / splits);
   const int re = r0 + static_cast<int>((static_cast<int64_t>(len) * (part + 1)) / splits);
-  out += part * split_stride;
-  const int tcnt = ts.count ? ts.count[ts.count_off + g] : ts.count_const;
-  for (int tb = 0; tb < ts.ld; tb += kThreads) {
-    const int i = tb + threadIdx.x;
-    T xt[DM];
-#pragma unroll
-    for (int k = 0; k < DM; ++k)
-      xt[k] = (k < d && i < tcnt) ? tcoord[g * ts.gstride + static_cast<int64_t>(k) * ts.ld + i] : T(0);
-    T acc[RC];
-#pragma unroll
-    for (int r = 0; r < RC; ++r) acc[r] = T(0);
-    for (int e = rb; e < re; ++e) {
-      const int s = col[e];
-      const int scnt = ss.count ? ss.count[ss.count_off + s] : ss.count_const;
-      for (int cb = 0; cb < scnt; cb += kSrcChunk) {
-        const int cn = min(kSrcChunk, scnt - cb);
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < DM * kSrcChunk; idx += kThreads) {
-          const int k = idx / kSrcChunk, j = idx % kSrcChunk;
-          sc[idx] = (j < cn && k < d) ? scoord[s * ss.gstride + static_cast<int64_t>(k) * ss.ld + cb + j] : T(0);
-        }
-        for (int idx = threadIdx.x; idx < RC * kSrcChunk; idx += kThreads) {
-          const int r = idx / kSrcChunk, j = idx % kSrcChunk;
-          sqs[idx] = (j < cn && r < Rc) ? sq[s * sq_gstride + static_cast<int64_t>(r) * sq_ld + cb + j] : T(0);
-        }
-        __syncthreads();
-        for (int j = 0; j < cn; ++j) {
-          T r2 = T(0);
-#pragma unroll
-          for (int k = 0; k < DM; ++k) {
-            const T df = xt[k] - sc[k * kSrcChunk + j];
-            r2 += df * df;
-          }
-          const T ph = phi_r2<T, KER>(r2, inv_sigma);
-#pragma unroll
-          for (int r = 0; r < RC; ++r) acc[r] += ph * sqs[r * kSrcChunk + j];
-        }
-      }
-    }
-    if (i < o_ld) {
-#pragma unroll
-      for (int r = 0; r < RC; ++r)
-        if (r < Rc) out[g * o_gstride + static_cast<int64_t>(r) * o_ld + i] = acc[r];
-    }
-  }
+  for (int tb = 0; tb < ts.ld; tb += kThreads)
+    ksum_targets<T, KER, DM, RC>(g, tb + static_cast<int>(threadIdx.x), o_ld, rb, re, col, d, inv_sigma, tcoord, ts,
+                                 scoord, ss, sq, sq_gstride, sq_ld, out + part * split_stride + g * o_gstride, o_ld,
+                                 Rc, sc, sqs);
 }
 
 template <typename T, int KER, int DM>
@@ -493,6 +434,7 @@ void build_sym_lists(Plan& P) {
   if (hbad) return;
   P.sym_nup = nup;
   P.sym_ok = true;
+  P.h_upcount = hu;
   sym_tc_order(P, hu);
 }
 
@@ -570,7 +512,7 @@ void launch_m2l(Plan& P, int Rc, bool fp64) {
   if (P.jmin > P.J) return;
   if (fp64) {
     P.m2l_engine = 0;
-    m2l_impl<double>(P, Rc, P.d_ynode64.p, P.mom64.p, P.loc64.p);
+    if (!m2l_fix(P, Rc)) m2l_impl<double>(P, Rc, P.d_ynode64.p, P.mom64.p, P.loc64.p);
   } else if (!m2l_f32_tuned(P, Rc)) {
     P.m2l_engine = 1;
     m2l_impl<float>(P, Rc, P.d_ynode32.p, P.mom32.p, P.loc32.p);
@@ -580,6 +522,7 @@ void launch_m2l(Plan& P, int Rc, bool fp64) {
 
 void launch_nearfield(Plan& P, int Rc, bool fp64, cudaStream_t s) {
   if (fp64) {
+    if (near_fix(P, Rc, s)) return;
     P.near_engine = 1;
     if (!near_sym(P, Rc, s)) {
       P.near_engine = 0;

@@ -712,6 +712,8 @@ void build_cluster_data(Plan& P) {
     k_leaf_block<<<ceil_div(np, 256), 256, 0, s>>>(reinterpret_cast<const double*>(P.scratch.p), P.N, d,
                                                    P.d_begin.p, P.d_count.p, P.L, P.m_pad, P.d_pts64.p,
                                                    P.d_pts32.p);
+  DW_CUDA(cudaMemcpyAsync(P.h_lo0, P.d_lo.p, sizeof(double) * d, cudaMemcpyDeviceToHost, s));
+  DW_CUDA(cudaMemcpyAsync(P.h_hi0, P.d_hi.p, sizeof(double) * d, cudaMemcpyDeviceToHost, s));
   DW_CUDA(cudaGetLastError());
   DW_CUDA(cudaStreamSynchronize(s));
   P.scratch.release();

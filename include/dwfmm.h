@@ -254,12 +254,14 @@ dwfmm_status dwfmm_evaluate(dwfmm_plan plan, const double* targets, int64_t nt, 
  * kernel, index-set size |Lambda| and leaf block size (equal leaf_size and
  * N >= leaf_size), d <= 16 and precision FP32 or MIXED; nrhs[i] (1..16) is
  * the number of right-hand sides of problem i for every later call.  The
- * near field of all problems is one launch of the kernel-summation engine,
- * the couplings (M2L) of all problems another, the upward and downward
- * passes one launch per tree height/level; the launch shape of each of the
- * two fused launches (CTA width; one padded launch or one per right-hand-side
- * class) is chosen by timing every candidate on the batch's data, and the
- * whole sequence is captured as a CUDA graph.
+ * near field of a right-hand-side class (1, up to 4, up to 8; symmetric lists,
+ * leaves of 32 to 256 sites) is one launch that evaluates each unordered pair
+ * once, otherwise one launch of the kernel-summation engine; the couplings
+ * (M2L) of all problems are another, the upward and downward passes one launch
+ * per tree height/level; the launch shape of the kernel-summation launches
+ * (CTA width; one padded launch or one per right-hand-side class) is chosen by
+ * timing every candidate on the batch's data, and the whole sequence is
+ * captured as a CUDA graph.
  * The plans must stay alive and keep their trees while the batch exists.
  * Synchronises `stream` before it starts.
  * dwfmm_batch_matvec: y[i] = K_tilde_i x[i] for every problem, x[i] and y[i]

@@ -67,10 +67,14 @@ void Plan::free_tree() {
   near_parts64.release();
   fx_state = -1;
   fx_sym = -1;
-  fx_chunks = 0;
-  fx_parts = false;
-  fx_chunk_t.release();
-  fx_chunk_ptr.release();
+  fx_rows.t.release();
+  fx_rows.ptr.release();
+  rot_state = -1;
+  rot.t.release();
+  rot.ptr.release();
+  rot_pf.release();
+  rot_pt.release();
+  near_parts = 0;
   h_upcount.clear();
   fx_pts.release();
   fx_nodes.release();

@@ -38,8 +38,16 @@ struct Batch {
   size_t far_smem = 0;
   struct Cls {
     int RC, leaf_first, leaf_count, clus_first, clus_count;
+    // near field: each unordered pair once (p2p_rot.cuh); its chunks, its
+    // first upper entry, and where its partial sums start
+    bool by_pair = false;
+    int chunk0 = 0, chunks = 0, e_base = 0;
+    size_t pf_off = 0, pt_off = 0;
   };
   std::vector<Cls> classes;
+  bool by_pair = false;          // some class is
+  DBuf<float> rot_pf, rot_pt;
+  DBuf<int32_t> uprow, up_s, lorow, lo_slot, chunk_t, chunk_ptr, cmax_of;   // over all leaves of the batch
   bool split = false;            // near field: one launch per right-hand-side class
   double tune_ms[2] = {0, 0};    // best padded / best per-class time of near field + couplings
   // tile shapes chosen by the autotuner: CTA width (targets per pass = 2 x
@@ -128,6 +136,31 @@ SumArgs p2p_args(Batch& B, int RC, int leaf_first) {
   return a;
 }
 
+RotArgs rot_args(Batch& B, const Batch::Cls& c) {
+  RotArgs a{};
+  a.pts = B.ptsk.p;
+  a.q = B.xq.p;
+  a.count = B.counts.p;
+  a.chunk_t = B.chunk_t.p;
+  a.chunk_ptr = B.chunk_ptr.p;
+  a.uprow = B.uprow.p;
+  a.up_s = B.up_s.p;
+  a.ld = B.ld;
+  a.Rc = c.RC;
+  a.cmax_of = B.cmax_of.p;
+  a.e_base = c.e_base;
+  a.chunk0 = c.chunk0;
+  a.pf = B.rot_pf.p + c.pf_off;
+  a.pt = B.rot_pt.p + c.pt_off;
+  return a;
+}
+
+BatchParts batch_parts(const Batch& B) {
+  BatchParts b{};
+  if (B.by_pair) b = BatchParts{B.chunk_ptr.p, B.lorow.p, B.lo_slot.p};
+  return b;
+}
+
 SumArgs m2l_args(Batch& B, int RC, int clus_first) {
   SumArgs a{};
   a.tgt = B.ynodek.p;
@@ -153,9 +186,10 @@ SumArgs m2l_args(Batch& B, int RC, int clus_first) {
 int threads_for(int ld) { return std::min(128, round_up((ld + 1) / 2, 32)); }
 
 // The fused near-field work: interleave charges, P2P launch(es) with
-// `threads` per CTA.
+// `threads` per CTA.  Classes whose pairs are evaluated once have launches of
+// their own (one shape).
 void enqueue_near(Batch& B, bool split, int threads, cudaStream_t s) {
-  if (!split) {
+  if (!split && !B.by_pair) {
     launch_interleave(B.xb.p, B.Ltot, B.ld, B.RCmax, B.xq.p, s);
     launch_sum_f32(B.D, B.kernel, B.RCmax, p2p_args(B, B.RCmax, 0), B.Ltot, threads,
                    sum_stage_bytes(B.D, B.RCmax, B.ld), s);
@@ -164,6 +198,10 @@ void enqueue_near(Batch& B, bool split, int threads, cudaStream_t s) {
   for (const auto& c : B.classes) {
     launch_interleave(B.xb.p + static_cast<int64_t>(c.leaf_first) * kRC * B.ld, c.leaf_count, B.ld, c.RC,
                       B.xq.p + static_cast<int64_t>(c.leaf_first) * B.ld * c.RC, s);
+    if (c.by_pair) {
+      launch_rot(B.D, B.kernel, c.RC, rot_args(B, c), c.chunks, s);
+      continue;
+    }
     launch_sum_f32(B.D, B.kernel, c.RC, p2p_args(B, c.RC, c.leaf_first), c.leaf_count, threads,
                    sum_stage_bytes(B.D, c.RC, B.ld), s);
   }
@@ -212,7 +250,9 @@ void enqueue_matvec(Batch& B, bool io = true) {
   for (size_t j = 0; j < B.down_off.size(); ++j)
     launch_downward_batched(B.probs.p, B.work.p + B.down_off[j], B.down_cnt[j], B.far_smem, s);
   DW_CUDA(cudaStreamWaitEvent(s, B.ev_join, 0));
-  if (io) launch_scatter_batched(B.probs.p, B.d_leaf_off.p, B.P, B.Ltot, B.ld, B.ynear.p, B.yfar.p, s);
+  if (io)
+    launch_scatter_batched(B.probs.p, B.d_leaf_off.p, B.P, B.Ltot, B.ld, *std::max_element(B.R.begin(), B.R.end()),
+                           batch_parts(B), B.ynear.p, B.yfar.p, s);
   DW_CUDA(cudaGetLastError());
 }
 
@@ -252,7 +292,11 @@ void tune_shapes(Batch& B) {
     double best = 1e30, bp = 1e30, bs = 1e30;
     bool bsplit = false;
     int bthr = widest;
-    for (int thr = 32; thr <= widest; thr = (thr * 2 > widest && thr < widest) ? widest : thr * 2) {
+    if (which == 0 && B.by_pair) {   // one shape: a launch per class, whole CTAs
+      best = bp = bs = time_shape(B, which, can_split, widest);
+      bsplit = can_split;
+    }
+    for (int thr = which == 0 && B.by_pair ? widest + 1 : 32; thr <= widest; thr = (thr * 2 > widest && thr < widest) ? widest : thr * 2) {
       for (int sp = 0; sp < (can_split ? 2 : 1); ++sp) {
         const double ms = time_shape(B, which, sp != 0, thr);
         if (sp) bs = std::min(bs, ms);
@@ -305,6 +349,7 @@ bool build_persist_args(Batch& B, int gs_near, int gs_m2l) {
   a.xb = B.xb.p;
   a.ynear = B.ynear.p;
   a.yfar = B.yfar.p;
+  a.parts = batch_parts(B);
   a.nup = static_cast<int>(B.up_off.size());
   a.ndown = static_cast<int>(B.down_off.size());
   for (int h = 0; h < a.nup; ++h) {
@@ -316,6 +361,7 @@ bool build_persist_args(Batch& B, int gs_near, int gs_m2l) {
     a.down_cnt[j] = B.down_cnt[j];
   }
   int rcn = 1, rcm = 1;
+  size_t rot_bytes = 0;
   // the largest right-hand-side class first: the longest items leave the queue first
   for (auto it = B.classes.rbegin(); it != B.classes.rend(); ++it) {
     const Batch::Cls& c = *it;
@@ -323,16 +369,24 @@ bool build_persist_args(Batch& B, int gs_near, int gs_m2l) {
       PersistSeg& sg = a.near[a.nnear++];
       sg.a = p2p_args(B, c.RC, c.leaf_first);
       sg.rc = c.RC;
-      sg.count = c.leaf_count;
+      sg.groups = c.leaf_count;
       sg.ilv_src = B.xb.p;
-      a.near_total += c.leaf_count;
-      rcn = std::max(rcn, c.RC);
+      if (c.by_pair) {
+        sg.by_pair = 1;
+        sg.r = rot_args(B, c);
+        sg.count = c.chunks;
+        rot_bytes = std::max(rot_bytes, persist_rot_bytes(B.D, c.RC, B.ld));
+      } else {
+        sg.count = c.leaf_count;
+        rcn = std::max(rcn, c.RC);
+      }
+      a.near_total += sg.count;
     }
     if (c.clus_count > 0) {
       PersistSeg& sg = a.m2l[a.nm2l++];
       sg.a = m2l_args(B, c.RC, c.clus_first);
       sg.rc = c.RC;
-      sg.count = c.clus_count;
+      sg.count = sg.groups = c.clus_count;
       sg.ilv_src = B.mom.p;
       a.m2l_total += c.clus_count;
       rcm = std::max(rcm, c.RC);
@@ -345,7 +399,7 @@ bool build_persist_args(Batch& B, int gs_near, int gs_m2l) {
   a.m2l_group_bytes = static_cast<int>(gm);
   a.sync = B.psync.p;
   a.err = B.err.p;
-  B.psmem = std::max({B.far_smem, static_cast<size_t>(kPersistThreads / gs_near) * gn,
+  B.psmem = std::max({B.far_smem, rot_bytes, static_cast<size_t>(kPersistThreads / gs_near) * gn,
                       static_cast<size_t>(kPersistThreads / gs_m2l) * gm});
   if (B.psmem > 227 * 1024) return false;
   const int per_sm = persist_blocks_per_sm(B.D, B.kernel, B.psmem);
@@ -445,7 +499,8 @@ void tune_persistent(Batch& B) {
   const int widest = pow2_width(threads_for(B.ld));
   double best = 1e30;
   int best_gs = 0;
-  for (int gs = 32; gs <= widest; gs *= 2) {
+  // chunks of pairs take the whole CTA
+  for (int gs = B.by_pair ? kPersistThreads : 32; gs <= (B.by_pair ? kPersistThreads : widest); gs *= 2) {
     if (!build_persist_args(B, gs, gs_m2l)) continue;
     if (!capture_engine(B, true, false, &g, &e)) return;
     const double ms = time_exec(B, e);
@@ -467,6 +522,99 @@ void tune_persistent(Batch& B) {
   B.persist_ok = true;
   B.engine_ms[1] = best;
   B.persistent = best < B.engine_ms[0];
+}
+
+// Upper near lists of all problems over the batch's leaves (host copies).
+struct PairLists {
+  std::vector<int32_t> uprow{0}, up_s, lorow{0}, lo_slot, cmax_of;
+  std::vector<int> least;   // per problem: sites of its smallest leaf, 0 = no symmetric lists
+};
+
+void add_pair_lists(Batch& B, int i, PairLists& l) {
+  Plan& p = *B.plans[i];
+  const int32_t e0 = static_cast<int32_t>(l.up_s.size()), k0 = static_cast<int32_t>(l.lo_slot.size());
+  int least = 1 << 30, most = 0;
+  for (int t = 0; t < p.L; ++t) {
+    least = std::min(least, p.h_count[p.L - 1 + t]);
+    most = std::max(most, p.h_count[p.L - 1 + t]);
+  }
+  l.cmax_of.insert(l.cmax_of.end(), p.L, most);
+  if (!p.sym_ok) {
+    l.least.push_back(0);
+    l.uprow.insert(l.uprow.end(), p.L, e0);
+    l.lorow.insert(l.lorow.end(), p.L, k0);
+    return;
+  }
+  l.least.push_back(least);
+  std::vector<int32_t> up(p.L + 1), lo(p.L + 1), s(p.sym_nup), slot;
+  DW_CUDA(cudaMemcpy(up.data(), p.sym_uprow.p, sizeof(int32_t) * (p.L + 1), cudaMemcpyDeviceToHost));
+  DW_CUDA(cudaMemcpy(lo.data(), p.sym_lorow.p, sizeof(int32_t) * (p.L + 1), cudaMemcpyDeviceToHost));
+  DW_CUDA(cudaMemcpy(s.data(), p.sym_s.p, sizeof(int32_t) * p.sym_nup, cudaMemcpyDeviceToHost));
+  slot.resize(lo[p.L]);
+  if (lo[p.L] > 0)
+    DW_CUDA(cudaMemcpy(slot.data(), p.sym_loslot.p, sizeof(int32_t) * lo[p.L], cudaMemcpyDeviceToHost));
+  for (int t = 0; t < p.L; ++t) {
+    l.uprow.push_back(e0 + up[t + 1]);
+    l.lorow.push_back(k0 + lo[t + 1]);
+  }
+  for (int32_t v : s) l.up_s.push_back(v + B.leaf_off[i]);
+  for (int32_t v : slot) l.lo_slot.push_back(v + e0);
+}
+
+// Classes that evaluate each pair once: their chunks and partial sums.
+void setup_pairs(Batch& B, const PairLists& l) {
+  constexpr size_t kMost = size_t(8) << 30;   // bytes of partial sums
+  const int per = rot_sources_per_chunk();
+  std::vector<int32_t> ct, cp(B.Ltot + 1, 0);
+  size_t npf = 0, npt = 0;
+  for (auto& c : B.classes) {
+    int least = 1 << 30;
+    for (int i = 0; i < B.P; ++i)
+      if (B.leaf_off[i] >= c.leaf_first && B.leaf_off[i] < c.leaf_first + c.leaf_count)
+        least = std::min(least, l.least[i]);
+    c.chunk0 = static_cast<int>(ct.size());
+    c.e_base = l.uprow[c.leaf_first];
+    const size_t entries = static_cast<size_t>(l.uprow[c.leaf_first + c.leaf_count]) - c.e_base;
+    const size_t row = static_cast<size_t>(c.RC) * B.ld;
+    c.by_pair = rot_fits(B.ld, least, c.RC) && (npf + npt + (entries + entries / 4 + B.Ltot) * row) * sizeof(float) <= kMost;
+    for (int t = c.leaf_first; t < c.leaf_first + c.leaf_count; ++t) {
+      const int n = c.by_pair ? ceil_div(static_cast<int64_t>(l.uprow[t + 1] - l.uprow[t]) * l.cmax_of[t], per) : 0;
+      ct.insert(ct.end(), n, t);
+      cp[t + 1] = static_cast<int32_t>(ct.size());
+    }
+    c.chunks = static_cast<int>(ct.size()) - c.chunk0;
+    c.pf_off = npf;
+    c.pt_off = npt;
+    if (!c.by_pair) continue;
+    B.by_pair = true;
+    npf += static_cast<size_t>(c.chunks) * row;
+    npt += entries * row;
+  }
+  if (!B.by_pair) return;
+  auto put = [](DBuf<int32_t>& d, const std::vector<int32_t>& v) {
+    d.alloc(std::max<size_t>(v.size(), 1));
+    if (!v.empty()) DW_CUDA(cudaMemcpy(d.p, v.data(), v.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+  };
+  put(B.uprow, l.uprow);
+  put(B.up_s, l.up_s);
+  put(B.lorow, l.lorow);
+  put(B.lo_slot, l.lo_slot);
+  put(B.chunk_t, ct);
+  put(B.chunk_ptr, cp);
+  put(B.cmax_of, l.cmax_of);
+  B.rot_pf.alloc(std::max<size_t>(npf, 1));
+  B.rot_pt.alloc(std::max<size_t>(npt, 1));
+  for (const auto& c : B.classes)
+    for (int i = 0; c.by_pair && i < B.P; ++i)
+      if (B.leaf_off[i] >= c.leaf_first && B.leaf_off[i] < c.leaf_first + c.leaf_count) {
+        ProbF32& q = B.h_probs[i];
+        q.pf = B.rot_pf.p + c.pf_off;
+        q.pt = B.rot_pt.p + c.pt_off;
+        q.rc = c.RC;
+        q.chunk0 = c.chunk0;
+        q.e_base = c.e_base;
+      }
+  DW_CUDA(cudaMemcpy(B.probs.p, B.h_probs, sizeof(ProbF32) * B.P, cudaMemcpyHostToDevice));
 }
 
 }  // namespace
@@ -536,6 +684,7 @@ void batch_create(Batch& B, Plan* const* plans, const int32_t* nrhs, int count) 
   DW_CUDA(cudaMemsetAsync(B.mom.p, 0, nc * sizeof(float), s));
   // scaled blocks at the common padded dimension; global CSR lists
   std::vector<int32_t> nr(B.Ltot + 1, 0), fr(B.Ctot + 1, 0), ncol, fcol, cnt(B.Ltot);
+  PairLists pl;
   for (int i = 0; i < count; ++i) {
     Plan& p = *B.plans[i];
     launch_scaled_blocks(p.d_pts64.p, p.L, p.d, B.D, B.ld, B.kernel, p.sigma,
@@ -552,6 +701,7 @@ void batch_create(Batch& B, Plan* const* plans, const int32_t* nrhs, int count) 
       cnt[B.leaf_off[i] + l] = p.h_count[p.L - 1 + l];
     }
     for (int64_t e = 0; e < p.nnear; ++e) ncol.push_back(cl[e] + B.leaf_off[i]);
+    add_pair_lists(B, i, pl);
     for (int c = 0; c < p.C; ++c) fr[B.clus_off[i] + c + 1] = frp[c + 1] - frp[c];
     for (int64_t e = 0; e < p.nfar; ++e) fcol.push_back(fcl[e] + B.clus_off[i]);
   }
@@ -644,6 +794,7 @@ void batch_create(Batch& B, Plan* const* plans, const int32_t* nrhs, int count) 
                                    B.clus_off[k] - B.clus_off[i]});
     i = k;
   }
+  setup_pairs(B, pl);
   DW_CUDA(cudaStreamSynchronize(s));
   // autotune the P2P/M2L launch shape, then capture the whole matvec
   tune_shapes(B);

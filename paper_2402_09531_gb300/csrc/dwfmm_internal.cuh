@@ -120,6 +120,17 @@ struct ProbF32 {
   const double* x;        // caller, column-major, ldx
   double* y;
   int64_t ldx, ldy;
+  // near field as chunk and transposed sums (nullptr: in the row layout)
+  const float* pf;        // [chunk - chunk0][rc][m_pad]
+  const float* pt;        // [entry - e_base][rc][m_pad]
+  int rc, chunk0, e_base;
+};
+
+// Lists of a batch's leaves for the sums of ProbF32::pf, pt.
+struct BatchParts {
+  const int32_t* chunk_ptr;   // [leaves + 1]
+  const int32_t* lorow;       // [leaves + 1] lower entries (t, s < t)
+  const int32_t* lo_slot;     // position of (s, t) in the upper list
 };
 
 // Arguments of the float32 kernel summation (P2P and M2L), see p2p_f32.cu.
@@ -143,6 +154,23 @@ struct SumArgs {
   int* err;
 };
 
+// The float32 near field that evaluates each unordered pair once (p2p_rot.cuh).
+struct RotArgs {
+  const float* pts;          // scaled blocks [leaf][D + 1][ld] (coordinates, squared norm)
+  const float* q;            // charges [leaf][ld][RC]
+  const int32_t* count;      // [leaf]
+  const int32_t* chunk_t;    // [chunk] target leaf
+  const int32_t* chunk_ptr;  // [leaf + 1]
+  const int32_t* uprow;      // [leaf + 1]
+  const int32_t* up_s;
+  int ld, Rc;
+  int cmax;                  // slots an entry takes in its row's stream: the largest leaf,
+  const int32_t* cmax_of;    // or one value per leaf
+  int e_base, chunk0;        // first entry of pt, first chunk of pf
+  float* pf;                 // [chunk - chunk0][Rc][ld]
+  float* pt;                 // [entry - e_base][Rc][ld]
+};
+
 // The persistent batch matvec (one cooperative launch, farfield.cu): the
 // phases of the batch's fused matvec as work items of one kernel, separated
 // by grid-wide barriers with bounded waits.
@@ -160,8 +188,11 @@ constexpr int kPersistSync = 2 * kPersistMaxLev + 8;   // barrier counters, then
 struct PersistSeg {
   SumArgs a;
   int rc;
-  int count;
+  int count;                  // items: target groups, or chunks if by_pair
+  int groups;                 // target groups
   const float* ilv_src;
+  int by_pair;                // near field: each unordered pair once (r), by the whole CTA
+  RotArgs r;
 };
 
 struct PersistArgs {
@@ -172,6 +203,7 @@ struct PersistArgs {
   float* xb;                  // gathered right-hand sides [Ltot][16][ld]
   const float* ynear;
   const float* yfar;
+  BatchParts parts;
   int nup, ndown;
   int up_off[kPersistMaxLev], up_cnt[kPersistMaxLev];
   int down_off[kPersistMaxLev], down_cnt[kPersistMaxLev];
@@ -330,6 +362,12 @@ struct CgState {
   }
 };
 
+// Rows of the upper near list cut into chunks of sources.
+struct RowChunks {
+  int n = 0, cmax = 0;        // chunks, sites of the largest leaf
+  DBuf<int32_t> t, ptr;       // [n] target leaf, [leaves + 1] first chunk of a leaf
+};
+
 struct Plan {
   // configuration
   int d = 0, kernel = 0, wrule = 0, leaf = 0, M = 0, prec = 0, max_rhs = 0;
@@ -401,9 +439,16 @@ struct Plan {
   DBuf<double> fx_colscale;             // [16]
   // symmetric form: row chunks of the upper near entries (batches of 64
   // sources per warp), built for the tree
-  int fx_sym = -1, fx_chunks = 0, fx_batches = 0, fx_cmax = 0;
-  DBuf<int32_t> fx_chunk_t, fx_chunk_ptr;
-  bool fx_parts = false;   // the last near field left its sums in sym_pf / sym_pt
+  int fx_sym = -1, fx_batches = 0;
+  RowChunks fx_rows;
+  // float32 near field, each unordered pair once (p2p_rot.cu): -1 = not
+  // looked at for this tree, 0 = does not apply, 1 = chunks are built
+  int rot_state = -1;
+  RowChunks rot;
+  DBuf<float> rot_pf, rot_pt;
+  // where the last near field left its sums: 0 = ynear, 1 = chunk sums in
+  // sym_pf and transposed sums in sym_pt (float64), 2 = rot_pf, rot_pt (float32)
+  int near_parts = 0;
   std::vector<int> h_upcount;   // upper near entries per leaf
 
   // scratch for tree build
@@ -489,14 +534,16 @@ void ensure_workspace(Plan& P, bool fp64);
 void farfield_set_smem_limits(Plan& P);
 size_t farfield_smem_need(const Plan& P, bool fp64);
 // colmax: also the columns' largest magnitudes (float64 sums in fixed point;
-// the scatter of the same pass clears them)
-void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64, bool colmax = false);
+// the scatter of the same pass clears them); xq: also the float32 charges
+// interleaved, [leaf][m_pad][padded rows]
+void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64, bool colmax = false,
+                   float* xq = nullptr);
 void launch_scatter(Plan& P, double* y, int64_t ldy, int r0, int Rc, bool fp64);
 void launch_farfield(Plan& P, int Rc, bool fp64);
 bool farfield_tc_eligible(const Plan& P);   // farfield_tc.cu
 void farfield_tc(Plan& P, int Rc);
 void launch_m2l(Plan& P, int Rc, bool fp64);
-void launch_nearfield(Plan& P, int Rc, bool fp64, cudaStream_t s);
+void launch_nearfield(Plan& P, int Rc, bool fp64, bool rot, cudaStream_t s);
 // Bit of the current device in a per-device mask (kernel attributes are set
 // per device); devices beyond 63 get no bit, so their setup simply repeats.
 uint64_t device_bit();
@@ -507,10 +554,13 @@ void m2l_autotune(Plan& P, int Rc);                         // p2p_f32.cu
 void build_far_sym_lists(Plan& P);                          // nearfield.cu
 bool near_sym_tc(Plan& P, int D, int Rc, cudaStream_t s);   // symmetric tensor-core P2P (MIXED, 9..16 RHS)
 int sm_count();
+bool row_chunks(Plan& P, int per, int least, RowChunks& out);   // p2p_rot.cu
+bool rot_ready(Plan& P, int Rc);
+void near_rot(Plan& P, int D, int Rc, cudaStream_t s);
 bool fix_ready(Plan& P);                    // sum_fix.cu: fixed-point float64 sums
 bool near_fix(Plan& P, int Rc, cudaStream_t s);
 bool m2l_fix(Plan& P, int Rc);
-bool p2p_f32_tuned(Plan& P, int Rc, cudaStream_t s);
+bool p2p_f32_tuned(Plan& P, int Rc, bool rot, cudaStream_t s);
 bool m2l_f32_tuned(Plan& P, int Rc);
 void check_device_error(Plan& P);
 // batches (batch.cu uses these)
@@ -520,8 +570,12 @@ void launch_moments_batched(const ProbF32* probs, const int2* work, int items, s
 void launch_downward_batched(const ProbF32* probs, const int2* work, int items, size_t smem, cudaStream_t s);
 void launch_gather_batched(const ProbF32* probs, const int* leaf_off, int P, int Ltot, int ld, float* xb,
                            cudaStream_t s);
-void launch_scatter_batched(const ProbF32* probs, const int* leaf_off, int P, int Ltot, int ld, const float* ynear,
-                            const float* yfar, cudaStream_t s);
+void launch_scatter_batched(const ProbF32* probs, const int* leaf_off, int P, int Ltot, int ld, int Rmax,
+                            const BatchParts& parts, const float* ynear, const float* yfar, cudaStream_t s);
+void launch_rot(int D, int kernel, int RC, const RotArgs& a, int chunks, cudaStream_t s);   // p2p_rot.cu
+int rot_sources_per_chunk();
+bool rot_fits(int ld, int least, int rc);   // slots, sites of the smallest leaf, padded right-hand sides
+size_t persist_rot_bytes(int D, int RC, int ld);
 // persistent batch matvec: dynamic shared memory and resident CTAs per SM
 // for a launch, and the cooperative launch itself (false if the launch was
 // refused, e.g. by a stream capture that cannot hold it)

@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "dwfmm_internal.cuh"
+#include "p2p_rot.cuh"
 #include "sum_f32.cuh"
 
 namespace dw {
@@ -305,9 +306,124 @@ __global__ void k_gather_batched(const ProbF32* probs, const int* leaf_off, int 
   gather_elem(probs, leaf_off, P, ld, xb, t);
 }
 
-// Element t of y = near + far, written to the caller's order (t < Ltot * 16 * ld).
-__device__ __forceinline__ void scatter_elem(const ProbF32* probs, const int* leaf_off, int P, int ld,
-                                             const float* ynear, const float* yfar, int64_t t) {
+// Running sum: float32 values with compensation (the float64 unit is too
+// narrow for a conversion and an addition per value), float64 values plainly.
+template <typename T>
+struct Running;
+template <>
+struct Running<float> {
+  float s = 0.0f, c = 0.0f;
+  __device__ __forceinline__ void add(float v) {
+    const float y = v - c, t = s + y;
+    c = (t - s) - y;
+    s = t;
+  }
+  __device__ __forceinline__ double value() const { return static_cast<double>(s) - static_cast<double>(c); }
+};
+template <>
+struct Running<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+
+// Part p of np of the near-field sums of one site: every np-th chunk sum of its
+// leaf's row (c0 .. c1 - 1) and a range of the transposed sums of its nlo lower
+// entries, `at` + index * step each.  Loads go out eight at a time.
+template <typename T>
+__device__ __forceinline__ double near_part(const T* pf, int c0, int c1, const T* pt, const int32_t* lo_slot, int nlo,
+                                            int e_base, int64_t at, int64_t step, int p, int np) {
+  Running<T> acc;
+  for (int e = c0 + p; e < c1; e += 4 * np) {
+    T w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) w[u] = e + u * np < c1 ? pf[(e + u * np) * step + at] : T(0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc.add(w[u]);
+  }
+  int k = static_cast<int>((static_cast<int64_t>(nlo) * p) / np);
+  const int ke = static_cast<int>((static_cast<int64_t>(nlo) * (p + 1)) / np);
+  for (; k < ke; k += 8) {
+    T w[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) w[u] = k + u < ke ? pt[(lo_slot[k + u] - e_base) * step + at] : T(0);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc.add(w[u]);
+  }
+  return acc.value();
+}
+
+constexpr int kPartThreads = 512;
+
+// y = near + far of right-hand side r of global leaf gl, written to the
+// caller's order, by `threads` threads (a divisor of kPartThreads; the parts of
+// the near-field sums are those of kPartThreads threads whatever it is, so the
+// result does not depend on it).  part: kPartThreads doubles of shared memory
+// when threads = kPartThreads.
+template <int THREADS>
+__device__ __forceinline__ void scatter_row(const ProbF32& p, int lo_leaf, int gl, int r, int ld,
+                                            const BatchParts& bp, const float* ynear, const float* yfar, double* part) {
+  const int leaf = gl - lo_leaf;
+  const int c = p.L - 1 + leaf;
+  const int cnt = p.count[c];
+  const int np = kPartThreads / ld;
+  const int tid = static_cast<int>(threadIdx.x);
+  const int64_t at = static_cast<int64_t>(r) * ld, step = static_cast<int64_t>(p.rc) * ld;
+  int c0 = 0, c1 = 0, k0 = 0, nlo = 0;
+  if (p.pf) {
+    c0 = bp.chunk_ptr[gl] - p.chunk0;
+    c1 = bp.chunk_ptr[gl + 1] - p.chunk0;
+    k0 = bp.lorow[gl];
+    nlo = bp.lorow[gl + 1] - k0;
+  }
+  auto near = [&](int q, int i) {
+    return near_part<float>(p.pf, c0, c1, p.pt, bp.lo_slot + k0, nlo, p.e_base, at + i, step, q, np);
+  };
+  auto put = [&](int i, double v) {
+    const int64_t t = (static_cast<int64_t>(gl) * kRC + r) * ld + i;
+    if (!p.pf) v = static_cast<double>(ynear[t]);
+    if (p.jmin <= p.J) v += static_cast<double>(yfar[t]);
+    p.y[static_cast<int64_t>(r) * p.ldy + p.perm[p.begin[c] + i]] = v;
+  };
+  if constexpr (THREADS == kPartThreads) {
+    const int q = tid / ld, i = tid - q * ld;
+    double v = 0.0;
+    if (p.pf && q < np && i < cnt) v = near(q, i);
+    part[tid] = v;
+    __syncthreads();
+    if (tid < cnt) {
+      for (int u = 1; u < np; ++u) v += part[u * ld + tid];
+      put(tid, v);
+    }
+  } else {
+    for (int i = tid; i < cnt; i += THREADS) {
+      double v = 0.0;
+      if (p.pf) {
+        v = near(0, i);
+        for (int u = 1; u < np; ++u) v += near(u, i);
+      }
+      put(i, v);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kPartThreads)
+k_scatter_batched(const ProbF32* probs, const int* leaf_off, int P, int Rmax, int ld, BatchParts bp, const float* ynear,
+                  const float* yfar) {
+  __shared__ double part[kPartThreads];
+  const int gl = static_cast<int>(blockIdx.x) / Rmax, r = static_cast<int>(blockIdx.x) % Rmax;
+  const int pi = problem_of(leaf_off, P, gl);
+  const ProbF32& p = probs[pi];
+  if (r >= p.R) return;
+  scatter_row<kPartThreads>(p, leaf_off[pi], gl, r, ld, bp, ynear, yfar, part);
+}
+
+// A batch without such sums, or with leaves too wide for kPartThreads: one
+// thread per element (t < Ltot * 16 * ld).
+__global__ void k_scatter_rows(const ProbF32* probs, const int* leaf_off, int P, int Ltot, int ld, const float* ynear,
+                               const float* yfar) {
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t >= static_cast<int64_t>(Ltot) * kRC * ld) return;
   const int i = static_cast<int>(t % ld);
   const int64_t lr = t / ld;
   const int r = static_cast<int>(lr % kRC);
@@ -319,13 +435,6 @@ __device__ __forceinline__ void scatter_elem(const ProbF32* probs, const int* le
   double v = static_cast<double>(ynear[t]);
   if (p.jmin <= p.J) v += static_cast<double>(yfar[t]);
   p.y[static_cast<int64_t>(r) * p.ldy + p.perm[p.begin[c] + i]] = v;
-}
-
-__global__ void k_scatter_batched(const ProbF32* probs, const int* leaf_off, int P, int Ltot, int ld,
-                                  const float* ynear, const float* yfar) {
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= static_cast<int64_t>(Ltot) * kRC * ld) return;
-  scatter_elem(probs, leaf_off, P, ld, ynear, yfar, t);
 }
 
 // ---------------------------------------------------------------------------
@@ -373,6 +482,13 @@ __device__ __forceinline__ bool persist_sum_item(const PersistSeg* segs, int nse
     ++s;
   }
   const PersistSeg& sg = segs[s];
+  if (sg.by_pair) {   // the whole CTA is the group
+    float* rsm = reinterpret_cast<float*>(sm);
+    if (sg.rc <= 1) rot::rot_chunk<D, 1, KER>(sg.r, idx, rsm);
+    else if (sg.rc <= 4) rot::rot_chunk<D, 4, KER>(sg.r, idx, rsm);
+    else rot::rot_chunk<D, 8, KER>(sg.r, idx, rsm);
+    return true;
+  }
   const int g = sg.a.first + idx;
   switch (sg.rc) {
     case 1: return sk::sum_block<D, 1, KER>(sg.a, g, G, sm, full, tiles);
@@ -497,7 +613,7 @@ __device__ __forceinline__ void persist_interleave(const PersistSeg* segs, int n
   for (int s = 0; s < nseg; ++s) {
     const PersistSeg& sg = segs[s];
     const int ld = sg.a.ld;
-    const int64_t n = static_cast<int64_t>(sg.count) * ld * sg.rc;
+    const int64_t n = static_cast<int64_t>(sg.groups) * ld * sg.rc;
     const float* src = sg.ilv_src + static_cast<int64_t>(sg.a.first) * kRC * ld;
     float* dst = const_cast<float*>(sg.a.q) + static_cast<int64_t>(sg.a.first) * sg.rc * ld;
     for (int64_t t = t0; t < n; t += stride) sk::interleave_elem(src, ld, sg.rc, dst, t);
@@ -554,27 +670,34 @@ __global__ void __launch_bounds__(kPersistThreads, 3) k_batch_persistent(const _
                                           pa.near_group_bytes, psm, sh, nullptr) < 0)
     return;
   if (!persist_barrier<D, KER>(pa, ph++, false, near_left, psm, sh)) return;
-  if (pa.io)
-    for (int64_t t = t0; t < nel; t += stride)
-      scatter_elem(pa.probs, pa.leaf_off, pa.P, pa.ld, pa.ynear, pa.yfar, t);
+  if (!pa.io) return;
+  for (int gl = static_cast<int>(blockIdx.x); gl < pa.Ltot; gl += static_cast<int>(gridDim.x)) {
+    const int pi = problem_of(pa.leaf_off, pa.P, gl);
+    const ProbF32& p = pa.probs[pi];
+    for (int r = 0; r < p.R; ++r)
+      scatter_row<kPersistThreads>(p, pa.leaf_off[pi], gl, r, pa.ld, pa.parts, pa.ynear, pa.yfar, nullptr);
+  }
 }
 
-// x (caller order, column-major) -> xb[leaf][r][m_pad] for r in [r0, r0+Rc).
+// x (caller order, column-major) -> xb[leaf][r][m_pad] for the columns
+// [r0, r0 + Rc), rows up to `rows` (the rest of them zero); xq, if given: the
+// same values interleaved, [leaf][m_pad][rows].
 template <typename T>
-__global__ void k_gather(const double* x, int64_t ldx, int r0, int Rc, const int32_t* perm,
-                         const int32_t* begin, const int32_t* count, int L, int m_pad, T* xb,
+__global__ void k_gather(const double* x, int64_t ldx, int r0, int Rc, int rows, const int32_t* perm,
+                         const int32_t* begin, const int32_t* count, int L, int m_pad, T* xb, T* xq,
                          unsigned long long* colmax) {
   const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t total = static_cast<int64_t>(L) * kRC * m_pad;
+  const int64_t total = static_cast<int64_t>(L) * rows * m_pad;
   if (t >= total) return;
   const int i = static_cast<int>(t % m_pad);
   const int64_t lr = t / m_pad;
-  const int r = static_cast<int>(lr % kRC);
-  const int leaf = static_cast<int>(lr / kRC);
+  const int r = static_cast<int>(lr % rows);
+  const int leaf = static_cast<int>(lr / rows);
   const int c = L - 1 + leaf;
   T v = T(0);
   if (r < Rc && i < count[c]) v = static_cast<T>(x[static_cast<int64_t>(r0 + r) * ldx + perm[begin[c] + i]]);
-  xb[t] = v;
+  xb[(static_cast<int64_t>(leaf) * kRC + r) * m_pad + i] = v;
+  if (xq) xq[(static_cast<int64_t>(leaf) * m_pad + i) * rows + r] = v;
   if (colmax && r < Rc) {
     // largest magnitude of each column; lanes of a warp may lie in two rows
     const unsigned act = __activemask();
@@ -587,38 +710,40 @@ __global__ void k_gather(const double* x, int64_t ldx, int r0, int Rc, const int
   }
 }
 
-// Scatter of the symmetric fixed-point near field: y = the row's chunk sums,
-// then the transposed sums of its lower entries, each in list order, plus the
-// far field.
-__global__ void k_scatter_parts(double* y, int64_t ldy, int r0, int Rc, const int32_t* perm, const int32_t* begin,
-                                const int32_t* count, int L, int m_pad, const int32_t* chunk_ptr, const int32_t* lorow,
-                                const int32_t* lo_slot, const double* pf, const double* pt, const double* yfar,
-                                int has_far, int* flags, unsigned long long* colmax) {
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t < 2) flags[t] = 0;   // every sum that reads them is done
-  if (t < kRC) colmax[t] = 0;
-  if (t >= static_cast<int64_t>(L) * Rc * m_pad) return;
-  const int i = static_cast<int>(t % m_pad);
-  const int64_t lr = t / m_pad;
-  const int r = static_cast<int>(lr % Rc);
-  const int leaf = static_cast<int>(lr / Rc);
-  const int c = L - 1 + leaf;
-  if (i >= count[c]) return;
-  const int64_t at = static_cast<int64_t>(r) * m_pad + i, step = static_cast<int64_t>(Rc) * m_pad;
-  double v = 0.0;
-  for (int e = chunk_ptr[leaf]; e < chunk_ptr[leaf + 1]; ++e) v += pf[e * step + at];
-  const int ke = lorow[leaf + 1];
-  int k = lorow[leaf];
-  for (; k + 8 <= ke; k += 8) {   // independent loads, sums in list order
-    double w[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) w[u] = pt[lo_slot[k + u] * step + at];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) v += w[u];
+// Scatter of the symmetric near fields: y = the row's chunk sums and the
+// transposed sums of its lower entries, plus the far field.  One CTA per leaf
+// and right-hand side; its threads' groups of m_pad take parts of both lists
+// (added in order), so that a short tree still has enough loads in flight: the
+// reads are rows of m_pad values all over the entries.  d = 8, N = 100003, 4
+// right-hand sides: 220 us with one thread per value and float64 additions.
+template <typename T>
+__global__ void __launch_bounds__(kPartThreads)
+k_scatter_parts(double* y, int64_t ldy, int r0, int Rc, const int32_t* perm, const int32_t* begin,
+                const int32_t* count, int L, int m_pad, const int32_t* chunk_ptr, const int32_t* lorow,
+                const int32_t* lo_slot, const T* pf, const T* pt, const T* yfar, int has_far, int* flags,
+                unsigned long long* colmax) {
+  __shared__ double part[kPartThreads];
+  const int tid = static_cast<int>(threadIdx.x);
+  if (blockIdx.x == 0) {   // every sum that reads them is done
+    if (flags && tid < 2) flags[tid] = 0;
+    if (colmax && tid < kRC) colmax[tid] = 0;
   }
-  for (; k < ke; ++k) v += pt[lo_slot[k] * step + at];
-  if (has_far) v += yfar[(static_cast<int64_t>(leaf) * kRC + r) * m_pad + i];
-  y[static_cast<int64_t>(r0 + r) * ldy + perm[begin[c] + i]] = v;
+  const int leaf = static_cast<int>(blockIdx.x) / Rc, r = static_cast<int>(blockIdx.x) % Rc;
+  const int c = L - 1 + leaf;
+  const int cnt = count[c];
+  const int np = kPartThreads / m_pad;
+  const int p = tid / m_pad, i = tid - p * m_pad;
+  const int k0 = lorow[leaf];
+  double v = 0.0;
+  if (p < np && i < cnt)
+    v = near_part<T>(pf, chunk_ptr[leaf], chunk_ptr[leaf + 1], pt, lo_slot + k0, lorow[leaf + 1] - k0, 0,
+                     static_cast<int64_t>(r) * m_pad + i, static_cast<int64_t>(Rc) * m_pad, p, np);
+  part[tid] = v;
+  __syncthreads();
+  if (tid >= cnt) return;
+  for (int u = 1; u < np; ++u) v += part[u * m_pad + tid];
+  if (has_far) v += static_cast<double>(yfar[(static_cast<int64_t>(leaf) * kRC + r) * m_pad + tid]);
+  y[static_cast<int64_t>(r0 + r) * ldy + perm[begin[c] + tid]] = v;
 }
 
 template <typename T>
@@ -629,16 +754,17 @@ __global__ void k_scatter(double* y, int64_t ldy, int r0, int Rc, const int32_t*
   const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (flags && t < 2) flags[t] = 0;   // every sum that reads them is done
   if (colmax && t < kRC) colmax[t] = 0;
-  const int64_t total = static_cast<int64_t>(L) * kRC * m_pad;
+  const int64_t total = static_cast<int64_t>(L) * Rc * m_pad;
   if (t >= total) return;
   const int i = static_cast<int>(t % m_pad);
   const int64_t lr = t / m_pad;
-  const int r = static_cast<int>(lr % kRC);
-  const int leaf = static_cast<int>(lr / kRC);
+  const int r = static_cast<int>(lr % Rc);
+  const int leaf = static_cast<int>(lr / Rc);
   const int c = L - 1 + leaf;
-  if (r >= Rc || i >= count[c]) return;
-  double v = static_cast<double>(ynear[t]);
-  if (has_far) v += static_cast<double>(yfar[t]);
+  if (i >= count[c]) return;
+  const int64_t o = (static_cast<int64_t>(leaf) * kRC + r) * m_pad + i;
+  double v = static_cast<double>(ynear[o]);
+  if (has_far) v += static_cast<double>(yfar[o]);
   y[static_cast<int64_t>(r0 + r) * ldy + perm[begin[c] + i]] = v;
 }
 
@@ -726,34 +852,37 @@ size_t farfield_smem_need(const Plan& P, bool fp64) {
   return std::max(a, b);
 }
 
-void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64, bool colmax) {
-  const int64_t total = static_cast<int64_t>(P.L) * kRC * P.m_pad;
+void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64, bool colmax, float* xq) {
+  const int rows = fp64 ? Rc : sum_padded_rc(Rc);
+  const int64_t total = static_cast<int64_t>(P.L) * rows * P.m_pad;
   if (fp64)
-    k_gather<double><<<ceil_div(total, 256), 256, 0, P.stream>>>(x, ldx, r0, Rc, P.d_perm.p, P.d_begin.p,
-                                                                 P.d_count.p, P.L, P.m_pad, P.xb64.p,
+    k_gather<double><<<ceil_div(total, 256), 256, 0, P.stream>>>(x, ldx, r0, Rc, rows, P.d_perm.p, P.d_begin.p,
+                                                                 P.d_count.p, P.L, P.m_pad, P.xb64.p, nullptr,
                                                                  colmax ? P.fx_colmax.p : nullptr);
   else
-    k_gather<float><<<ceil_div(total, 256), 256, 0, P.stream>>>(x, ldx, r0, Rc, P.d_perm.p, P.d_begin.p,
-                                                                P.d_count.p, P.L, P.m_pad, P.xb32.p, nullptr);
+    k_gather<float><<<ceil_div(total, 256), 256, 0, P.stream>>>(x, ldx, r0, Rc, rows, P.d_perm.p, P.d_begin.p,
+                                                                P.d_count.p, P.L, P.m_pad, P.xb32.p, xq, nullptr);
   DW_CUDA(cudaGetLastError());
 }
 
 void launch_scatter(Plan& P, double* y, int64_t ldy, int r0, int Rc, bool fp64) {
-  const int64_t total = static_cast<int64_t>(P.L) * kRC * P.m_pad;
+  const int64_t total = static_cast<int64_t>(P.L) * Rc * P.m_pad;
   const int has_far = P.jmin <= P.J;
-  if (fp64 && P.fx_parts)
-    k_scatter_parts<<<ceil_div(static_cast<int64_t>(P.L) * Rc * P.m_pad, 256), 256, 0, P.stream>>>(
-        y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad, P.fx_chunk_ptr.p, P.sym_lorow.p,
+  const int grid = ceil_div(total, 256);
+  if (P.near_parts == 1)
+    k_scatter_parts<double><<<P.L * Rc, kPartThreads, 0, P.stream>>>(
+        y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad, P.fx_rows.ptr.p, P.sym_lorow.p,
         P.sym_loslot.p, P.sym_pf.p, P.sym_pt.p, P.yfar64.p, has_far, P.fx_flag.p, P.fx_colmax.p);
+  else if (P.near_parts == 2)
+    k_scatter_parts<float><<<P.L * Rc, kPartThreads, 0, P.stream>>>(
+        y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad, P.rot.ptr.p, P.sym_lorow.p,
+        P.sym_loslot.p, P.rot_pf.p, P.rot_pt.p, P.yfar32.p, has_far, nullptr, nullptr);
   else if (fp64)
-    k_scatter<double><<<ceil_div(total, 256), 256, 0, P.stream>>>(y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p,
-                                                                  P.d_count.p, P.L, P.m_pad, P.ynear64.p,
-                                                                  P.yfar64.p, has_far, P.fx_flag.p,
-                                                                  P.fx_colmax.p);
+    k_scatter<double><<<grid, 256, 0, P.stream>>>(y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad,
+                                                  P.ynear64.p, P.yfar64.p, has_far, P.fx_flag.p, P.fx_colmax.p);
   else
-    k_scatter<float><<<ceil_div(total, 256), 256, 0, P.stream>>>(y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p,
-                                                                 P.d_count.p, P.L, P.m_pad, P.ynear32.p,
-                                                                 P.yfar32.p, has_far, nullptr, nullptr);
+    k_scatter<float><<<grid, 256, 0, P.stream>>>(y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad,
+                                                 P.ynear32.p, P.yfar32.p, has_far, nullptr, nullptr);
   DW_CUDA(cudaGetLastError());
 }
 
@@ -783,10 +912,14 @@ void launch_gather_batched(const ProbF32* probs, const int* leaf_off, int P, int
   k_gather_batched<<<ceil_div(total, 256), 256, 0, s>>>(probs, leaf_off, P, Ltot, ld, xb);
 }
 
-void launch_scatter_batched(const ProbF32* probs, const int* leaf_off, int P, int Ltot, int ld, const float* ynear,
-                            const float* yfar, cudaStream_t s) {
+void launch_scatter_batched(const ProbF32* probs, const int* leaf_off, int P, int Ltot, int ld, int Rmax,
+                            const BatchParts& parts, const float* ynear, const float* yfar, cudaStream_t s) {
+  if (parts.chunk_ptr) {
+    k_scatter_batched<<<Ltot * Rmax, kPartThreads, 0, s>>>(probs, leaf_off, P, Rmax, ld, parts, ynear, yfar);
+    return;
+  }
   const int64_t total = static_cast<int64_t>(Ltot) * kRC * ld;
-  k_scatter_batched<<<ceil_div(total, 256), 256, 0, s>>>(probs, leaf_off, P, Ltot, ld, ynear, yfar);
+  k_scatter_rows<<<ceil_div(total, 256), 256, 0, s>>>(probs, leaf_off, P, Ltot, ld, ynear, yfar);
 }
 
 size_t persist_group_bytes(int D, int RC, int ld, int threads) { return sk::group_stage_bytes(D, RC, ld, threads); }

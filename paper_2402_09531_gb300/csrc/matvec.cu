@@ -58,6 +58,7 @@ void ensure_workspace(Plan& P, bool fp64) {
     P.mom32.alloc(nc);
     P.loc32.alloc(nc);
     P.lco32.alloc(nc);
+    P.xq32.alloc(nl);
   }
 }
 
@@ -70,19 +71,21 @@ void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy
   for (int r0 = 0; r0 < R; r0 += kRC) {
     const int Rc = std::min(kRC, R - r0);
     timer_begin(P, 0, s);
-    launch_gather(P, x, ldx, r0, Rc, fp64, fix);
+    P.near_parts = 0;
+    launch_gather(P, x, ldx, r0, Rc, fp64, fix, fp64 ? nullptr : P.xq32.p);
     timer_end(P, 0, s, 1);
+    const bool rot = !fp64 && rot_ready(P, Rc);
     if (!fp64) m2l_autotune(P, Rc);   // once per tree, before the near field starts
     if (P.tm.on && P.tm.serialize) {  // every phase alone on the caller's stream
       launch_farfield(P, Rc, fp64);
       timer_begin(P, 4, s);
-      launch_nearfield(P, Rc, fp64, s);
+      launch_nearfield(P, Rc, fp64, rot, s);
       timer_end(P, 4, s, 1);
     } else {
       DW_CUDA(cudaEventRecord(P.ev_fork, s));
       DW_CUDA(cudaStreamWaitEvent(P.side, P.ev_fork, 0));
       timer_begin(P, 4, P.side);
-      launch_nearfield(P, Rc, fp64, P.side);
+      launch_nearfield(P, Rc, fp64, rot, P.side);
       timer_end(P, 4, P.side, 1);
       DW_CUDA(cudaEventRecord(P.ev_join, P.side));
       launch_farfield(P, Rc, fp64);

@@ -520,7 +520,7 @@ void launch_m2l(Plan& P, int Rc, bool fp64) {
   DW_CUDA(cudaGetLastError());
 }
 
-void launch_nearfield(Plan& P, int Rc, bool fp64, cudaStream_t s) {
+void launch_nearfield(Plan& P, int Rc, bool fp64, bool rot, cudaStream_t s) {
   if (fp64) {
     if (near_fix(P, Rc, s)) return;
     P.near_engine = 1;
@@ -528,7 +528,7 @@ void launch_nearfield(Plan& P, int Rc, bool fp64, cudaStream_t s) {
       P.near_engine = 0;
       p2p_impl<double>(P, Rc, P.d_pts64.p, P.xb64.p, P.ynear64.p, s);
     }
-  } else if (!p2p_f32_tuned(P, Rc, s)) {
+  } else if (!p2p_f32_tuned(P, Rc, rot, s)) {
     P.near_engine = 2;
     p2p_impl<float>(P, Rc, P.d_pts32.p, P.xb32.p, P.ynear32.p, s);
   }

@@ -1,5 +1,6 @@
 // Tuned float32 kernel summation for sm_103a: the P2P near field and the M2L
-// couplings of the DW-FMM (Sec. 5.2), y_i = sum_j phi(|x_i - x_j| / sigma) q_j.
+// couplings of the DW-FMM (Sec. 5.2), y_i = sum_j phi(|x_i - x_j| / sigma) q_j,
+// where p2p_rot.cu and the tensor-core kernels do not apply, and direct sums.
 //
 // Design (one CTA per target group: a leaf, or a cluster's node set):
 //  - Source blocks (scaled coordinates plus a norm row, then R charge rows)
@@ -197,7 +198,8 @@ void launch_scaled_blocks(const double* src, int64_t groups, int d, int D, int l
     k_scaled_blocks<<<ceil_div(groups * ld, 256), 256, 0, s>>>(src, groups, d, D, ld, kernel, sigma, dst);
 }
 
-bool p2p_f32_tuned(Plan& P, int Rc, cudaStream_t s) {
+// rot: each unordered pair once (rot_ready).  The charges are in P.xq32.
+bool p2p_f32_tuned(Plan& P, int Rc, bool rot, cudaStream_t s) {
   const int D = padded_dim(P.d);
   if (D < 0) return false;
   const int RC = padded_rc(Rc);
@@ -210,9 +212,13 @@ bool p2p_f32_tuned(Plan& P, int Rc, cudaStream_t s) {
     DW_CUDA(cudaEventRecord(P.ev_scaled, P.stream));
     DW_CUDA(cudaStreamWaitEvent(s, P.ev_scaled, 0));
   }
-  P.xq32.alloc(static_cast<size_t>(P.L) * P.m_pad * kRC);
-  const int64_t nq = static_cast<int64_t>(P.L) * P.m_pad * RC;
-  k_interleave<<<ceil_div(nq, 256), 256, 0, s>>>(P.xb32.p, P.L, P.m_pad, RC, P.xq32.p);
+  if (rot) {
+    P.near_engine = 2;
+    near_rot(P, D, Rc, s);
+    P.near_parts = 2;
+    DW_CUDA(cudaGetLastError());
+    return true;
+  }
   // MIXED plans with 9..16 right-hand sides: contraction on the tensor cores,
   // each unordered near pair once where the symmetric kernel applies
   P.near_engine = 4;

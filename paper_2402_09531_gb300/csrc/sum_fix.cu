@@ -3,7 +3,6 @@
 // fix64.cuh).
 #include <algorithm>
 #include <cmath>
-#include <vector>
 
 #include "sum_fix.cuh"
 
@@ -137,32 +136,12 @@ void shape(FixArgs& a, int n) {
 bool sym_ready(Plan& P) {
   if (P.fx_sym >= 0) return P.fx_sym == 1;
   P.fx_sym = 0;
-  if (!P.sym_ok || P.m_pad > fx::kThreads || static_cast<int>(P.h_upcount.size()) != P.L) return false;
-  int cmin = 1 << 30, cmax = 0;
-  for (int l = 0; l < P.L; ++l) {
-    cmin = std::min(cmin, P.h_count[P.L - 1 + l]);
-    cmax = std::max(cmax, P.h_count[P.L - 1 + l]);
-  }
-  if (cmin < 32) return false;
+  if (P.m_pad > fx::kThreads || P.sym_nup <= 0) return false;
   // a warp takes 64 sources at a time; 8 such batches where that still leaves
   // every SM 32 warps, fewer on small trees
-  const int64_t batches = P.sym_nup * cmax / 64;
-  const int64_t per_sm = batches / (32 * sm_count());
+  const int64_t per_sm = P.sym_nup * P.m_pad / 64 / (32 * sm_count());
   P.fx_batches = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(8, per_sm)));
-  const int per = fx::kThreads / 32 * 64 * P.fx_batches;
-  std::vector<int32_t> ptr(P.L + 1, 0), ct;
-  for (int t = 0; t < P.L; ++t) {
-    const int n = ceil_div(static_cast<int64_t>(P.h_upcount[t]) * cmax, per);
-    ptr[t + 1] = ptr[t] + n;
-    ct.insert(ct.end(), n, t);
-  }
-  P.fx_chunks = ptr[P.L];
-  P.fx_cmax = cmax;
-  P.fx_chunk_t.alloc(ct.size());
-  P.fx_chunk_ptr.alloc(ptr.size());
-  DW_CUDA(cudaMemcpyAsync(P.fx_chunk_t.p, ct.data(), ct.size() * sizeof(int32_t), cudaMemcpyHostToDevice, P.stream));
-  DW_CUDA(cudaMemcpyAsync(P.fx_chunk_ptr.p, ptr.data(), ptr.size() * sizeof(int32_t), cudaMemcpyHostToDevice, P.stream));
-  DW_CUDA(cudaStreamSynchronize(P.stream));
+  if (!row_chunks(P, fx::kThreads / 32 * 64 * P.fx_batches, 32, P.fx_rows)) return false;
   P.fx_sym = 1;
   return true;
 }
@@ -222,13 +201,13 @@ bool fix_ready(Plan& P) {
 }
 
 bool near_fix(Plan& P, int Rc, cudaStream_t s) {
-  P.fx_parts = false;
+  P.near_parts = 0;
   if (P.fx_state != 1) return false;
   const int RC = padded_r(Rc);
   k_fix_charges<<<ceil_div(static_cast<int64_t>(P.L) * RC * 32, 128), 128, 0, s>>>(
       P.xb64.p, 0, P.L, P.m_pad, Rc, RC, P.fx_colmax.p, reinterpret_cast<int2*>(P.fx_q.p), P.fx_qs.p, P.fx_colscale.p,
       P.fx_flag.p);
-  const size_t npf = static_cast<size_t>(P.fx_chunks) * Rc * P.m_pad, npt = static_cast<size_t>(P.sym_nup) * Rc * P.m_pad;
+  const size_t npf = static_cast<size_t>(P.fx_rows.n) * Rc * P.m_pad, npt = static_cast<size_t>(P.sym_nup) * Rc * P.m_pad;
   if (P.fx_sym == 1 && RC <= 4 && (npf + npt) * sizeof(double) <= kSymMaxBytes) {
     P.sym_pf.alloc(npf);
     P.sym_pt.alloc(npt);
@@ -239,13 +218,13 @@ bool near_fix(Plan& P, int Rc, cudaStream_t s) {
     b.table = P.fx_table.p;
     b.c = P.fx_c;
     b.count = P.d_count.p + P.L - 1;
-    b.chunk_t = P.fx_chunk_t.p;
-    b.chunk_ptr = P.fx_chunk_ptr.p;
+    b.chunk_t = P.fx_rows.t.p;
+    b.chunk_ptr = P.fx_rows.ptr.p;
     b.uprow = P.sym_uprow.p;
     b.up_s = P.sym_s.p;
     b.ld = P.m_pad;
     b.Rc = Rc;
-    b.cmax = P.fx_cmax;
+    b.cmax = P.fx_rows.cmax;
     b.batches = P.fx_batches;
     b.pf = P.sym_pf.p;
     b.pt = P.sym_pt.p;
@@ -254,8 +233,8 @@ bool near_fix(Plan& P, int Rc, cudaStream_t s) {
     b.inv_sigma = 1.0 / P.sigma;
     b.coord = P.d_pts64.p;
     b.charge = P.xb64.p;
-    dispatch_sym(P.kernel, P.d, RC, b, P.fx_chunks, s);
-    P.fx_parts = true;
+    dispatch_sym(P.kernel, P.d, RC, b, P.fx_rows.n, s);
+    P.near_parts = 1;
     P.near_engine = 1;
     return true;
   }

@@ -434,8 +434,7 @@ dwfmm_status dwfmm_phase_times(dwfmm_plan plan, double* ms, int64_t* launches, i
  * host application whose framework owns the device memory pool (its caching
  * allocator has reserved nearly all of it) or a latency-critical loop that
  * cannot take the device synchronisation of cudaMalloc/cudaFree.  The paper
- * has no counterpart of this entry point; it reuses the library's float32
- * near-field kernel on blocks of 256 sites.
+ * has no counterpart of this entry point.
  *
  * pts, x, y: device pointers (float64) of the current device (or managed
  * memory); unlike dwfmm_matvec this entry point does not stage host
@@ -443,12 +442,12 @@ dwfmm_status dwfmm_phase_times(dwfmm_plan plan, double* ms, int64_t* launches, i
  * row-major (leading dimension ld_pts >= d); x and y are column-major
  * N x nrhs (leading dimensions ldx, ldy >= N).  Limits: N <= 8192,
  * 1 <= d <= 16, 1 <= nrhs <= 16; larger sizes return DWFMM_ERR_INVALID_ARG.
- * The result is float32-accurate (relative error ~1e-7); a bounded
- * shared-memory wait that gave up writes NaN into y.
+ * The result is float32-accurate (relative error ~1e-7).
  *
- * All intermediates live in one fixed device array of about 1.6 MB inside
- * the library, which every GPU that loads the library keeps until the
- * process exits.  The first call on each device sets kernel attributes and
+ * Up to 1536 sites, with y apart from the sites and charges, one kernel works
+ * on the caller's buffers alone.  Otherwise the intermediates live in one
+ * fixed device array of about 1.1 MB inside the library, which every GPU that
+ * loads the library keeps until the process exits.  The first call on each device sets kernel attributes and
  * looks up that array's device address (no allocation); make that first
  * call before any stream capture: a first call made while `stream` is
  * capturing returns DWFMM_ERR_STATE.  Later calls outside capture look the

@@ -64,11 +64,19 @@ void Plan::free_tree() {
   momq32.release();
   bq32.release();
   bqm32.release();
+  part_rows.release();
+  near_parts32.release();
   near_parts64.release();
   fx_state = -1;
   fx_sym = -1;
   fx_rows.t.release();
   fx_rows.ptr.release();
+  ev_blk.release();
+  ev_out64.release();
+  ev_blk32.release();
+  ev_out32.release();
+  ev_rows.release();
+  ev_col.release();
   rot_state = -1;
   rot.t.release();
   rot.ptr.release();

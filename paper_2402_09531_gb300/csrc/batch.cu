@@ -129,7 +129,7 @@ SumArgs p2p_args(Batch& B, int RC, int leaf_first) {
   a.count = B.counts.p;
   a.count_off = 0;
   a.count_const = 0;
-  a.first = leaf_first;
+  a.first = a.first_row = leaf_first;
   a.ld = B.ld;
   a.Rc = RC;
   a.err = B.err.p;
@@ -147,6 +147,7 @@ RotArgs rot_args(Batch& B, const Batch::Cls& c) {
   a.up_s = B.up_s.p;
   a.ld = B.ld;
   a.Rc = c.RC;
+  a.ldp = B.ld;
   a.cmax_of = B.cmax_of.p;
   a.e_base = c.e_base;
   a.chunk0 = c.chunk0;
@@ -176,7 +177,7 @@ SumArgs m2l_args(Batch& B, int RC, int clus_first) {
   a.count = nullptr;
   a.count_off = 0;
   a.count_const = B.n;
-  a.first = clus_first;
+  a.first = a.first_row = clus_first;
   a.ld = B.n_pad;
   a.Rc = RC;
   a.err = B.err.p;

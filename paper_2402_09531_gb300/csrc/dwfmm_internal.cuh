@@ -143,8 +143,12 @@ struct SumArgs {
   int64_t q_gstride;
   float* out;              // [g][16][ld]
   int64_t out_gstride;
-  const int32_t* rowptr;   // CSR over target groups (indexed by first + blockIdx.x)
+  const int32_t* rowptr;   // CSR
   const int32_t* col;      // source group ids
+  // list of part p of group first + b: row first_row + b * row_step + p, sums
+  // at out + p * split_stride
+  int first_row = 0, row_step = 1, parts = 1;
+  int64_t split_stride = 0;
   const int32_t* count;    // group sizes (count[count_off + g]); nullptr -> count_const
   int count_off;
   int count_const;
@@ -164,11 +168,12 @@ struct RotArgs {
   const int32_t* uprow;      // [leaf + 1]
   const int32_t* up_s;
   int ld, Rc;
+  int ldp;                   // row stride of the partial sums (>= every leaf's size)
   int cmax;                  // slots an entry takes in its row's stream: the largest leaf,
   const int32_t* cmax_of;    // or one value per leaf
   int e_base, chunk0;        // first entry of pt, first chunk of pf
-  float* pf;                 // [chunk - chunk0][Rc][ld]
-  float* pt;                 // [entry - e_base][Rc][ld]
+  float* pf;                 // [chunk - chunk0][Rc][ldp]
+  float* pt;                 // [entry - e_base][Rc][ldp]
 };
 
 // The persistent batch matvec (one cooperative launch, farfield.cu): the
@@ -422,6 +427,10 @@ struct Plan {
   DBuf<double> xb64, ynear64, yfar64, mom64, loc64, lco64;
   DBuf<float> xb32, ynear32, yfar32, mom32, loc32, lco32;
   DBuf<double> stage_in, stage_out;   // host-pointer staging
+  // evaluation at new points (kept between calls; released with the tree)
+  DBuf<double> ev_blk, ev_out64;
+  DBuf<float> ev_blk32, ev_out32;
+  DBuf<int32_t> ev_rows, ev_col;   // float64: CSR over target blocks; float32: one row of all leaves
   // solve workspace
   DBuf<double> cg_r, cg_p, cg_ap, cg_c, cg_f, cg_dot, cg_tmp;
 
@@ -460,6 +469,8 @@ struct Plan {
   DBuf<float> xq32, momq32;   // charges interleaved per source, [g][ld][RC]
   DBuf<float> bq32;           // TF32 hi/lo charge blocks for the tensor-core P2P
   DBuf<float> bqm32;          // the same for the tensor-core M2L (moments at the nodes)
+  DBuf<int32_t> part_rows;    // the near lists in parts
+  DBuf<float> near_parts32;   // partial near-field sums of small float32 problems
   DBuf<double> near_parts64;  // partial near-field sums of small float64 problems (split lists)
   // symmetric float64 near field: upper entries (T, S >= T) of the near list,
   // per-leaf rows of the upper and lower lists, slots of the lower entries,
@@ -597,10 +608,10 @@ bool sum_tc(int D, int kernel, const float* tgt, int64_t tgt_gstride, const floa
             int first, int ngroups, int ld, int Rc, bool gauss_factored, int* err, cudaStream_t s);
 void evaluate(Plan& P, const double* tgt, int64_t nt, int64_t ldt, const double* c, int64_t ldc, double* out,
               int64_t ldo, int R);
-void eval_f64(Plan& P, const double* tgt64, int G, const int32_t* rowptr, const int32_t* col, int Rc, double* out,
-              cudaStream_t s);
-void eval_f32(Plan& P, const double* tgt64, int G, const int32_t* rowptr, const int32_t* col, int Rc, float* out,
-              DBuf<float>& scratch, cudaStream_t s);
+void eval_f64(Plan& P, const double* tgt64, int G, const int32_t* rowptr, const int32_t* col, int splits,
+              int64_t split_stride, int Rc, double* out, cudaStream_t s);
+void eval_f32(Plan& P, const float* tgtk, int G, const int32_t* rowptr, const int32_t* col,
+              int parts, int64_t split_stride, int Rc, float* out, cudaStream_t s);
 struct Batch;
 Batch* batch_new();
 void batch_delete(Batch* b);

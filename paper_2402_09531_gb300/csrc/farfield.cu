@@ -490,11 +490,13 @@ __device__ __forceinline__ bool persist_sum_item(const PersistSeg* segs, int nse
     return true;
   }
   const int g = sg.a.first + idx;
+  const int rb = sg.a.rowptr[g], re = sg.a.rowptr[g + 1];
+  float* out = sg.a.out + g * sg.a.out_gstride;
   switch (sg.rc) {
-    case 1: return sk::sum_block<D, 1, KER>(sg.a, g, G, sm, full, tiles);
-    case 4: return sk::sum_block<D, 4, KER>(sg.a, g, G, sm, full, tiles);
-    case 8: return sk::sum_block<D, 8, KER>(sg.a, g, G, sm, full, tiles);
-    default: return sk::sum_block<D, 16, KER>(sg.a, g, G, sm, full, tiles);
+    case 1: return sk::sum_block<D, 1, KER>(sg.a, g, rb, re, out, G, sm, full, tiles);
+    case 4: return sk::sum_block<D, 4, KER>(sg.a, g, rb, re, out, G, sm, full, tiles);
+    case 8: return sk::sum_block<D, 8, KER>(sg.a, g, rb, re, out, G, sm, full, tiles);
+    default: return sk::sum_block<D, 16, KER>(sg.a, g, rb, re, out, G, sm, full, tiles);
   }
 }
 
@@ -719,7 +721,7 @@ __global__ void k_gather(const double* x, int64_t ldx, int r0, int Rc, int rows,
 template <typename T>
 __global__ void __launch_bounds__(kPartThreads)
 k_scatter_parts(double* y, int64_t ldy, int r0, int Rc, const int32_t* perm, const int32_t* begin,
-                const int32_t* count, int L, int m_pad, const int32_t* chunk_ptr, const int32_t* lorow,
+                const int32_t* count, int L, int m_pad, int ldp, const int32_t* chunk_ptr, const int32_t* lorow,
                 const int32_t* lo_slot, const T* pf, const T* pt, const T* yfar, int has_far, int* flags,
                 unsigned long long* colmax) {
   __shared__ double part[kPartThreads];
@@ -731,17 +733,17 @@ k_scatter_parts(double* y, int64_t ldy, int r0, int Rc, const int32_t* perm, con
   const int leaf = static_cast<int>(blockIdx.x) / Rc, r = static_cast<int>(blockIdx.x) % Rc;
   const int c = L - 1 + leaf;
   const int cnt = count[c];
-  const int np = kPartThreads / m_pad;
-  const int p = tid / m_pad, i = tid - p * m_pad;
+  const int np = kPartThreads / ldp;
+  const int p = tid / ldp, i = tid - p * ldp;
   const int k0 = lorow[leaf];
   double v = 0.0;
   if (p < np && i < cnt)
     v = near_part<T>(pf, chunk_ptr[leaf], chunk_ptr[leaf + 1], pt, lo_slot + k0, lorow[leaf + 1] - k0, 0,
-                     static_cast<int64_t>(r) * m_pad + i, static_cast<int64_t>(Rc) * m_pad, p, np);
+                     static_cast<int64_t>(r) * ldp + i, static_cast<int64_t>(Rc) * ldp, p, np);
   part[tid] = v;
   __syncthreads();
   if (tid >= cnt) return;
-  for (int u = 1; u < np; ++u) v += part[u * m_pad + tid];
+  for (int u = 1; u < np; ++u) v += part[u * ldp + tid];
   if (has_far) v += static_cast<double>(yfar[(static_cast<int64_t>(leaf) * kRC + r) * m_pad + tid]);
   y[static_cast<int64_t>(r0 + r) * ldy + perm[begin[c] + tid]] = v;
 }
@@ -871,11 +873,11 @@ void launch_scatter(Plan& P, double* y, int64_t ldy, int r0, int Rc, bool fp64) 
   const int grid = ceil_div(total, 256);
   if (P.near_parts == 1)
     k_scatter_parts<double><<<P.L * Rc, kPartThreads, 0, P.stream>>>(
-        y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad, P.fx_rows.ptr.p, P.sym_lorow.p,
+        y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad, P.m_pad, P.fx_rows.ptr.p, P.sym_lorow.p,
         P.sym_loslot.p, P.sym_pf.p, P.sym_pt.p, P.yfar64.p, has_far, P.fx_flag.p, P.fx_colmax.p);
   else if (P.near_parts == 2)
     k_scatter_parts<float><<<P.L * Rc, kPartThreads, 0, P.stream>>>(
-        y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad, P.rot.ptr.p, P.sym_lorow.p,
+        y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad, round_up(P.rot.cmax, 8), P.rot.ptr.p, P.sym_lorow.p,
         P.sym_loslot.p, P.rot_pf.p, P.rot_pt.p, P.yfar32.p, has_far, nullptr, nullptr);
   else if (fp64)
     k_scatter<double><<<grid, 256, 0, P.stream>>>(y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad,

@@ -497,15 +497,16 @@ void build_far_sym_lists(Plan& P) {
   P.fsym_ok = true;
 }
 
-// Every target block against every source leaf in float64 (exact evaluation).
-void eval_f64(Plan& P, const double* tgt64, int G, const int32_t* rowptr, const int32_t* col, int Rc, double* out,
-              cudaStream_t s) {
+// Every target block against every source leaf in float64 (exact evaluation),
+// the sources in `splits` parts; part p writes at out + p * split_stride.
+void eval_f64(Plan& P, const double* tgt64, int G, const int32_t* rowptr, const int32_t* col, int splits,
+              int64_t split_stride, int Rc, double* out, cudaStream_t s) {
   const int64_t gs = static_cast<int64_t>(P.d) * P.m_pad;
   Side ts{gs, P.m_pad, nullptr, 0, P.m_pad};
   Side ss{gs, P.m_pad, P.d_count.p, P.L - 1, 0};
   dispatch_ksum<double>(P.kernel, G, 0, rowptr, col, P.d, 1.0 / P.sigma, tgt64, ts, P.d_pts64.p, ss, P.xb64.p,
                         static_cast<int64_t>(kRC) * P.m_pad, P.m_pad, out, static_cast<int64_t>(kRC) * P.m_pad,
-                        P.m_pad, Rc, s);
+                        P.m_pad, Rc, s, splits, split_stride);
 }
 
 void launch_m2l(Plan& P, int Rc, bool fp64) {

@@ -23,7 +23,6 @@
 //    shared memory).
 #include <atomic>
 #include <cstdint>
-#include <string>
 
 #include "dwfmm_internal.cuh"
 #include "sum_f32.cuh"
@@ -34,7 +33,8 @@ namespace {
 
 using namespace sk;
 
-// One CTA per target group g = a.first + blockIdx.x (the whole CTA is the group).
+// One CTA per target group and part of its list (the whole CTA is the group):
+// part p writes at out + p * split_stride.
 template <int D, int RC, int KER>
 __global__ void __launch_bounds__(kThreadsMax, 3) k_sum_f32(SumArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -47,7 +47,38 @@ __global__ void __launch_bounds__(kThreadsMax, 3) k_sum_f32(SumArgs a) {
   __syncthreads();
   int tile_base = 0;
   const Grp G{static_cast<int>(threadIdx.x), static_cast<int>(blockDim.x), 0};
-  (void)sum_block<D, RC, KER>(a, a.first + static_cast<int>(blockIdx.x), G, smem, full, tile_base);
+  // the parts' boundaries are read, not computed: any arithmetic on them takes
+  // the list walk out of the uniform registers (31 more registers a thread)
+  const int part = static_cast<int>(blockIdx.y);
+  const int g = a.first + static_cast<int>(blockIdx.x);
+  const int row = a.first_row + static_cast<int>(blockIdx.x) * a.row_step + part;
+  const int rb = a.rowptr[row], re = a.rowptr[row + 1];
+  (void)sum_block<D, RC, KER>(a, g, rb, re, a.out + part * a.split_stride + g * a.out_gstride, G, smem, full,
+                              tile_base);
+}
+
+// Rows of `parts` equal pieces of every list (rows * parts + 1 boundaries).
+__global__ void k_part_rows(const int32_t* rowptr, int rows, int parts, int32_t* out) {
+  const int t = static_cast<int>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t > rows * parts) return;
+  const int g = t < rows * parts ? t / parts : rows - 1, p = t < rows * parts ? t % parts : parts;
+  const int64_t len = rowptr[g + 1] - rowptr[g];
+  out[t] = rowptr[g] + static_cast<int32_t>((len * p) / parts);
+}
+
+// out[g][r][i] = the parts' sums added in order, compensated (r < Rc).
+__global__ void k_add_parts(const float* part, int splits, int64_t stride, int groups, int ld, int Rc, float* out) {
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t >= static_cast<int64_t>(groups) * Rc * ld) return;
+  const int64_t gr = t / ld;
+  const int64_t at = ((gr / Rc) * kRC + gr % Rc) * ld + t % ld;
+  float s = part[at], c = 0.0f;
+  for (int p = 1; p < splits; ++p) {
+    const float y = part[p * stride + at] - c, z = s + y;
+    c = (z - s) - y;
+    s = z;
+  }
+  out[at] = s;
 }
 
 // Row layout [g][16][ld] -> interleaved [g][ld][RC] (first RC rows).
@@ -82,13 +113,13 @@ template <int D, int RC>
 void launch_kernel_type(int kernel, SumArgs a, int groups, int threads, size_t smem, cudaStream_t s) {
   switch (kernel) {
     case DWFMM_K_EXP:
-      k_sum_f32<D, RC, DWFMM_K_EXP><<<groups, threads, smem, s>>>(a);
+      k_sum_f32<D, RC, DWFMM_K_EXP><<<dim3(groups, a.parts), threads, smem, s>>>(a);
       break;
     case DWFMM_K_MATERN32:
-      k_sum_f32<D, RC, DWFMM_K_MATERN32><<<groups, threads, smem, s>>>(a);
+      k_sum_f32<D, RC, DWFMM_K_MATERN32><<<dim3(groups, a.parts), threads, smem, s>>>(a);
       break;
     default:
-      k_sum_f32<D, RC, DWFMM_K_GAUSS><<<groups, threads, smem, s>>>(a);
+      k_sum_f32<D, RC, DWFMM_K_GAUSS><<<dim3(groups, a.parts), threads, smem, s>>>(a);
   }
 }
 
@@ -250,28 +281,43 @@ bool p2p_f32_tuned(Plan& P, int Rc, bool rot, cudaStream_t s) {
   a.Rc = Rc;
   a.err = P.d_err.p;
   const int threads = std::min(kThreadsMax, round_up(ceil_div(P.m_pad, kTT), 32));
-  dispatch(D, P.kernel, RC, a, P.L, threads, smem, s);
+  // few leaves: their lists in up to 16 parts, until every SM has 4 CTAs
+  // (d = 10 Gaussian, N = 3362, 12 right-hand sides, 16 leaves: the product
+  // took 177 us in one part, 45 us in 16)
+  const int splits = std::max(1, std::min(16, 4 * sm_count() / P.L));
+  if (splits > 1) {
+    if (!P.part_rows.p) {   // once per tree
+      P.part_rows.alloc(static_cast<size_t>(P.L) * splits + 1);
+      k_part_rows<<<ceil_div(static_cast<int64_t>(P.L) * splits + 1, 256), 256, 0, s>>>(P.d_near_rowptr.p, P.L, splits,
+                                                                                       P.part_rows.p);
+    }
+    a.rowptr = P.part_rows.p;
+    a.row_step = a.parts = splits;
+    a.split_stride = static_cast<int64_t>(P.L) * a.out_gstride;
+    P.near_parts32.alloc(static_cast<size_t>(splits) * a.split_stride);
+    a.out = P.near_parts32.p;
+    dispatch(D, P.kernel, RC, a, P.L, threads, smem, s);
+    k_add_parts<<<ceil_div(static_cast<int64_t>(P.L) * Rc * P.m_pad, 256), 256, 0, s>>>(
+        P.near_parts32.p, splits, a.split_stride, P.L, P.m_pad, Rc, P.ynear32.p);
+  } else {
+    dispatch(D, P.kernel, RC, a, P.L, threads, smem, s);
+  }
   DW_CUDA(cudaGetLastError());
   return true;
 }
 
-// Every target block against every source leaf in float32 (exact evaluation);
-// falls back to the generic kernel when d > 20.
-void eval_f32(Plan& P, const double* tgt64, int G, const int32_t* rowptr, const int32_t* col, int Rc, float* out,
-              DBuf<float>& scratch, cudaStream_t s) {
+// Every target block against every source leaf in float32 (exact evaluation),
+// the sources in `parts` parts; part p writes at out + p * split_stride.
+// tgtk: scaled target blocks; rowptr, col: one row of all leaves, cut into the
+// parts.
+void eval_f32(Plan& P, const float* tgtk, int G, const int32_t* rowptr, const int32_t* col,
+              int parts, int64_t split_stride, int Rc, float* out, cudaStream_t s) {
   const int D = padded_dim(P.d);
-  if (D < 0) fail(DWFMM_ERR_INVALID_ARG, "evaluation in float32 needs d <= 20");
   const int RC = padded_rc(Rc);
   ensure_attrs();
   ensure_scaled(P, D);
-  scratch.alloc(static_cast<size_t>(G) * (D + 1) * P.m_pad);
-  k_scaled_blocks<<<ceil_div(static_cast<int64_t>(G) * P.m_pad, 256), 256, 0, s>>>(tgt64, G, P.d, D, P.m_pad, P.kernel,
-                                                                                  P.sigma, scratch.p);
-  P.xq32.alloc(static_cast<size_t>(P.L) * P.m_pad * kRC);
-  const int64_t nq = static_cast<int64_t>(P.L) * P.m_pad * RC;
-  k_interleave<<<ceil_div(nq, 256), 256, 0, s>>>(P.xb32.p, P.L, P.m_pad, RC, P.xq32.p);
   SumArgs a{};
-  a.tgt = scratch.p;
+  a.tgt = tgtk;
   a.tgt_gstride = static_cast<int64_t>(D + 1) * P.m_pad;
   a.src = P.d_ptsk.p;
   a.src_gstride = a.tgt_gstride;
@@ -281,10 +327,11 @@ void eval_f32(Plan& P, const double* tgt64, int G, const int32_t* rowptr, const 
   a.out_gstride = static_cast<int64_t>(kRC) * P.m_pad;
   a.rowptr = rowptr;
   a.col = col;
+  a.row_step = 0;
+  a.parts = parts;
+  a.split_stride = split_stride;
   a.count = P.d_count.p;
   a.count_off = P.L - 1;
-  a.count_const = 0;
-  a.first = 0;
   a.ld = P.m_pad;
   a.Rc = Rc;
   a.err = P.d_err.p;
@@ -388,7 +435,7 @@ bool m2l_f32_tuned(Plan& P, int Rc) {
   a.count = nullptr;
   a.count_off = 0;
   a.count_const = P.n;
-  a.first = first;
+  a.first = a.first_row = first;
   a.ld = P.n_pad;
   a.Rc = Rc;
   a.err = P.d_err.p;
@@ -396,192 +443,6 @@ bool m2l_f32_tuned(Plan& P, int Rc) {
   dispatch(D, P.kernel, RC, a, P.C - first, threads, smem, P.stream);
   DW_CUDA(cudaGetLastError());
   return true;
-}
-
-
-// ---------------------------------------------------------------------------
-// Allocation-free direct sum (dwfmm_direct_sum_noalloc).
-//
-// Some callers cannot call cudaMalloc: host applications whose framework
-// owns the device memory pool (a caching allocator that has reserved nearly
-// all of it, so a fresh cudaMalloc fails or fragments the pool), and
-// latency-sensitive loops that cannot afford the device synchronisation
-// that cudaMalloc/cudaFree imply.  For them this entry point computes the
-// exact y = K x over all N sites (no tree) with the same tuned kernel as the
-// near field, and keeps every intermediate in one file-scope device array.
-//
-// The array is shared by every call on a device and holds the last call's
-// data; each call rewrites all of it that it reads.  Calls whose work
-// overlaps on the GPU (different streams, no ordering) race on it.
-// ---------------------------------------------------------------------------
-
-namespace {
-
-constexpr int kNaBlock = 256;                       // sites per block
-constexpr int kNaMaxN = 8192;                       // largest N
-constexpr int kNaMaxD = 16;                         // largest d (padded dimension <= 16)
-constexpr int kNaGroups = kNaMaxN / kNaBlock;       // 32
-constexpr size_t kNaCoord = static_cast<size_t>(kNaGroups) * (kNaMaxD + 1) * kNaBlock;
-constexpr size_t kNaCharge = static_cast<size_t>(kNaGroups) * kRC * kNaBlock;
-constexpr size_t kNaInts = 1 + kNaGroups + 1 + kNaGroups + static_cast<size_t>(kNaGroups) * kNaGroups;
-constexpr size_t kNaFloats = kNaCoord + 2 * kNaCharge + kNaInts;
-
-static __device__ __align__(256) float g_noalloc_scratch[kNaFloats];
-
-// Scratch layout (floats): coords [G][D+1][256] | charges [G][16][256] |
-// out [G][16][256] | ints: err, counts[G], rowptr[G+1], col[G*G].
-struct NaLayout {
-  float* coord;
-  float* charge;
-  float* out;
-  int* err;
-  int* count;
-  int* rowptr;
-  int* col;
-};
-
-NaLayout na_layout(float* base) {
-  NaLayout l;
-  l.coord = base;
-  l.charge = base + kNaCoord;
-  l.out = l.charge + kNaCharge;
-  int* ints = reinterpret_cast<int*>(l.out + kNaCharge);
-  l.err = ints;
-  l.count = ints + 1;
-  l.rowptr = l.count + kNaGroups;
-  l.col = l.rowptr + kNaGroups + 1;
-  return l;
-}
-
-// Fills every scratch entry the sum reads: scaled coordinates and norm row,
-// charges (zero past N and past nrhs), counts, a complete block list, and
-// clears the error flag.
-__global__ void k_na_prepare(const double* pts, int64_t n, int d, int64_t ldp, int D, int kernel,
-                             double sigma, const double* x, int R, int RC, int64_t ldx, NaLayout l, int G) {
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t == 0) *l.err = 0;
-  if (t < G) {
-    const int64_t rem = n - t * kNaBlock;
-    l.count[t] = static_cast<int>(rem < kNaBlock ? rem : kNaBlock);
-    l.rowptr[t] = static_cast<int>(t) * G;
-    if (t == G - 1) l.rowptr[G] = G * G;
-  }
-  if (t < static_cast<int64_t>(G) * G) l.col[t] = static_cast<int>(t % G);
-  if (t >= static_cast<int64_t>(G) * kNaBlock) return;
-  const int g = static_cast<int>(t / kNaBlock), i = static_cast<int>(t % kNaBlock);
-  const int64_t src = t < n ? t : static_cast<int64_t>(g) * kNaBlock;   // padding repeats the block's first site
-  double scale;
-  if (kernel == DWFMM_K_GAUSS) scale = sqrt(1.4426950408889634 / (2.0 * sigma * sigma));
-  else if (kernel == DWFMM_K_EXP) scale = 1.4426950408889634 / sigma;
-  else scale = 1.7320508075688772 / sigma;
-  double n2 = 0.0;
-  for (int k = 0; k < D; ++k) {
-    const float f = k < d ? static_cast<float>(pts[src * ldp + k] * scale) : 0.0f;
-    l.coord[(static_cast<int64_t>(g) * (D + 1) + k) * kNaBlock + i] = f;
-    n2 += static_cast<double>(f) * static_cast<double>(f);
-  }
-  l.coord[(static_cast<int64_t>(g) * (D + 1) + D) * kNaBlock + i] = static_cast<float>(n2);
-  for (int r = 0; r < RC; ++r)   // interleaved per site: [g][256][RC]
-    l.charge[(static_cast<int64_t>(g) * kNaBlock + i) * RC + r] =
-        (t < n && r < R) ? static_cast<float>(x[r * ldx + t]) : 0.0f;
-}
-
-// y[:, r] from the per-block sums; NaN if a bounded wait gave up.
-__global__ void k_na_finish(NaLayout l, int64_t n, int R, double* y, int64_t ldy) {
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= n * R) return;
-  const int r = static_cast<int>(t / n);
-  const int64_t i = t % n;
-  const int g = static_cast<int>(i / kNaBlock), j = static_cast<int>(i % kNaBlock);
-  const double v = static_cast<double>(l.out[(static_cast<int64_t>(g) * kRC + r) * kNaBlock + j]);
-  y[r * ldy + i] = (*l.err) ? __longlong_as_double(0x7ff8000000000000ll) : v;
-}
-
-// Device address of the scratch array.  Outside stream capture it is looked
-// up on every call (cudaGetSymbolAddress allocates nothing), so a context
-// that was reset still gets the right address; the last address seen per
-// device serves calls made during capture, where the first call on a device
-// must not load the module or set kernel attributes.
-constexpr int kNaMaxDevices = 64;
-std::atomic<float*> g_na_ptr[kNaMaxDevices];
-
-float* na_scratch_for_current_device(cudaStream_t s) {
-  int dev = 0;
-  DW_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= kNaMaxDevices) fail(DWFMM_ERR_INVALID_ARG, "device index out of range");
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  DW_CUDA(cudaStreamIsCapturing(s, &cap));
-  if (cap != cudaStreamCaptureStatusNone) {
-    float* p = g_na_ptr[dev].load();
-    if (!p)
-      fail(DWFMM_ERR_STATE,
-           "direct_sum_noalloc: the first call on a device sets it up and must come before any stream capture");
-    return p;
-  }
-  ensure_attrs();
-  void* p = nullptr;
-  DW_CUDA(cudaGetSymbolAddress(&p, g_noalloc_scratch));
-  g_na_ptr[dev].store(static_cast<float*>(p));
-  return static_cast<float*>(p);
-}
-
-// Buffers the kernels read or write directly: device (or managed) memory of
-// the current device.  A host pointer would fault on the GPU.
-void na_check_device_buffer(const void* p, int dev, const char* name) {
-  cudaPointerAttributes a;
-  const cudaError_t e = cudaPointerGetAttributes(&a, p);
-  if (e != cudaSuccess) (void)cudaGetLastError();
-  const bool ok = e == cudaSuccess &&
-                  ((a.type == cudaMemoryTypeDevice && a.device == dev) || a.type == cudaMemoryTypeManaged);
-  if (!ok)
-    fail(DWFMM_ERR_INVALID_ARG, std::string("direct_sum_noalloc: ") + name +
-                                    " must be device memory of the current device");
-}
-
-}  // namespace
-
-dwfmm_status direct_sum_noalloc(int kernel, double sigma, const double* pts, int64_t n, int d, int64_t ldp,
-                                const double* x, double* y, int R, int64_t ldx, int64_t ldy,
-                                cudaStream_t s) {
-  if (kernel < 0 || kernel > 2 || !(sigma > 0.0) || n < 0 || n > kNaMaxN || d < 1 || d > kNaMaxD ||
-      R < 1 || R > kRC)
-    fail(DWFMM_ERR_INVALID_ARG, "direct_sum_noalloc: needs N <= 8192, 1 <= d <= 16, 1 <= nrhs <= 16");
-  if (n == 0) return DWFMM_OK;
-  if (!pts || !x || !y || ldp < d || ldx < n || ldy < n)
-    fail(DWFMM_ERR_INVALID_ARG, "direct_sum_noalloc: NULL buffer or leading dimension too small");
-  int dev = 0;
-  DW_CUDA(cudaGetDevice(&dev));
-  na_check_device_buffer(pts, dev, "pts");
-  na_check_device_buffer(x, dev, "x");
-  na_check_device_buffer(y, dev, "y");
-  const int D = padded_dim(d);
-  const int RC = padded_rc(R);
-  const int G = static_cast<int>((n + kNaBlock - 1) / kNaBlock);
-  const NaLayout l = na_layout(na_scratch_for_current_device(s));
-  k_na_prepare<<<ceil_div(static_cast<int64_t>(G) * kNaBlock + G * G, 256), 256, 0, s>>>(
-      pts, n, d, ldp, D, kernel, sigma, x, R, RC, ldx, l, G);
-  SumArgs a{};
-  a.tgt = l.coord;
-  a.tgt_gstride = static_cast<int64_t>(D + 1) * kNaBlock;
-  a.src = l.coord;
-  a.src_gstride = a.tgt_gstride;
-  a.q = l.charge;
-  a.q_gstride = static_cast<int64_t>(RC) * kNaBlock;
-  a.out = l.out;
-  a.out_gstride = static_cast<int64_t>(kRC) * kNaBlock;
-  a.rowptr = l.rowptr;
-  a.col = l.col;
-  a.count = l.count;
-  a.count_off = 0;
-  a.count_const = 0;
-  a.first = 0;
-  a.ld = kNaBlock;
-  a.Rc = R;
-  a.err = l.err;
-  dispatch(D, kernel, RC, a, G, kThreadsMax, stage_bytes(D, RC, kNaBlock), s);
-  k_na_finish<<<ceil_div(n * R, 256), 256, 0, s>>>(l, n, R, y, ldy);
-  DW_CUDA(cudaGetLastError());
-  return DWFMM_OK;
 }
 
 }  // namespace dw

@@ -118,7 +118,8 @@ bool rot_ready(Plan& P, int Rc) {
   if (sum_padded_dim(P.d) < 0 || !rot_fits(P.m_pad, kRotMinLeaf, sum_padded_rc(Rc))) return false;
   if (P.rot_state < 0) P.rot_state = row_chunks(P, kRotPer, kRotMinLeaf, P.rot) ? 1 : 0;
   if (P.rot_state == 0) return false;
-  const size_t npf = static_cast<size_t>(P.rot.n) * Rc * P.m_pad, npt = static_cast<size_t>(P.sym_nup) * Rc * P.m_pad;
+  const size_t row = static_cast<size_t>(Rc) * round_up(P.rot.cmax, 8);
+  const size_t npf = P.rot.n * row, npt = P.sym_nup * row;
   if ((npf + npt) * sizeof(float) > kRotMaxBytes) return false;
   P.rot_pf.alloc(npf);
   P.rot_pt.alloc(npt);
@@ -137,6 +138,7 @@ void near_rot(Plan& P, int D, int Rc, cudaStream_t s) {
   a.up_s = P.sym_s.p;
   a.ld = P.m_pad;
   a.Rc = Rc;
+  a.ldp = round_up(P.rot.cmax, 8);
   a.cmax = P.rot.cmax;
   a.pf = P.rot_pf.p;
   a.pt = P.rot_pt.p;

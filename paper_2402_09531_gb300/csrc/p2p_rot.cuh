@@ -212,7 +212,7 @@ __device__ __forceinline__ void rot_chunk(const RotArgs& a, int chunk, float* rs
     up2(t2[1][r], v[2], v[3]);
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-      if (ent[u] >= 0) a.pt[(static_cast<int64_t>(ent[u]) * a.Rc + r) * ld + slot[u]] = v[u];
+      if (ent[u] >= 0) a.pt[(static_cast<int64_t>(ent[u]) * a.Rc + r) * a.ldp + slot[u]] = v[u];
   }
   __syncthreads();
   for (int i = threadIdx.x; i < a.Rc * c; i += kRotThreads) {
@@ -225,7 +225,7 @@ __device__ __forceinline__ void rot_chunk(const RotArgs& a, int chunk, float* rs
       lost += (v - (sum - back)) + (f - back);
       v = sum;
     }
-    a.pf[(static_cast<int64_t>(chunk) * a.Rc + r) * ld + t] = v + lost;
+    a.pf[(static_cast<int64_t>(chunk) * a.Rc + r) * a.ldp + t] = v + lost;
   }
 }
 

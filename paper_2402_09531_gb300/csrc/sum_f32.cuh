@@ -151,8 +151,8 @@ __host__ __device__ constexpr size_t group_stage_bytes(int D, int RC, int ld, in
          static_cast<size_t>(kTT) * (RC >= 2 ? RC / 2 : 1) * threads * sizeof(unsigned long long);
 }
 
-// Target group g (all of its targets, kTT * G.size per pass) against its
-// list a.rowptr[g] .. a.rowptr[g + 1].  `smem` holds the group's two stages
+// Target group g (all of its targets, kTT * G.size per pass) against the
+// entries rb .. re - 1 of the list a.col, into the group's rows at out.  `smem` holds the group's two stages
 // and its compensation array (group_stage_bytes), `full` its two stage
 // barriers, initialised with count 1; `tile_base` counts the stages the
 // barriers have completed so far and is advanced.  Returns false (after
@@ -162,15 +162,14 @@ __host__ __device__ constexpr size_t group_stage_bytes(int D, int RC, int ld, in
 // adjacent: (acc_r, acc_r+1) += (phi, phi) * (q_r, q_r+1) is one fma.f32x2.
 // Distances pair up consecutive sources: (e_j, e_j+1) += (2x_k, 2x_k) * (s_jk, s_j+1,k).
 template <int D, int RC, int KER>
-__device__ __forceinline__ bool sum_block(const SumArgs& a, int g, const Grp& G, unsigned char* smem, uint64_t* full,
-                                          int& tile_base) {
+__device__ __forceinline__ bool sum_block(const SumArgs& a, int g, int rb, int re, float* out, const Grp& G,
+                                          unsigned char* smem, uint64_t* full, int& tile_base) {
   constexpr int RP = RC >= 2 ? RC / 2 : 1;   // packed accumulators per target
   const int ld = a.ld;
   const int stage_floats = (D + 1) * ld + RC * ld;
   float* stage0 = reinterpret_cast<float*>(smem);
   // Kahan compensation, [kTT * RP][group size] packed pairs (or floats when RC == 1)
   u64* comp = reinterpret_cast<u64*>(stage0 + 2 * stage_floats);
-  const int rb = a.rowptr[g], re = a.rowptr[g + 1];
   const uint32_t coord_bytes = static_cast<uint32_t>((D + 1) * ld * sizeof(float));
   const uint32_t q_bytes = static_cast<uint32_t>(RC * ld * sizeof(float));
 
@@ -212,7 +211,9 @@ __device__ __forceinline__ bool sum_block(const SumArgs& a, int g, const Grp& G,
 #pragma unroll
       for (int p = 0; p < RP; ++p) {
         acc[t][p] = 0ull;
-        comp[(t * RP + p) * G.size + G.tid] = 0ull;
+        // each thread clears the slots it will use: no barrier follows before the first fold
+        if constexpr (RC == 1) reinterpret_cast<float*>(comp)[t * G.size + G.tid] = 0.0f;
+        else comp[(t * RP + p) * G.size + G.tid] = 0ull;
       }
     }
 
@@ -345,7 +346,7 @@ __device__ __forceinline__ bool sum_block(const SumArgs& a, int g, const Grp& G,
 #pragma unroll
     for (int t = 0; t < kTT; ++t) {
       if (ti[t] < ld) {
-        float* op = a.out + g * a.out_gstride + ti[t];
+        float* op = out + ti[t];
         if constexpr (RC == 1) {
           if (a.Rc > 0) op[0] = acc1[t];
         } else {

@@ -369,8 +369,9 @@ dwfmm_status dwfmm_near_engine(dwfmm_plan plan, int32_t* engine);
  * hi*hi + hi*lo + lo*hi accumulated in FP32 by tcgen05.mma, per-cluster
  * contractions in 64-wide chunks folded in FP32, the transforms one GEMM per
  * tree level with the constant V^{-1} tile.  MIXED plans take engine 2 when
- * |Lambda| <= 128, leaves hold 128 or 256 sites and a multi-index has at
- * most 20 nonzero entries; otherwise engine 1.  Errors: INVALID_ARG. */
+ * |Lambda| <= 128, leaves hold 128 or 256 sites, a multi-index has at most 20
+ * nonzero entries and more than 2 right-hand sides are passed (CG iterations:
+ * any number); otherwise engine 1.  Errors: INVALID_ARG. */
 dwfmm_status dwfmm_far_engine(dwfmm_plan plan, int32_t* engine);
 
 /* Which engine ran the couplings (M2L, Eq. (5.4): the far blocks S_{t,s}

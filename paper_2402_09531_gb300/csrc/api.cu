@@ -65,6 +65,7 @@ void Plan::free_tree() {
   bq32.release();
   bqm32.release();
   part_rows.release();
+  entry_parts32.release();
   near_parts32.release();
   near_parts64.release();
   fx_state = -1;
@@ -146,6 +147,10 @@ void Plan::free_all() {
   d_nodes.release();
   d_vinv.release();
   d_vinv32.release();
+  d_vinvt.release();
+  d_vinvt32.release();
+  d_act.release();
+  d_leg64.release();
   far_vt.release();
   far_vexp.release();
   far_vt_ok = false;
@@ -283,7 +288,6 @@ dwfmm_status dwfmm_plan_create(const dwfmm_config* cfg, void* stream, dwfmm_plan
     dw::setup_expansion(P);
     if (dw::farfield_smem_need(P, true) > 220 * 1024)
       fail(DWFMM_ERR_INVALID_ARG, "index set too large for the far-field kernels");
-    dw::farfield_set_smem_limits(P);
     return DWFMM_OK;
   });
   if (st != DWFMM_OK) {

@@ -187,10 +187,10 @@ SumArgs m2l_args(Batch& B, int RC, int clus_first) {
 int threads_for(int ld) { return std::min(128, round_up((ld + 1) / 2, 32)); }
 
 // The fused near-field work: interleave charges, P2P launch(es) with
-// `threads` per CTA.  Classes whose pairs are evaluated once have launches of
-// their own (one shape).
-void enqueue_near(Batch& B, bool split, int threads, cudaStream_t s) {
-  if (!split && !B.by_pair) {
+// `threads` per CTA.  With by_pair, classes whose pairs are evaluated once have
+// launches of their own (one shape).
+void enqueue_near(Batch& B, bool split, int threads, bool by_pair, cudaStream_t s) {
+  if (!split && !by_pair) {
     launch_interleave(B.xb.p, B.Ltot, B.ld, B.RCmax, B.xq.p, s);
     launch_sum_f32(B.D, B.kernel, B.RCmax, p2p_args(B, B.RCmax, 0), B.Ltot, threads,
                    sum_stage_bytes(B.D, B.RCmax, B.ld), s);
@@ -199,7 +199,7 @@ void enqueue_near(Batch& B, bool split, int threads, cudaStream_t s) {
   for (const auto& c : B.classes) {
     launch_interleave(B.xb.p + static_cast<int64_t>(c.leaf_first) * kRC * B.ld, c.leaf_count, B.ld, c.RC,
                       B.xq.p + static_cast<int64_t>(c.leaf_first) * B.ld * c.RC, s);
-    if (c.by_pair) {
+    if (by_pair && c.by_pair) {
       launch_rot(B.D, B.kernel, c.RC, rot_args(B, c), c.chunks, s);
       continue;
     }
@@ -234,8 +234,12 @@ cudaError_t enqueue_persistent(Batch& B, cudaStream_t s, bool io) {
   return launch_batch_persistent(B.D, B.kernel, a, B.pgrid, B.psmem, s);
 }
 
-void enqueue_matvec(Batch& B, bool io = true) {
-  if (B.persistent) {
+// steady: the float32 sums of single plans' CG iterations (one order, see
+// apply_op in solve.cu), so that a problem's iterates are the same alone and in
+// a batch.
+void enqueue_matvec(Batch& B, bool io = true, bool steady = false) {
+  const bool by_pair = B.by_pair && !steady;
+  if (B.persistent && (by_pair || !B.by_pair)) {
     DW_CUDA(enqueue_persistent(B, B.stream, io));
     return;
   }
@@ -243,7 +247,7 @@ void enqueue_matvec(Batch& B, bool io = true) {
   if (io) launch_gather_batched(B.probs.p, B.d_leaf_off.p, B.P, B.Ltot, B.ld, B.xb.p, s);
   DW_CUDA(cudaEventRecord(B.ev_fork, s));
   DW_CUDA(cudaStreamWaitEvent(B.side, B.ev_fork, 0));
-  enqueue_near(B, B.split, B.thr_near, B.side);
+  enqueue_near(B, B.split, B.thr_near, by_pair, B.side);
   DW_CUDA(cudaEventRecord(B.ev_join, B.side));
   for (size_t h = 0; h < B.up_off.size(); ++h)
     launch_moments_batched(B.probs.p, B.work.p + B.up_off[h], B.up_cnt[h], B.far_smem, s);
@@ -253,7 +257,7 @@ void enqueue_matvec(Batch& B, bool io = true) {
   DW_CUDA(cudaStreamWaitEvent(s, B.ev_join, 0));
   if (io)
     launch_scatter_batched(B.probs.p, B.d_leaf_off.p, B.P, B.Ltot, B.ld, *std::max_element(B.R.begin(), B.R.end()),
-                           batch_parts(B), B.ynear.p, B.yfar.p, s);
+                           by_pair ? batch_parts(B) : BatchParts{}, B.ynear.p, B.yfar.p, s);
   DW_CUDA(cudaGetLastError());
 }
 
@@ -266,7 +270,7 @@ double time_shape(Batch& B, int which, bool split, int threads) {
   float best = 1e30f;
   for (int rep = 0; rep < 2; ++rep) {
     DW_CUDA(cudaEventRecord(a, B.stream));
-    if (which == 0) enqueue_near(B, split, threads, B.stream);
+    if (which == 0) enqueue_near(B, split, threads, B.by_pair, B.stream);
     else enqueue_m2l(B, split, threads, B.stream);
     DW_CUDA(cudaEventRecord(b, B.stream));
     DW_CUDA(cudaEventSynchronize(b));
@@ -646,10 +650,11 @@ void batch_create(Batch& B, Plan* const* plans, const int32_t* nrhs, int count) 
   B.n_pad = P0.n_pad;
   B.ld = P0.m_pad;
   B.D = 0;
-  int lsum_max = 0, Rmax = 1;
+  int lsum_max = 0, nnz_max = 1, Rmax = 1;
   for (int i = 0; i < count; ++i) {
     B.D = std::max(B.D, sum_padded_dim(B.plans[i]->d));
     lsum_max = std::max(lsum_max, B.plans[i]->lsum);
+    nnz_max = std::max(nnz_max, B.plans[i]->nnz_max);
     Rmax = std::max(Rmax, B.R[i]);
   }
   B.RCmax = sum_padded_rc(Rmax);
@@ -739,6 +744,7 @@ void batch_create(Batch& B, Plan* const* plans, const int32_t* nrhs, int count) 
     q.lo = p.d_lo32.p;
     q.iext = p.d_iext32.p;
     q.vinv = p.d_vinv32.p;
+    q.vinvt = p.d_vinvt32.p;
     q.xb = B.xb.p + static_cast<size_t>(B.leaf_off[i]) * kRC * B.ld;
     q.yfar = B.yfar.p + static_cast<size_t>(B.leaf_off[i]) * kRC * B.ld;
     q.mom = B.mom.p + static_cast<size_t>(B.clus_off[i]) * kRC * B.n_pad;
@@ -782,8 +788,8 @@ void batch_create(Batch& B, Plan* const* plans, const int32_t* nrhs, int count) 
   }
   B.work.alloc(std::max<size_t>(w.size(), 1));
   if (!w.empty()) DW_CUDA(cudaMemcpy(B.work.p, w.data(), sizeof(int2) * w.size(), cudaMemcpyHostToDevice));
-  B.far_smem = batch_far_smem(lsum_max, B.n_pad);
-  if (B.far_smem > 200 * 1024) fail(DWFMM_ERR_INVALID_ARG, "index sets too large for a batch");
+  B.far_smem = batch_far_smem(lsum_max, B.n, B.n_pad, nnz_max, Rmax);
+  if (batch_far_need(lsum_max, B.n_pad) > 200 * 1024) fail(DWFMM_ERR_INVALID_ARG, "index sets too large for a batch");
   batch_far_attrs();
   ensure_sum_attrs();
   // right-hand-side classes (contiguous in the internal order)
@@ -1068,7 +1074,7 @@ void batch_cg_step(Batch& B, int iters, cudaStream_t s) {
     cudaStream_t bst = B.stream;
     DW_CUDA(cudaStreamBeginCapture(bst, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < iters; ++k) {
-      enqueue_matvec(B);
+      enqueue_matvec(B, true, true);
       k_bcg_partial<<<nblk, kBcgThreads, 0, bst>>>(d_items, d_segs, d_blk, 0, B.cg_part.p);
       k_bcg_scalar<<<ceil_div(nseg, 64), 64, 0, bst>>>(d_items, d_segs, nseg, 0, B.cg_part.p);
       k_bcg_partial<<<nblk, kBcgThreads, 0, bst>>>(d_items, d_segs, d_blk, 1, B.cg_part.p);

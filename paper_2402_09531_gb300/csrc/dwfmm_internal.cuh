@@ -97,6 +97,9 @@ struct ExpDev {
   const int16_t* fac;   // [n][nnz_max] offsets into a point's Legendre table, -1 = none
   const int32_t* qk;    // [d] max degree per dimension
   const int32_t* loff;  // [d] offset of dimension k in a point's Legendre table
+  const int32_t* act;   // [nact] dimensions with a degree above 0
+  int nact;
+  const double2* leg64; // coefficients (a_j, b_j) of the normalised Legendre recurrence
 };
 
 // One problem of a batch, float32 (device table entry).  Arrays marked
@@ -112,6 +115,7 @@ struct ProbF32 {
   const float* lo;        // [C][d]
   const float* iext;      // [C][d]
   const float* vinv;      // [n_pad][n_pad]
+  const float* vinvt;     // its transpose
   float* xb;              // slice [L][16][m_pad]
   float* mom;             // slice [C][16][n_pad]
   float* loc;             // slice
@@ -148,6 +152,9 @@ struct SumArgs {
   // list of part p of group first + b: row first_row + b * row_step + p, sums
   // at out + p * split_stride
   int first_row = 0, row_step = 1, parts = 1;
+  // one CTA per entry e of the list instead: target group entry_t[2 e] - entry_off
+  const int32_t* entry_t = nullptr;
+  int entry_off = 0;
   int64_t split_stride = 0;
   const int32_t* count;    // group sizes (count[count_off + g]); nullptr -> count_const
   int count_off;
@@ -330,12 +337,12 @@ struct Timers {
 struct CgGraphKey {
   int tree_gen = -1, R = 0, iters = 0;
   double lam = 0.0;
-  bool fp64 = false;
+  bool fp64 = false, steady = false;
   cudaStream_t stream = nullptr;
   const void* bufs[6] = {};
   bool operator==(const CgGraphKey& o) const {
     if (tree_gen != o.tree_gen || R != o.R || iters != o.iters || lam != o.lam || fp64 != o.fp64 ||
-        stream != o.stream)
+        steady != o.steady || stream != o.stream)
       return false;
     for (int i = 0; i < 6; ++i)
       if (bufs[i] != o.bufs[i]) return false;
@@ -347,6 +354,7 @@ struct CgState {
   int R = 0;
   double lam = 0.0, rtol = 1e-6;
   bool active = false, stepped = false;
+  bool steady = true;           // operator of the iterations (apply_op)
   DBuf<int> d_int;              // status[R], iters[R]
   int* h_snap = nullptr;        // pinned: status[R], iters[R] | rr[R] at byte 128*4
   cudaEvent_t ev = nullptr;
@@ -396,6 +404,10 @@ struct Plan {
   DBuf<double> d_nodes;           // [n][d]
   DBuf<double> d_vinv;            // [n_pad][n_pad] row-major, zero padded
   DBuf<float> d_vinv32;
+  DBuf<double> d_vinvt;           // the transpose
+  DBuf<float> d_vinvt32;
+  DBuf<int32_t> d_act;            // dimensions with a degree above 0
+  DBuf<double2> d_leg64;          // Legendre recurrence
   bool have_nodes = false;
 
   // tree (Sec. 5.1)
@@ -470,6 +482,7 @@ struct Plan {
   DBuf<float> bq32;           // TF32 hi/lo charge blocks for the tensor-core P2P
   DBuf<float> bqm32;          // the same for the tensor-core M2L (moments at the nodes)
   DBuf<int32_t> part_rows;    // the near lists in parts
+  DBuf<float> entry_parts32;  // one sum per near entry (steady near field)
   DBuf<float> near_parts32;   // partial near-field sums of small float32 problems
   DBuf<double> near_parts64;  // partial near-field sums of small float64 problems (split lists)
   // symmetric float64 near field: upper entries (T, S >= T) of the near list,
@@ -522,7 +535,8 @@ struct Plan {
   CgState cgs;
 
   ExpDev exp_dev() const {
-    return ExpDev{n, n_pad, d, lsum, nnz_max, d_fac.p, d_qk.p, d_loff.p};
+    return ExpDev{n, n_pad, d, lsum, nnz_max, d_fac.p, d_qk.p, d_loff.p, d_act.p, static_cast<int>(d_act.n),
+                  d_leg64.p};
   }
   TreeDev tree_dev() const { return TreeDev{N, J, L, C, m_pad, d_begin.p, d_count.p}; }
   void free_tree();
@@ -540,9 +554,10 @@ void build_cluster_data(Plan& P);           // extents, nodes, leaf-blocked site
 
 // ---- matvec (farfield.cu, nearfield.cu, matvec.cu) ----
 // x, y: device, caller order, column-major.
-void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy, int R, bool fp64);
+// steady: the sums keep one order (CG iterations, see apply_op in solve.cu).
+void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy, int R, bool fp64,
+                   bool steady = false);
 void ensure_workspace(Plan& P, bool fp64);
-void farfield_set_smem_limits(Plan& P);
 size_t farfield_smem_need(const Plan& P, bool fp64);
 // colmax: also the columns' largest magnitudes (float64 sums in fixed point;
 // the scatter of the same pass clears them); xq: also the float32 charges
@@ -550,11 +565,11 @@ size_t farfield_smem_need(const Plan& P, bool fp64);
 void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64, bool colmax = false,
                    float* xq = nullptr);
 void launch_scatter(Plan& P, double* y, int64_t ldy, int r0, int Rc, bool fp64);
-void launch_farfield(Plan& P, int Rc, bool fp64);
+void launch_farfield(Plan& P, int Rc, bool fp64, bool steady);
 bool farfield_tc_eligible(const Plan& P);   // farfield_tc.cu
-void farfield_tc(Plan& P, int Rc);
-void launch_m2l(Plan& P, int Rc, bool fp64);
-void launch_nearfield(Plan& P, int Rc, bool fp64, bool rot, cudaStream_t s);
+void farfield_tc(Plan& P, int Rc, bool steady);
+void launch_m2l(Plan& P, int Rc, bool fp64, bool steady);
+void launch_nearfield(Plan& P, int Rc, bool fp64, bool rot, bool steady, cudaStream_t s);
 // Bit of the current device in a per-device mask (kernel attributes are set
 // per device); devices beyond 63 get no bit, so their setup simply repeats.
 uint64_t device_bit();
@@ -571,12 +586,13 @@ void near_rot(Plan& P, int D, int Rc, cudaStream_t s);
 bool fix_ready(Plan& P);                    // sum_fix.cu: fixed-point float64 sums
 bool near_fix(Plan& P, int Rc, cudaStream_t s);
 bool m2l_fix(Plan& P, int Rc);
-bool p2p_f32_tuned(Plan& P, int Rc, bool rot, cudaStream_t s);
-bool m2l_f32_tuned(Plan& P, int Rc);
+bool p2p_f32_tuned(Plan& P, int Rc, bool rot, bool steady, cudaStream_t s);
+bool m2l_f32_tuned(Plan& P, int Rc, bool steady);
 void check_device_error(Plan& P);
 // batches (batch.cu uses these)
 void batch_far_attrs();
-size_t batch_far_smem(int lsum, int n_pad);
+size_t batch_far_smem(int lsum, int n, int n_pad, int nnz, int Rmax);
+size_t batch_far_need(int lsum, int n_pad);   // what the limit on index sets looks at
 void launch_moments_batched(const ProbF32* probs, const int2* work, int items, size_t smem, cudaStream_t s);
 void launch_downward_batched(const ProbF32* probs, const int2* work, int items, size_t smem, cudaStream_t s);
 void launch_gather_batched(const ProbF32* probs, const int* leaf_off, int P, int Ltot, int ld, float* xb,

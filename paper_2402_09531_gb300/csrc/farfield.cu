@@ -14,6 +14,7 @@
 // P2M and M2M are one kernel (Legendre moments of a box from point charges,
 // then V^{-T}); L2L, V^{-1} and (on the leaf level) L2P are one kernel.
 #include <algorithm>
+#include <atomic>
 
 #include "dwfmm_internal.cuh"
 #include "p2p_rot.cuh"
@@ -24,232 +25,330 @@ namespace dw {
 namespace {
 
 constexpr int kFarThreads = 128;
-constexpr int kChunk = 32;
+constexpr size_t kFarMaxSmem = 200 * 1024;
+constexpr int kAcceptChunk = 32;               // farfield_smem_need: the limit on index sets
+constexpr size_t kFarTableBytes = 40 * 1024;   // Legendre tables of a chunk of points
 
-// p_hat_j(t) = sqrt(2j+1) P_j(2t-1), j = 0..qk.
+// Stride of a point's Legendre table (odd: consecutive points fall into
+// different banks); its last used slot holds 1, the value of a missing factor.
+__host__ __device__ constexpr int far_stride(int lsum) { return (lsum + 1) | 1; }
+
+// Points per chunk of tables.
 template <typename T>
-__device__ __forceinline__ void legendre_row(T t, int qk, T* tab) {
+__host__ __device__ constexpr int far_points(int lsum) {
+  const int most = static_cast<int>(kFarTableBytes / sizeof(T)) / far_stride(lsum);
+  return most >= 128 ? 128 : most >= 64 ? 64 : 32;
+}
+
+// Shared memory of both passes: tables, two arrays of n_pad x RC, the threads'
+// partial sums, a chunk's charges, the multi-indices.
+template <typename T>
+constexpr size_t far_smem(int lsum, int n, int n_pad, int nnz, int RC) {
+  const int pc = far_points<T>(lsum);
+  return (static_cast<size_t>(pc) * far_stride(lsum) + (2 * static_cast<size_t>(n_pad) + kFarThreads + pc) * RC) *
+             sizeof(T) +
+         static_cast<size_t>(n) * nnz * sizeof(int16_t);
+}
+
+// Order of the sums.  STEADY: one thread a row of results, its terms in order,
+// and P_j by its division, then the factor sqrt(2j+1): what the conjugate
+// gradient iterations repeat bit for bit (apply_op in solve.cu); float32 always
+// runs so.  Otherwise (float64): several threads a row and the recurrence from a
+// table.
+template <typename T, bool STEADY>
+constexpr bool in_order() { return STEADY || sizeof(T) == 4; }
+
+// p_hat_j(t) = sqrt(2j+1) P_j(2t-1), j = 1 .. deg, into row[j]; not in order: by
+// the normalised recurrence p_{j+1} = a_j u p_j - b_j p_{j-1} (a division and a
+// root are ~20 instructions each on a float64 unit of 2 a clock).
+template <typename T, bool STEADY>
+__device__ __forceinline__ void legendre_row(const ExpDev& e, T t, int deg, T* row) {
   const T u = T(2) * t - T(1);
-  T pm = T(1), pc = u;
-  tab[0] = T(1);
-  if (qk >= 1) tab[1] = u * sqrt(T(3));
-  for (int j = 1; j < qk; ++j) {
-    const T pn = (T(2 * j + 1) * u * pc - T(j) * pm) / T(j + 1);
-    tab[j + 1] = pn * sqrt(T(2 * j + 3));
-    pm = pc;
-    pc = pn;
+  if constexpr (in_order<T, STEADY>()) {
+    T pm = T(1), pc = u;
+    row[1] = u * sqrt(T(3));
+    for (int j = 1; j < deg; ++j) {
+      const T pn = (T(2 * j + 1) * u * pc - T(j) * pm) / T(j + 1);
+      row[j + 1] = pn * sqrt(T(2 * j + 3));
+      pm = pc;
+      pc = pn;
+    }
+  } else {
+    double prev = 1.0, cur = e.leg64[0].x * u;
+    row[1] = cur;
+    for (int j = 1; j < deg; ++j) {
+      const double2 c = e.leg64[j];
+      const double next = c.x * u * cur - c.y * prev;
+      row[j + 1] = next;
+      prev = cur;
+      cur = next;
+    }
   }
 }
 
+// Legendre tables of cn points at t = (y - lo) iext, one point and dimension
+// per thread and step.  Only dimensions with a degree above 0 are looked at,
+// and degree 0 is not stored (a factor never names it).  point(p): the point's
+// first coordinate; ys: between coordinates.
+template <typename T, bool STEADY, class F>
+__device__ __forceinline__ void fill_tables(const ExpDev& e, int cn, int ys, const T* lo, const T* iext, T* tab,
+                                            F point) {
+  const int LS = far_stride(e.lsum);
+  const int tid = static_cast<int>(threadIdx.x);
+  for (int p = tid; p < cn; p += kFarThreads) tab[p * LS + e.lsum] = T(1);
+  for (int q = tid; q < cn * e.nact; q += kFarThreads) {
+    const int m = q / cn, p = q - m * cn;
+    const int k = e.act[m];
+    const T t = (point(p)[static_cast<int64_t>(k) * ys] - lo[k]) * iext[k];
+    legendre_row<T, STEADY>(e, t, e.qk[k], tab + p * LS + e.loff[k]);
+  }
+}
+
+// Basis value of the multi-index with factors fac[0..nnz) at a point's table.
 template <typename T>
 __device__ __forceinline__ T basis_value(const T* tab, const int16_t* fac, int nnz) {
-  T v = T(1);
-  for (int z = 0; z < nnz; ++z) {
-    const int o = fac[z];
-    if (o < 0) break;
-    v *= tab[o];
-  }
+  T v = tab[fac[0]];
+  for (int z = 1; z < nnz; ++z) v *= tab[fac[z]];
   return v;
 }
 
-// Legendre table of one point: for every dimension k the values at
-// t_k = (y_k - lo_k) * iext_k.
-template <typename T>
-__device__ __forceinline__ void point_table(const ExpDev& e, const T* y, int64_t ystride,
-                                            const T* lo, const T* iext, T* tab) {
-  for (int k = 0; k < e.d; ++k) {
-    const T t = (y[k * ystride] - lo[k]) * iext[k];
-    legendre_row<T>(t, e.qk[k], tab + e.loff[k]);
+// Multi-indices in shared memory, missing factors pointing at the slot of 1.
+__device__ __forceinline__ void load_factors(const ExpDev& e, int16_t* fac) {
+  for (int i = threadIdx.x; i < e.n * e.nnz_max; i += kFarThreads) {
+    const int16_t f = e.fac[i];
+    fac[i] = f < 0 ? static_cast<int16_t>(e.lsum) : f;
   }
 }
 
-// Moments of cluster g = first + blockIdx.x, then m = V^{-T} mu.
+// Threads over `rows` results: one thread a row (in order), or thread (row, sub)
+// sums the terms sub, sub + nsub, ..., and `reduce` adds a row's sums; small
+// index sets (10 indices are common) leave most of the CTA idle with one thread
+// a row.
+template <typename T, bool STEADY>
+struct Split {
+  int per, row, sub, nsub;
+  bool on;
+  __device__ __forceinline__ explicit Split(int rows) {
+    per = rows < kFarThreads ? rows : kFarThreads;
+    nsub = in_order<T, STEADY>() ? 1 : kFarThreads / per;
+    sub = static_cast<int>(threadIdx.x) / per;
+    row = static_cast<int>(threadIdx.x) - sub * per;
+    on = sub < nsub;
+  }
+};
+
+// put(row, r, value) for every row and right-hand side; red: kFarThreads x RC.
+template <typename T, int RC, class S, class F>
+__device__ __forceinline__ void reduce(const S& s, int rows, const T (&acc)[RC], T* red, F put) {
+  __syncthreads();
+  if (s.on) {
+#pragma unroll
+    for (int r = 0; r < RC; ++r) red[(s.sub * s.per + s.row) * RC + r] = acc[r];
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < rows * RC; q += kFarThreads) {
+    T v = red[q];
+    for (int u = 1; u < s.nsub; ++u) v += red[u * s.per * RC + q];
+    put(q / RC, q % RC, v);
+  }
+}
+
+// Moments of cluster g, then m = V^{-T} mu, for the right-hand sides r0 .. r0 +
+// RC - 1 (rows beyond Rc zero).
 //  leaf mode:     sources = the leaf's sites, charges = right-hand sides.
 //  children mode: sources = nodes of both children, charges = their m.
-template <typename T>
+template <typename T, int RC, bool STEADY>
 __device__ __forceinline__ void moments_body(const ExpDev& e, int g, int leaf_mode, int L, const int32_t* count,
                                              const T* pts, int m_pad, const T* xb, const T* ynode,
-                                             const T* lo_all, const T* iext_all, const T* vinv, int Rc, T* mom) {
-  extern __shared__ unsigned char smem_raw[];
-  T* tab = reinterpret_cast<T*>(smem_raw);          // [kChunk][lsum]
-  T* qs = tab + kChunk * e.lsum;                   // [kChunk][kRC]
-  T* mu = qs + kChunk * kRC;                       // [n_pad][kRC]
-  const int n = e.n, np = e.n_pad, d = e.d;
+                                             const T* lo_all, const T* iext_all, const T* vinv, int r0, int Rc, T* mom) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n = e.n, np = e.n_pad, d = e.d, nnz = e.nnz_max;
+  const int LS = far_stride(e.lsum), PC = far_points<T>(e.lsum);
+  T* tab = reinterpret_cast<T*>(smem_raw);     // [PC][LS]
+  T* mu = tab + PC * LS;                       // [n_pad][RC]
+  T* red = mu + 2 * np * RC;                   // [kFarThreads][RC]
+  T* qs = red + kFarThreads * RC;              // [PC][RC]
+  int16_t* fac = reinterpret_cast<int16_t*>(qs + PC * RC);
   const T* lo = lo_all + static_cast<int64_t>(g) * d;
   const T* iext = iext_all + static_cast<int64_t>(g) * d;
-  int S;
-  if (leaf_mode) S = count[g];
-  else S = 2 * n;
-
+  const int leaf = g - (L - 1);
+  const int S = leaf_mode ? count[g] : 2 * n;
+  load_factors(e, fac);
+  auto point = [&](int p) -> const T* {
+    if (leaf_mode) return pts + static_cast<int64_t>(leaf) * d * m_pad + p;
+    const int ch = p >= n ? 1 : 0;
+    return ynode + static_cast<int64_t>(2 * g + 1 + ch) * d * np + (p - ch * n);
+  };
+  auto charge = [&](int p, int r) -> T {
+    if (r0 + r >= Rc) return T(0);
+    if (leaf_mode) return xb[(static_cast<int64_t>(leaf) * kRC + r0 + r) * m_pad + p];
+    const int ch = p >= n ? 1 : 0;
+    return mom[(static_cast<int64_t>(2 * g + 1 + ch) * kRC + r0 + r) * np + (p - ch * n)];
+  };
   for (int ab = 0; ab < n; ab += kFarThreads) {
-    const int a = ab + threadIdx.x;
-    T acc[kRC];
+    const int rows = min(kFarThreads, n - ab);
+    const Split<T, STEADY> s(rows);
+    T acc[RC];
 #pragma unroll
-    for (int r = 0; r < kRC; ++r) acc[r] = T(0);
-    for (int cb = 0; cb < S; cb += kChunk) {
-      const int cn = min(kChunk, S - cb);
-      if (threadIdx.x < cn) {
-        const int p = cb + threadIdx.x;
-        const T* y;
-        int64_t ys;
-        if (leaf_mode) {
-          y = pts + static_cast<int64_t>(g - (L - 1)) * d * m_pad + p;
-          ys = m_pad;
-        } else {
-          const int ch = 2 * g + 1 + (p >= n);
-          const int pa = p % n;
-          y = ynode + static_cast<int64_t>(ch) * d * np + pa;
-          ys = np;
-        }
-        point_table<T>(e, y, ys, lo, iext, tab + threadIdx.x * e.lsum);
-      }
-      for (int idx = threadIdx.x; idx < cn * kRC; idx += kFarThreads) {
-        const int pl = idx / kRC, r = idx % kRC;
-        const int p = cb + pl;
-        T v = T(0);
-        if (r < Rc) {
-          if (leaf_mode) v = xb[(static_cast<int64_t>(g - (L - 1)) * kRC + r) * m_pad + p];
-          else {
-            const int ch = 2 * g + 1 + (p >= n);
-            v = mom[(static_cast<int64_t>(ch) * kRC + r) * np + (p % n)];
-          }
-        }
-        qs[idx] = v;
-      }
+    for (int r = 0; r < RC; ++r) acc[r] = T(0);
+    for (int cb = 0; cb < S; cb += PC) {
+      const int cn = min(PC, S - cb);
       __syncthreads();
-      if (a < n) {
-        const int16_t* fac = e.fac + a * e.nnz_max;
-        for (int pl = 0; pl < cn; ++pl) {
-          const T b = basis_value<T>(tab + pl * e.lsum, fac, e.nnz_max);
+      fill_tables<T, STEADY>(e, cn, leaf_mode ? m_pad : np, lo, iext, tab, [&](int p) { return point(cb + p); });
 #pragma unroll
-          for (int r = 0; r < kRC; ++r) acc[r] += b * qs[pl * kRC + r];
+      for (int r = 0; r < RC; ++r)
+        for (int p = threadIdx.x; p < cn; p += kFarThreads) qs[p * RC + r] = charge(cb + p, r);
+      __syncthreads();
+      if (s.on) {
+        const int16_t* f = fac + (ab + s.row) * nnz;
+        for (int p = s.sub; p < cn; p += s.nsub) {
+          const T b = basis_value<T>(tab + p * LS, f, nnz);
+#pragma unroll
+          for (int r = 0; r < RC; ++r) acc[r] += b * qs[p * RC + r];
         }
       }
-      __syncthreads();
     }
-    if (a < np) {
-#pragma unroll
-      for (int r = 0; r < kRC; ++r) mu[a * kRC + r] = (a < n) ? acc[r] : T(0);
-    }
+    reduce<T, RC>(s, rows, acc, red, [&](int a, int r, T v) { mu[(ab + a) * RC + r] = v; });
   }
   __syncthreads();
   // m = V^{-T} mu
-  for (int a = threadIdx.x; a < np; a += kFarThreads) {
-    T out[kRC];
+  for (int ab = 0; ab < n; ab += kFarThreads) {
+    const int rows = min(kFarThreads, n - ab);
+    const Split<T, STEADY> s(rows);
+    T acc[RC];
 #pragma unroll
-    for (int r = 0; r < kRC; ++r) out[r] = T(0);
-    for (int b = 0; b < n; ++b) {
-      const T v = vinv[b * np + a];
+    for (int r = 0; r < RC; ++r) acc[r] = T(0);
+    if (s.on)
+      for (int b = s.sub; b < n; b += s.nsub) {
+        const T v = vinv[b * np + ab + s.row];
 #pragma unroll
-      for (int r = 0; r < kRC; ++r) out[r] += v * mu[b * kRC + r];
-    }
-    for (int r = 0; r < kRC; ++r) mom[(static_cast<int64_t>(g) * kRC + r) * np + a] = r < Rc ? out[r] : T(0);
+        for (int r = 0; r < RC; ++r) acc[r] += v * mu[b * RC + r];
+      }
+    reduce<T, RC>(s, rows, acc, red, [&](int a, int r, T v) {
+      mom[(static_cast<int64_t>(g) * kRC + r0 + r) * np + ab + a] = r0 + r < Rc ? v : T(0);
+    });
   }
+  for (int q = threadIdx.x; q < (np - n) * RC; q += kFarThreads)
+    mom[(static_cast<int64_t>(g) * kRC + r0 + q / (np - n)) * np + n + q % (np - n)] = T(0);
 }
 
-template <typename T>
+// One cluster per CTA, RC right-hand sides in registers.  Bound by latency (a
+// few thousand clocks a level) and, at float64, by the unit's 2 multiply-adds a
+// clock: d = 4, N = 4096 float64, 10 indices, 1 right-hand side, 4 levels:
+// 164 us with 16 right-hand sides' sums in 10 threads, 34 us with one side's
+// in 120.
+template <typename T, int RC, bool STEADY>
 __global__ void __launch_bounds__(kFarThreads)
 k_moments(ExpDev e, int first, int leaf_mode, int L, const int32_t* count, const T* pts, int m_pad,
-          const T* xb, const T* ynode, const T* lo_all, const T* iext_all, const T* vinv, int Rc,
+          const T* xb, const T* ynode, const T* lo_all, const T* iext_all, const T* vinv, int r0, int Rc,
           T* mom) {
-  moments_body<T>(e, first + blockIdx.x, leaf_mode, L, count, pts, m_pad, xb, ynode, lo_all, iext_all, vinv,
-                  Rc, mom);
+  moments_body<T, RC, STEADY>(e, first + blockIdx.x, leaf_mode, L, count, pts, m_pad, xb, ynode, lo_all, iext_all, vinv,
+                      r0, Rc, mom);
 }
 
-// Downward pass on cluster g = first + blockIdx.x (level `level`):
+// Downward pass on cluster g of level `level`, right-hand sides r0 .. r0 + RC - 1:
 //   l_g += B_g lambda_parent  (if level > jmin), lambda_g = V^{-1} l_g,
 //   and on the leaf level y_far = P_leaf lambda_leaf.
-template <typename T>
+// vinvt: the transpose of V^{-1} (consecutive threads read consecutive entries).
+template <typename T, int RC, bool STEADY>
 __device__ __forceinline__ void downward_body(const ExpDev& e, int g, int level, int jmin, int J, int L,
                                               const int32_t* count, const T* pts, int m_pad, const T* ynode,
                                               const T* lo_all, const T* iext_all, const T* loc, T* lco,
-                                              const T* vinv, int Rc, T* yfar) {
-  extern __shared__ unsigned char smem_raw[];
-  T* lamp = reinterpret_cast<T*>(smem_raw);        // [n_pad][kRC]
-  T* lsm = lamp + e.n_pad * kRC;                  // [n_pad][kRC]
-  T* tab = lsm + e.n_pad * kRC;                   // [kFarThreads][lsum]
-  const int n = e.n, np = e.n_pad, d = e.d;
-  for (int idx = threadIdx.x; idx < np * kRC; idx += kFarThreads) {
-    const int a = idx / kRC, r = idx % kRC;
-    lsm[idx] = (r < Rc && a < n) ? loc[(static_cast<int64_t>(g) * kRC + r) * np + a] : T(0);
-  }
+                                              const T* vinvt, int r0, int Rc, T* yfar) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n = e.n, np = e.n_pad, d = e.d, nnz = e.nnz_max;
+  const int LS = far_stride(e.lsum), PC = far_points<T>(e.lsum);
+  T* tab = reinterpret_cast<T*>(smem_raw);     // [PC][LS]
+  T* lamp = tab + PC * LS;                     // [n_pad][RC]
+  T* lsm = lamp + np * RC;                     // [n_pad][RC]
+  T* red = lsm + np * RC;                      // [kFarThreads][RC]
+  int16_t* fac = reinterpret_cast<int16_t*>(red + (kFarThreads + PC) * RC);
+  load_factors(e, fac);
+  auto row_of = [&](const T* x, int c, T* dst) {
+#pragma unroll
+    for (int r = 0; r < RC; ++r)
+      for (int a = threadIdx.x; a < n; a += kFarThreads)
+        dst[a * RC + r] = r0 + r < Rc ? x[(static_cast<int64_t>(c) * kRC + r0 + r) * np + a] : T(0);
+  };
+  row_of(loc, g, lsm);
   if (level > jmin) {
     const int p = (g - 1) / 2;
-    for (int idx = threadIdx.x; idx < np * kRC; idx += kFarThreads) {
-      const int a = idx / kRC, r = idx % kRC;
-      lamp[idx] = (r < Rc && a < n) ? lco[(static_cast<int64_t>(p) * kRC + r) * np + a] : T(0);
-    }
-    __syncthreads();
+    row_of(lco, p, lamp);
     const T* lo = lo_all + static_cast<int64_t>(p) * d;
     const T* iext = iext_all + static_cast<int64_t>(p) * d;
-    T* mytab = tab + threadIdx.x * e.lsum;
-    for (int ab = 0; ab < n; ab += kFarThreads) {
-      const int a = ab + threadIdx.x;
-      if (a < n) {
-        point_table<T>(e, ynode + static_cast<int64_t>(g) * d * np + a, np, lo, iext, mytab);
-        T acc[kRC];
+    const T* yn = ynode + static_cast<int64_t>(g) * d * np;
+    for (int ab = 0; ab < n; ab += PC) {
+      const int rows = min(PC, n - ab);
+      __syncthreads();
+      fill_tables<T, STEADY>(e, rows, np, lo, iext, tab, [&](int a) { return yn + ab + a; });
+      __syncthreads();
+      const Split<T, STEADY> s(rows);
+      T acc[RC];
 #pragma unroll
-        for (int r = 0; r < kRC; ++r) acc[r] = T(0);
-        for (int b = 0; b < n; ++b) {
-          const T v = basis_value<T>(mytab, e.fac + b * e.nnz_max, e.nnz_max);
+      for (int r = 0; r < RC; ++r) acc[r] = T(0);
+      if (s.on)
+        for (int b = s.sub; b < n; b += s.nsub) {
+          const T v = basis_value<T>(tab + s.row * LS, fac + b * nnz, nnz);
 #pragma unroll
-          for (int r = 0; r < kRC; ++r) acc[r] += v * lamp[b * kRC + r];
+          for (int r = 0; r < RC; ++r) acc[r] += v * lamp[b * RC + r];
         }
-#pragma unroll
-        for (int r = 0; r < kRC; ++r) lsm[a * kRC + r] += acc[r];
-      }
+      reduce<T, RC>(s, rows, acc, red, [&](int a, int r, T v) { lsm[(ab + a) * RC + r] += v; });
     }
   }
   __syncthreads();
   // lambda_g = V^{-1} l_g  (into lamp)
-  for (int a = threadIdx.x; a < np; a += kFarThreads) {
-    T out[kRC];
+  for (int ab = 0; ab < n; ab += kFarThreads) {
+    const int rows = min(kFarThreads, n - ab);
+    const Split<T, STEADY> s(rows);
+    T acc[RC];
 #pragma unroll
-    for (int r = 0; r < kRC; ++r) out[r] = T(0);
-    for (int b = 0; b < n; ++b) {
-      const T v = vinv[a * np + b];
+    for (int r = 0; r < RC; ++r) acc[r] = T(0);
+    if (s.on)
+      for (int b = s.sub; b < n; b += s.nsub) {
+        const T v = vinvt[b * np + ab + s.row];
 #pragma unroll
-      for (int r = 0; r < kRC; ++r) out[r] += v * lsm[b * kRC + r];
-    }
-#pragma unroll
-    for (int r = 0; r < kRC; ++r) {
-      lamp[a * kRC + r] = out[r];
-      if (level < J) lco[(static_cast<int64_t>(g) * kRC + r) * np + a] = out[r];
-    }
+        for (int r = 0; r < RC; ++r) acc[r] += v * lsm[b * RC + r];
+      }
+    reduce<T, RC>(s, rows, acc, red, [&](int a, int r, T v) {
+      lamp[(ab + a) * RC + r] = v;
+      if (level < J) lco[(static_cast<int64_t>(g) * kRC + r0 + r) * np + ab + a] = v;
+    });
   }
   if (level < J) return;
-  __syncthreads();
   // L2P on the leaf's sites
   const int leaf = g - (L - 1);
   const int cnt = count[g];
   const T* lo = lo_all + static_cast<int64_t>(g) * d;
   const T* iext = iext_all + static_cast<int64_t>(g) * d;
-  T* mytab = tab + threadIdx.x * e.lsum;
-  for (int ib = 0; ib < m_pad; ib += kFarThreads) {
-    const int i = ib + threadIdx.x;
-    if (i >= m_pad) break;
-    T acc[kRC];
+  const T* pp = pts + static_cast<int64_t>(leaf) * d * m_pad;
+  for (int ib = 0; ib < cnt; ib += PC) {
+    const int rows = min(PC, cnt - ib);
+    __syncthreads();
+    fill_tables<T, STEADY>(e, rows, m_pad, lo, iext, tab, [&](int i) { return pp + ib + i; });
+    __syncthreads();
+    const Split<T, STEADY> s(rows);
+    T acc[RC];
 #pragma unroll
-    for (int r = 0; r < kRC; ++r) acc[r] = T(0);
-    if (i < cnt) {
-      point_table<T>(e, pts + static_cast<int64_t>(leaf) * d * m_pad + i, m_pad, lo, iext, mytab);
-      for (int b = 0; b < n; ++b) {
-        const T v = basis_value<T>(mytab, e.fac + b * e.nnz_max, e.nnz_max);
+    for (int r = 0; r < RC; ++r) acc[r] = T(0);
+    if (s.on)
+      for (int b = s.sub; b < n; b += s.nsub) {
+        const T v = basis_value<T>(tab + s.row * LS, fac + b * nnz, nnz);
 #pragma unroll
-        for (int r = 0; r < kRC; ++r) acc[r] += v * lamp[b * kRC + r];
+        for (int r = 0; r < RC; ++r) acc[r] += v * lamp[b * RC + r];
       }
-    }
-    for (int r = 0; r < Rc; ++r) yfar[(static_cast<int64_t>(leaf) * kRC + r) * m_pad + i] = acc[r];
+    reduce<T, RC>(s, rows, acc, red, [&](int i, int r, T v) {
+      if (r0 + r < Rc) yfar[(static_cast<int64_t>(leaf) * kRC + r0 + r) * m_pad + ib + i] = v;
+    });
   }
 }
 
-template <typename T>
+template <typename T, int RC, bool STEADY>
 __global__ void __launch_bounds__(kFarThreads)
 k_downward(ExpDev e, int first, int level, int jmin, int J, int L, const int32_t* count,
            const T* pts, int m_pad, const T* ynode, const T* lo_all, const T* iext_all,
-           const T* loc, T* lco, const T* vinv, int Rc, T* yfar) {
-  downward_body<T>(e, first + blockIdx.x, level, jmin, J, L, count, pts, m_pad, ynode, lo_all, iext_all, loc,
-                   lco, vinv, Rc, yfar);
+           const T* loc, T* lco, const T* vinvt, int r0, int Rc, T* yfar) {
+  downward_body<T, RC, STEADY>(e, first + blockIdx.x, level, jmin, J, L, count, pts, m_pad, ynode, lo_all, iext_all, loc,
+                       lco, vinvt, r0, Rc, yfar);
 }
 
 // ---- many problems in one launch (batches) --------------------------------
@@ -258,20 +357,36 @@ k_downward(ExpDev e, int first, int level, int jmin, int J, int L, const int32_t
 
 __device__ __forceinline__ int level_of(int g) { return 31 - __clz(g + 1); }
 
+// Up to 4 right-hand sides in registers, or up to 16.
+__device__ __forceinline__ void moments_item(const ProbF32& p, int c) {
+  const int leaf = level_of(c) == p.J;
+  if (p.R <= 4)
+    moments_body<float, 4, true>(p.e, c, leaf, p.L, p.count, p.pts, p.m_pad, p.xb, p.ynode, p.lo, p.iext, p.vinv, 0, p.R,
+                           p.mom);
+  else
+    moments_body<float, 16, true>(p.e, c, leaf, p.L, p.count, p.pts, p.m_pad, p.xb, p.ynode, p.lo, p.iext, p.vinv, 0, p.R,
+                            p.mom);
+}
+
+__device__ __forceinline__ void downward_item(const ProbF32& p, int c) {
+  if (p.R <= 4)
+    downward_body<float, 4, true>(p.e, c, level_of(c), p.jmin, p.J, p.L, p.count, p.pts, p.m_pad, p.ynode, p.lo, p.iext,
+                            p.loc, p.lco, p.vinvt, 0, p.R, p.yfar);
+  else
+    downward_body<float, 16, true>(p.e, c, level_of(c), p.jmin, p.J, p.L, p.count, p.pts, p.m_pad, p.ynode, p.lo, p.iext,
+                             p.loc, p.lco, p.vinvt, 0, p.R, p.yfar);
+}
+
 __global__ void __launch_bounds__(kFarThreads)
 k_moments_batched(const ProbF32* probs, const int2* work) {
   const int2 w = work[blockIdx.x];
-  const ProbF32& p = probs[w.x];
-  moments_body<float>(p.e, w.y, level_of(w.y) == p.J, p.L, p.count, p.pts, p.m_pad, p.xb, p.ynode, p.lo, p.iext,
-                      p.vinv, p.R, p.mom);
+  moments_item(probs[w.x], w.y);
 }
 
 __global__ void __launch_bounds__(kFarThreads)
 k_downward_batched(const ProbF32* probs, const int2* work) {
   const int2 w = work[blockIdx.x];
-  const ProbF32& p = probs[w.x];
-  downward_body<float>(p.e, w.y, level_of(w.y), p.jmin, p.J, p.L, p.count, p.pts, p.m_pad, p.ynode, p.lo, p.iext,
-                       p.loc, p.lco, p.vinv, p.R, p.yfar);
+  downward_item(probs[w.x], w.y);
 }
 
 // Problem of a global leaf (binary search in the leaf offsets).
@@ -594,9 +709,7 @@ __device__ __noinline__ bool persist_barrier(const PersistArgs& pa, int ph, bool
 __device__ __forceinline__ void persist_up_items(const PersistArgs& pa, int h) {
   for (int i = static_cast<int>(blockIdx.x); i < pa.up_cnt[h]; i += static_cast<int>(gridDim.x)) {
     const int2 w = pa.work[pa.up_off[h] + i];
-    const ProbF32& p = pa.probs[w.x];
-    moments_body<float>(p.e, w.y, level_of(w.y) == p.J, p.L, p.count, p.pts, p.m_pad, p.xb, p.ynode, p.lo, p.iext,
-                        p.vinv, p.R, p.mom);
+    moments_item(pa.probs[w.x], w.y);
     __syncthreads();
   }
 }
@@ -604,9 +717,7 @@ __device__ __forceinline__ void persist_up_items(const PersistArgs& pa, int h) {
 __device__ __forceinline__ void persist_down_items(const PersistArgs& pa, int j) {
   for (int i = static_cast<int>(blockIdx.x); i < pa.down_cnt[j]; i += static_cast<int>(gridDim.x)) {
     const int2 w = pa.work[pa.down_off[j] + i];
-    const ProbF32& p = pa.probs[w.x];
-    downward_body<float>(p.e, w.y, level_of(w.y), p.jmin, p.J, p.L, p.count, p.pts, p.m_pad, p.ynode, p.lo, p.iext,
-                         p.loc, p.lco, p.vinv, p.R, p.yfar);
+    downward_item(pa.probs[w.x], w.y);
     __syncthreads();
   }
 }
@@ -773,7 +884,7 @@ __global__ void k_scatter(double* y, int64_t ldy, int r0, int Rc, const int32_t*
 template <typename T>
 struct Bufs {
   T *xb, *ynear, *yfar, *mom, *loc, *lco;
-  const T *pts, *ynode, *lo, *iext, *vinv;
+  const T *pts, *ynode, *lo, *iext, *vinv, *vinvt;
 };
 
 template <typename T>
@@ -782,74 +893,97 @@ Bufs<T> bufs(Plan& P);
 template <>
 Bufs<double> bufs<double>(Plan& P) {
   return Bufs<double>{P.xb64.p,   P.ynear64.p, P.yfar64.p,  P.mom64.p,  P.loc64.p, P.lco64.p,
-                      P.d_pts64.p, P.d_ynode64.p, P.d_lo.p, P.d_iext.p, P.d_vinv.p};
+                      P.d_pts64.p, P.d_ynode64.p, P.d_lo.p, P.d_iext.p, P.d_vinv.p, P.d_vinvt.p};
 }
 template <>
 Bufs<float> bufs<float>(Plan& P) {
   return Bufs<float>{P.xb32.p,   P.ynear32.p, P.yfar32.p,  P.mom32.p,   P.loc32.p,  P.lco32.p,
-                     P.d_pts32.p, P.d_ynode32.p, P.d_lo32.p, P.d_iext32.p, P.d_vinv32.p};
+                     P.d_pts32.p, P.d_ynode32.p, P.d_lo32.p, P.d_iext32.p, P.d_vinv32.p, P.d_vinvt32.p};
+}
+
+// Upward passes (levels J .. jmin) or downward passes (jmin .. J).
+template <typename T, int RC, bool STEADY>
+int far_levels(Plan& P, bool up, int Rc) {
+  cudaStream_t s = P.stream;
+  const Bufs<T> B = bufs<T>(P);
+  const ExpDev e = P.exp_dev();
+  const int J = P.J, L = P.L;
+  const size_t smem = far_smem<T>(e.lsum, e.n, e.n_pad, e.nnz_max, RC);
+  static std::atomic<uint64_t> done{0};
+  const uint64_t bit = device_bit();
+  if (!(done.load() & bit)) {   // large index sets
+    DW_CUDA(cudaFuncSetAttribute(k_moments<T, RC, STEADY>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFarMaxSmem));
+    DW_CUDA(cudaFuncSetAttribute(k_downward<T, RC, STEADY>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFarMaxSmem));
+    done.fetch_or(bit);
+  }
+  int launches = 0;
+  for (int i = 0; i <= J - P.jmin; ++i) {
+    const int j = up ? J - i : P.jmin + i;
+    const int first = (1 << j) - 1;
+    for (int r0 = 0; r0 < Rc; r0 += RC, ++launches) {
+      if (up)
+        k_moments<T, RC, STEADY><<<1 << j, kFarThreads, smem, s>>>(e, first, j == J, L, P.d_count.p, B.pts, P.m_pad, B.xb,
+                                                           B.ynode, B.lo, B.iext, B.vinv, r0, Rc, B.mom);
+      else
+        k_downward<T, RC, STEADY><<<1 << j, kFarThreads, smem, s>>>(e, first, j, P.jmin, J, L, P.d_count.p, B.pts, P.m_pad,
+                                                            B.ynode, B.lo, B.iext, B.loc, B.lco, B.vinvt, r0, Rc,
+                                                            B.yfar);
+    }
+  }
+  return launches;
+}
+
+// The right-hand sides a thread keeps: the padded count, or fewer at a time
+// where an index set of hundreds of entries needs the shared memory.
+template <typename T, bool STEADY>
+int far_levels_rc(Plan& P, bool up, int Rc) {
+  auto fits = [&](int RC) { return far_smem<T>(P.lsum, P.n, P.n_pad, P.nnz_max, RC) <= kFarMaxSmem; };
+  if (Rc > 8 && fits(16)) return far_levels<T, 16, STEADY>(P, up, Rc);
+  if (Rc > 4 && fits(8)) return far_levels<T, 8, STEADY>(P, up, Rc);
+  if (Rc > 1 && fits(4)) return far_levels<T, 4, STEADY>(P, up, Rc);
+  return far_levels<T, 1, STEADY>(P, up, Rc);
 }
 
 template <typename T>
-void farfield_impl(Plan& P, int Rc) {
-  cudaStream_t s = P.stream;
-  Bufs<T> B = bufs<T>(P);
-  const ExpDev e = P.exp_dev();
-  const int J = P.J, L = P.L;
-  const int64_t ny = static_cast<int64_t>(L) * kRC * P.m_pad;
-  if (P.jmin > J) {  // no admissible block: the far field is empty
-    DW_CUDA(cudaMemsetAsync(B.yfar, 0, ny * sizeof(T), s));
+int far_pass(Plan& P, bool up, int Rc, bool steady) {
+  if (steady || sizeof(T) == 4) return far_levels_rc<T, true>(P, up, Rc);
+  return far_levels_rc<T, false>(P, up, Rc);
+}
+
+template <typename T>
+void farfield_impl(Plan& P, int Rc, bool steady) {
+  if (P.jmin > P.J) {  // no admissible block: the far field is empty (the scatter does not read it)
     P.far_engine = sizeof(T) == 8 ? 0 : 1;
     return;
   }
-  if (sizeof(T) == 4 && farfield_tc_eligible(P)) {
+  cudaStream_t s = P.stream;
+  // one or two right-hand sides leave the tensor tile of 16 columns empty: the
+  // CUDA cores take half as many launches, with work that fits the sides given
+  // (d = 16, 20 indices, N = 50021, 7 levels up and down: 375 us on the tensor
+  // cores; the error against float64 is 0.3 to 0.6 times as large, too)
+  if (sizeof(T) == 4 && (Rc > 2 || steady) && farfield_tc_eligible(P)) {
     P.far_engine = 2;
-    farfield_tc(P, Rc);
+    farfield_tc(P, Rc, steady);
     return;
   }
   P.far_engine = sizeof(T) == 8 ? 0 : 1;
-  const size_t sm_mom = (static_cast<size_t>(kChunk) * e.lsum + kChunk * kRC + static_cast<size_t>(e.n_pad) * kRC) * sizeof(T);
-  const size_t sm_down = (2 * static_cast<size_t>(e.n_pad) * kRC + static_cast<size_t>(kFarThreads) * e.lsum) * sizeof(T);
   timer_begin(P, 1, s);
-  int launches = 0;
-  for (int j = J; j >= P.jmin; --j) {
-    const int first = (1 << j) - 1;
-    k_moments<T><<<1 << j, kFarThreads, sm_mom, s>>>(e, first, j == J, L, P.d_count.p, B.pts, P.m_pad,
-                                                     B.xb, B.ynode, B.lo, B.iext, B.vinv, Rc, B.mom);
-    ++launches;
-  }
+  int launches = far_pass<T>(P, true, Rc, steady);
   timer_end(P, 1, s, launches);
   timer_begin(P, 2, s);
-  launch_m2l(P, Rc, sizeof(T) == 8);
+  launch_m2l(P, Rc, sizeof(T) == 8, steady);
   timer_end(P, 2, s, 1);
   timer_begin(P, 3, s);
-  launches = 0;
-  for (int j = P.jmin; j <= J; ++j) {
-    const int first = (1 << j) - 1;
-    k_downward<T><<<1 << j, kFarThreads, sm_down, s>>>(e, first, j, P.jmin, J, L, P.d_count.p, B.pts,
-                                                       P.m_pad, B.ynode, B.lo, B.iext, B.loc, B.lco,
-                                                       B.vinv, Rc, B.yfar);
-    ++launches;
-  }
+  launches = far_pass<T>(P, false, Rc, steady);
   timer_end(P, 3, s, launches);
   DW_CUDA(cudaGetLastError());
 }
 
 }  // namespace
 
-void farfield_set_smem_limits(Plan& P) {
-  // Raise the dynamic shared-memory limit once per plan (large index sets).
-  const int big = 200 * 1024;
-  DW_CUDA(cudaFuncSetAttribute(k_moments<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-  DW_CUDA(cudaFuncSetAttribute(k_moments<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-  DW_CUDA(cudaFuncSetAttribute(k_downward<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-  DW_CUDA(cudaFuncSetAttribute(k_downward<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-  (void)P;
-}
-
 size_t farfield_smem_need(const Plan& P, bool fp64) {
   const size_t es = fp64 ? 8 : 4;
-  const size_t a = (static_cast<size_t>(kChunk) * P.lsum + kChunk * kRC + static_cast<size_t>(P.n_pad) * kRC) * es;
+  const size_t a = (static_cast<size_t>(kAcceptChunk) * P.lsum + kAcceptChunk * kRC + static_cast<size_t>(P.n_pad) * kRC) * es;
   const size_t b = (2 * static_cast<size_t>(P.n_pad) * kRC + static_cast<size_t>(kFarThreads) * P.lsum) * es;
   return std::max(a, b);
 }
@@ -894,8 +1028,12 @@ void batch_far_attrs() {
   DW_CUDA(cudaFuncSetAttribute(k_downward_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
 }
 
-size_t batch_far_smem(int lsum, int n_pad) {
-  const size_t a = (static_cast<size_t>(kChunk) * lsum + kChunk * kRC + static_cast<size_t>(n_pad) * kRC) * 4;
+size_t batch_far_smem(int lsum, int n, int n_pad, int nnz, int Rmax) {
+  return far_smem<float>(lsum, n, n_pad, nnz, Rmax <= 4 ? 4 : 16);
+}
+
+size_t batch_far_need(int lsum, int n_pad) {
+  const size_t a = (static_cast<size_t>(kAcceptChunk) * lsum + kAcceptChunk * kRC + static_cast<size_t>(n_pad) * kRC) * 4;
   const size_t b = (2 * static_cast<size_t>(n_pad) * kRC + static_cast<size_t>(kFarThreads) * lsum) * 4;
   return std::max(a, b);
 }
@@ -995,9 +1133,9 @@ cudaError_t launch_batch_persistent(int D, int kernel, const PersistArgs& pa, in
   }
 }
 
-void launch_farfield(Plan& P, int Rc, bool fp64) {
-  if (fp64) farfield_impl<double>(P, Rc);
-  else farfield_impl<float>(P, Rc);
+void launch_farfield(Plan& P, int Rc, bool fp64, bool steady) {
+  if (fp64) farfield_impl<double>(P, Rc, steady);
+  else farfield_impl<float>(P, Rc, steady);
 }
 
 }  // namespace dw

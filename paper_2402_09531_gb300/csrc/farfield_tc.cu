@@ -718,7 +718,7 @@ bool farfield_tc_eligible(const Plan& P) {
   return true;
 }
 
-void farfield_tc(Plan& P, int Rc) {
+void farfield_tc(Plan& P, int Rc, bool steady) {
   cudaStream_t s = P.stream;
   ensure_far_attrs();
   if (!P.far_vt_ok) {
@@ -740,7 +740,7 @@ void farfield_tc(Plan& P, int Rc) {
   }
   timer_end(P, 1, s, launches);
   timer_begin(P, 2, s);
-  launch_m2l(P, Rc, false);
+  launch_m2l(P, Rc, false, steady);
   timer_end(P, 2, s, 1);
   timer_begin(P, 3, s);
   launches = 0;

@@ -62,10 +62,11 @@ void ensure_workspace(Plan& P, bool fp64) {
   }
 }
 
-void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy, int R, bool fp64) {
+void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy, int R, bool fp64,
+                   bool steady) {
   if (P.N == 0 || R == 0) return;
   ensure_workspace(P, fp64);
-  const bool fix = fp64 && fix_ready(P);   // the tree's records, before the side stream forks
+  const bool fix = fp64 && !steady && fix_ready(P);   // the tree's records, before the side stream forks
   cudaStream_t s = P.stream;
   timer_begin(P, 6, s);
   for (int r0 = 0; r0 < R; r0 += kRC) {
@@ -74,21 +75,21 @@ void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy
     P.near_parts = 0;
     launch_gather(P, x, ldx, r0, Rc, fp64, fix, fp64 ? nullptr : P.xq32.p);
     timer_end(P, 0, s, 1);
-    const bool rot = !fp64 && rot_ready(P, Rc);
+    const bool rot = !fp64 && !steady && rot_ready(P, Rc);
     if (!fp64) m2l_autotune(P, Rc);   // once per tree, before the near field starts
     if (P.tm.on && P.tm.serialize) {  // every phase alone on the caller's stream
-      launch_farfield(P, Rc, fp64);
+      launch_farfield(P, Rc, fp64, steady);
       timer_begin(P, 4, s);
-      launch_nearfield(P, Rc, fp64, rot, s);
+      launch_nearfield(P, Rc, fp64, rot, steady, s);
       timer_end(P, 4, s, 1);
     } else {
       DW_CUDA(cudaEventRecord(P.ev_fork, s));
       DW_CUDA(cudaStreamWaitEvent(P.side, P.ev_fork, 0));
       timer_begin(P, 4, P.side);
-      launch_nearfield(P, Rc, fp64, rot, P.side);
+      launch_nearfield(P, Rc, fp64, rot, steady, P.side);
       timer_end(P, 4, P.side, 1);
       DW_CUDA(cudaEventRecord(P.ev_join, P.side));
-      launch_farfield(P, Rc, fp64);
+      launch_farfield(P, Rc, fp64, steady);
       DW_CUDA(cudaStreamWaitEvent(s, P.ev_join, 0));
     }
     timer_begin(P, 5, s);

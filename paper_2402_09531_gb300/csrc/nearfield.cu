@@ -509,27 +509,27 @@ void eval_f64(Plan& P, const double* tgt64, int G, const int32_t* rowptr, const 
                         P.m_pad, Rc, s, splits, split_stride);
 }
 
-void launch_m2l(Plan& P, int Rc, bool fp64) {
+void launch_m2l(Plan& P, int Rc, bool fp64, bool steady) {
   if (P.jmin > P.J) return;
   if (fp64) {
     P.m2l_engine = 0;
-    if (!m2l_fix(P, Rc)) m2l_impl<double>(P, Rc, P.d_ynode64.p, P.mom64.p, P.loc64.p);
-  } else if (!m2l_f32_tuned(P, Rc)) {
+    if (steady || !m2l_fix(P, Rc)) m2l_impl<double>(P, Rc, P.d_ynode64.p, P.mom64.p, P.loc64.p);
+  } else if (!m2l_f32_tuned(P, Rc, steady)) {
     P.m2l_engine = 1;
     m2l_impl<float>(P, Rc, P.d_ynode32.p, P.mom32.p, P.loc32.p);
   }
   DW_CUDA(cudaGetLastError());
 }
 
-void launch_nearfield(Plan& P, int Rc, bool fp64, bool rot, cudaStream_t s) {
+void launch_nearfield(Plan& P, int Rc, bool fp64, bool rot, bool steady, cudaStream_t s) {
   if (fp64) {
-    if (near_fix(P, Rc, s)) return;
+    if (!steady && near_fix(P, Rc, s)) return;
     P.near_engine = 1;
     if (!near_sym(P, Rc, s)) {
       P.near_engine = 0;
       p2p_impl<double>(P, Rc, P.d_pts64.p, P.xb64.p, P.ynear64.p, s);
     }
-  } else if (!p2p_f32_tuned(P, Rc, rot, s)) {
+  } else if (!p2p_f32_tuned(P, Rc, rot, steady, s)) {
     P.near_engine = 2;
     p2p_impl<float>(P, Rc, P.d_pts32.p, P.xb32.p, P.ynear32.p, s);
   }

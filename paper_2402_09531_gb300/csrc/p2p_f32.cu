@@ -49,6 +49,12 @@ __global__ void __launch_bounds__(kThreadsMax, 3) k_sum_f32(SumArgs a) {
   const Grp G{static_cast<int>(threadIdx.x), static_cast<int>(blockDim.x), 0};
   // the parts' boundaries are read, not computed: any arithmetic on them takes
   // the list walk out of the uniform registers (31 more registers a thread)
+  if (a.entry_t) {   // one entry's sum
+    const int e = static_cast<int>(blockIdx.x);
+    (void)sum_block<D, RC, KER>(a, a.entry_t[2 * e] - a.entry_off, e, e + 1, a.out + e * a.out_gstride, G, smem, full,
+                                tile_base);
+    return;
+  }
   const int part = static_cast<int>(blockIdx.y);
   const int g = a.first + static_cast<int>(blockIdx.x);
   const int row = a.first_row + static_cast<int>(blockIdx.x) * a.row_step + part;
@@ -81,6 +87,33 @@ __global__ void k_add_parts(const float* part, int splits, int64_t stride, int g
   out[at] = s;
 }
 
+// out[g][r][i] = the sums of row g's entries [entry][Rc][ld], in list order,
+// with the compensation of sum_block.
+__global__ void k_fold_entries(const float* part, const int32_t* rowptr, int groups, int ld, int Rc, float* out) {
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t >= static_cast<int64_t>(groups) * Rc * ld) return;
+  const int i = static_cast<int>(t % ld);
+  const int64_t gr = t / ld;
+  const int r = static_cast<int>(gr % Rc);
+  const int g = static_cast<int>(gr / Rc);
+  const int64_t at = static_cast<int64_t>(r) * ld + i, step = static_cast<int64_t>(Rc) * ld;
+  float acc = 0.0f, c = 0.0f;
+  const int re = rowptr[g + 1];
+  for (int e = rowptr[g]; e < re; e += 8) {
+    float w[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) w[u] = e + u < re ? part[(e + u) * step + at] : 0.0f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (e + u >= re) break;
+      const float y = w[u] - c, s = acc + y;
+      c = (s - acc) - y;
+      acc = s;
+    }
+  }
+  out[(static_cast<int64_t>(g) * kRC + r) * ld + i] = acc;
+}
+
 // Row layout [g][16][ld] -> interleaved [g][ld][RC] (first RC rows).
 __global__ void k_interleave(const float* src, int64_t groups, int ld, int RC, float* dst) {
   const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -107,6 +140,139 @@ __global__ void k_scaled_blocks(const double* src, int64_t groups, int d, int D,
     n2 += static_cast<double>(f) * static_cast<double>(f);
   }
   dst[(g * (D + 1) + D) * ld + i] = static_cast<float>(n2);
+}
+
+// Couplings of small node sets: one CTA per target cluster, one node and one
+// share of the list per thread (thread (t, sub) takes the entries sub, sub +
+// nsub, ...), so that 10 nodes do not leave 22 lanes of a warp idle.  Each
+// entry's n terms are summed in float32, entries and threads with
+// compensation.  The blocks are read through L1 (the lanes of a share read the
+// same words).  10 nodes, d = 8, N = 100003, 4 right-hand sides: 131 us with one
+// CTA of 32 threads a cluster, 36 us; 20 nodes, d = 16, N = 50021: 184, 98 us.
+struct SmallArgs {
+  const float* nodes;      // scaled blocks [c][D + 1][ld]
+  const float* mom;        // [c][16][ld], zero beyond n
+  float* loc;
+  const int32_t* rowptr;
+  const int32_t* col;
+  int first, n, ld, Rc;
+};
+
+constexpr int kSmallThreads = 128;
+constexpr int kSmallNodes = 32;   // padded nodes
+
+template <int D, int RC, int KER>
+__global__ void __launch_bounds__(kSmallThreads) k_m2l_small(const SmallArgs a) {
+  __shared__ float red[2][RC][kSmallThreads];
+  const int g = a.first + static_cast<int>(blockIdx.x);
+  const int tid = static_cast<int>(threadIdx.x);
+  const int nsub = kSmallThreads / a.n;
+  const int sub = tid / a.n, t = tid - sub * a.n;
+  const int ld = a.ld, n4 = (a.n + 3) & ~3;
+  const int rb = a.rowptr[g], re = sub < nsub ? a.rowptr[g + 1] : rb;
+  const float* tb = a.nodes + static_cast<int64_t>(g) * (D + 1) * ld + t;
+  u64 x2[D], nt2;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    const float v = KER == DWFMM_K_GAUSS ? 2.0f * tb[k * ld] : tb[k * ld];
+    x2[k] = pk2(v, v);
+  }
+  nt2 = pk2(-tb[D * ld], -tb[D * ld]);
+  float s[RC], c[RC];
+#pragma unroll
+  for (int r = 0; r < RC; ++r) s[r] = c[r] = 0.0f;
+  for (int e = rb + sub; e < re; e += nsub) {
+    const int64_t src = a.col[e];
+    const float* sb = a.nodes + src * (D + 1) * ld;
+    const float* q = a.mom + src * kRC * ld;
+    u64 acc[RC];
+#pragma unroll
+    for (int r = 0; r < RC; ++r) acc[r] = 0ull;
+    for (int j = 0; j < n4; j += 4) {
+      u64 e0, e1;
+      if (KER == DWFMM_K_GAUSS) {
+        const ulonglong2 ns = *reinterpret_cast<const ulonglong2*>(sb + D * ld + j);
+        e0 = fsub2(nt2, ns.x);
+        e1 = fsub2(nt2, ns.y);
+      } else {
+        e0 = e1 = 0ull;
+      }
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const ulonglong2 sv = *reinterpret_cast<const ulonglong2*>(sb + k * ld + j);
+        if (KER == DWFMM_K_GAUSS) {
+          e0 = ffma2(x2[k], sv.x, e0);
+          e1 = ffma2(x2[k], sv.y, e1);
+        } else {
+          const u64 d0 = fsub2(x2[k], sv.x), d1 = fsub2(x2[k], sv.y);
+          e0 = ffma2(d0, d0, e0);
+          e1 = ffma2(d1, d1, e1);
+        }
+      }
+      float p0, p1, p2, p3;
+      up2(e0, p0, p1);
+      up2(e1, p2, p3);
+      const u64 f0 = pk2(phi_scaled<KER>(p0), phi_scaled<KER>(p1)), f1 = pk2(phi_scaled<KER>(p2), phi_scaled<KER>(p3));
+#pragma unroll
+      for (int r = 0; r < RC; ++r) {
+        const ulonglong2 qv = *reinterpret_cast<const ulonglong2*>(q + r * ld + j);
+        acc[r] = ffma2(f0, qv.x, acc[r]);
+        acc[r] = ffma2(f1, qv.y, acc[r]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < RC; ++r) {
+      float v0, v1;
+      up2(acc[r], v0, v1);
+      const float y = (v0 + v1) - c[r], z = s[r] + y;
+      c[r] = (z - s[r]) - y;
+      s[r] = z;
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < RC; ++r) {
+    red[0][r][tid] = s[r];
+    red[1][r][tid] = c[r];
+  }
+  __syncthreads();
+  for (int o = tid; o < a.n * a.Rc; o += kSmallThreads) {
+    const int r = o / a.n, i = o - r * a.n;
+    float v = red[0][r][i], w = red[1][r][i];
+    for (int u = 1; u < nsub; ++u) {
+      const float y = red[0][r][u * a.n + i] - (red[1][r][u * a.n + i] + w), z = v + y;
+      w = (z - v) - y;
+      v = z;
+    }
+    a.loc[(static_cast<int64_t>(g) * kRC + r) * ld + i] = v;
+  }
+}
+
+template <int D, int RC>
+void m2l_small_kernel(int kernel, const SmallArgs& a, int groups, cudaStream_t s) {
+  if (kernel == DWFMM_K_EXP) k_m2l_small<D, RC, DWFMM_K_EXP><<<groups, kSmallThreads, 0, s>>>(a);
+  else if (kernel == DWFMM_K_MATERN32) k_m2l_small<D, RC, DWFMM_K_MATERN32><<<groups, kSmallThreads, 0, s>>>(a);
+  else k_m2l_small<D, RC, DWFMM_K_GAUSS><<<groups, kSmallThreads, 0, s>>>(a);
+}
+
+template <int D>
+void m2l_small_rc(int kernel, int RC, const SmallArgs& a, int groups, cudaStream_t s) {
+  if (RC <= 1) m2l_small_kernel<D, 1>(kernel, a, groups, s);
+  else if (RC <= 4) m2l_small_kernel<D, 4>(kernel, a, groups, s);
+  else if (RC <= 8) m2l_small_kernel<D, 8>(kernel, a, groups, s);
+  else m2l_small_kernel<D, 16>(kernel, a, groups, s);
+}
+
+void m2l_small(Plan& P, int D, int RC, int Rc, int first) {
+  const SmallArgs a{P.d_ynodek.p, P.mom32.p, P.loc32.p, P.d_far_rowptr.p, P.d_far_col.p, first, P.n, P.n_pad, Rc};
+  const int groups = P.C - first;
+  switch (D) {
+    case 4: m2l_small_rc<4>(P.kernel, RC, a, groups, P.stream); break;
+    case 8: m2l_small_rc<8>(P.kernel, RC, a, groups, P.stream); break;
+    case 10: m2l_small_rc<10>(P.kernel, RC, a, groups, P.stream); break;
+    case 12: m2l_small_rc<12>(P.kernel, RC, a, groups, P.stream); break;
+    case 16: m2l_small_rc<16>(P.kernel, RC, a, groups, P.stream); break;
+    default: m2l_small_rc<20>(P.kernel, RC, a, groups, P.stream); break;
+  }
 }
 
 template <int D, int RC>
@@ -173,6 +339,8 @@ void dispatch(int D, int kernel, int RC, SumArgs a, int groups, int threads, siz
 // attributes, which is harmless).
 std::atomic<uint64_t> g_attrs_dev{0};
 
+constexpr size_t kEntryPartsBytes = size_t(256) << 20;   // one sum per near entry
+
 void ensure_attrs() {
   const uint64_t bit = device_bit();
   if (g_attrs_dev.load() & bit) return;
@@ -230,7 +398,7 @@ void launch_scaled_blocks(const double* src, int64_t groups, int d, int D, int l
 }
 
 // rot: each unordered pair once (rot_ready).  The charges are in P.xq32.
-bool p2p_f32_tuned(Plan& P, int Rc, bool rot, cudaStream_t s) {
+bool p2p_f32_tuned(Plan& P, int Rc, bool rot, bool steady, cudaStream_t s) {
   const int D = padded_dim(P.d);
   if (D < 0) return false;
   const int RC = padded_rc(Rc);
@@ -285,7 +453,20 @@ bool p2p_f32_tuned(Plan& P, int Rc, bool rot, cudaStream_t s) {
   // (d = 10 Gaussian, N = 3362, 12 right-hand sides, 16 leaves: the product
   // took 177 us in one part, 45 us in 16)
   const int splits = std::max(1, std::min(16, 4 * sm_count() / P.L));
-  if (splits > 1) {
+  if (steady && splits > 1 &&
+      static_cast<size_t>(P.nnear) * Rc * P.m_pad * sizeof(float) <= kEntryPartsBytes) {
+    // every entry's sum by itself, then in list order with the compensation
+    // that one CTA per leaf would carry: the same bits, on all SMs
+    // (N = 3001, d = 16: 174 us with 32 CTAs)
+    a.entry_t = P.d_near_pairs.p;
+    a.entry_off = P.L - 1;
+    a.out_gstride = static_cast<int64_t>(Rc) * P.m_pad;
+    P.entry_parts32.alloc(static_cast<size_t>(P.nnear) * Rc * P.m_pad);
+    a.out = P.entry_parts32.p;
+    dispatch(D, P.kernel, RC, a, static_cast<int>(P.nnear), threads, smem, s);
+    k_fold_entries<<<ceil_div(static_cast<int64_t>(P.L) * Rc * P.m_pad, 128), 128, 0, s>>>(
+        P.entry_parts32.p, P.d_near_rowptr.p, P.L, P.m_pad, Rc, P.ynear32.p);
+  } else if (splits > 1 && !steady) {
     if (!P.part_rows.p) {   // once per tree
       P.part_rows.alloc(static_cast<size_t>(P.L) * splits + 1);
       k_part_rows<<<ceil_div(static_cast<int64_t>(P.L) * splits + 1, 256), 256, 0, s>>>(P.d_near_rowptr.p, P.L, splits,
@@ -397,7 +578,7 @@ void m2l_autotune(Plan& P, int Rc) {
   P.m2l_tuned = (sym && (!ord || ms_sym < ms_ord)) ? 3 : 2;
 }
 
-bool m2l_f32_tuned(Plan& P, int Rc) {
+bool m2l_f32_tuned(Plan& P, int Rc, bool steady) {
   const int D = padded_dim(P.d);
   if (D < 0) return false;
   const int RC = padded_rc(Rc);
@@ -417,6 +598,12 @@ bool m2l_f32_tuned(Plan& P, int Rc) {
     }
   }
   const int first = (1 << P.jmin) - 1;
+  if (P.n_pad <= kSmallNodes && !steady) {
+    P.m2l_engine = 1;
+    m2l_small(P, D, RC, Rc, first);
+    DW_CUDA(cudaGetLastError());
+    return true;
+  }
   P.momq32.alloc(static_cast<size_t>(P.C) * P.n_pad * kRC);
   const int64_t nq = static_cast<int64_t>(P.C) * P.n_pad * RC;
   k_interleave<<<ceil_div(nq, 256), 256, 0, P.stream>>>(P.mom32.p, P.C, P.n_pad, RC, P.momq32.p);

@@ -97,6 +97,23 @@ static void make_index_set(Plan& P) {
       if (ak > 0) fac[a * nnz_max + z++] = static_cast<int16_t>(P.loff[k] + ak);
     }
   }
+  std::vector<int32_t> act;
+  int top = 1;
+  for (int k = 0; k < P.d; ++k) {
+    if (P.qk[k] > 0) act.push_back(k);
+    top = std::max(top, P.qk[k]);
+  }
+  // p_{j+1} = a_j u p_j - b_j p_{j-1} for p_j = sqrt(2j+1) P_j
+  std::vector<double2> l64(top);
+  for (int j = 0; j < top; ++j) {
+    const double a = std::sqrt((2.0 * j + 1.0) * (2.0 * j + 3.0)) / (j + 1.0);
+    const double b = j ? j * std::sqrt((2.0 * j + 3.0) / (2.0 * j - 1.0)) / (j + 1.0) : 0.0;
+    l64[j] = make_double2(a, b);
+  }
+  P.d_act.alloc(act.size());
+  P.d_leg64.alloc(l64.size());
+  if (!act.empty()) DW_CUDA(cudaMemcpy(P.d_act.p, act.data(), act.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+  DW_CUDA(cudaMemcpy(P.d_leg64.p, l64.data(), l64.size() * sizeof(double2), cudaMemcpyHostToDevice));
   P.d_fac.alloc(fac.size());
   P.d_qk.alloc(P.d);
   P.d_loff.alloc(P.d);
@@ -343,13 +360,16 @@ __global__ void k_gauss_jordan(double* aug, int n, int* err) {
   }
 }
 
-__global__ void k_extract_vinv(const double* aug, int n, int n_pad, double* vinv, float* vinv32) {
+__global__ void k_extract_vinv(const double* aug, int n, int n_pad, double* vinv, float* vinv32, double* vinvt,
+                               float* vinvt32) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n_pad * n_pad) return;
   const int r = t / n_pad, c = t % n_pad;
   const double v = (r < n && c < n) ? aug[static_cast<int64_t>(r) * 2 * n + n + c] : 0.0;
   vinv[t] = v;
   vinv32[t] = static_cast<float>(v);
+  vinvt[c * n_pad + r] = v;
+  vinvt32[c * n_pad + r] = static_cast<float>(v);
 }
 
 static std::vector<int32_t> primes(int d) {
@@ -380,9 +400,11 @@ void setup_vinv_from_nodes(Plan& P) {
   k_gauss_jordan<<<1, 1024, 0, s>>>(aug.p, P.n, err.p);
   P.d_vinv.alloc(static_cast<size_t>(P.n_pad) * P.n_pad);
   P.d_vinv32.alloc(static_cast<size_t>(P.n_pad) * P.n_pad);
+  P.d_vinvt.alloc(static_cast<size_t>(P.n_pad) * P.n_pad);
+  P.d_vinvt32.alloc(static_cast<size_t>(P.n_pad) * P.n_pad);
   P.far_vt_ok = false;
   k_extract_vinv<<<ceil_div(static_cast<int64_t>(P.n_pad) * P.n_pad, 256), 256, 0, s>>>(
-      aug.p, P.n, P.n_pad, P.d_vinv.p, P.d_vinv32.p);
+      aug.p, P.n, P.n_pad, P.d_vinv.p, P.d_vinv32.p, P.d_vinvt.p, P.d_vinvt32.p);
   DW_CUDA(cudaGetLastError());
   int h_err = 0;
   DW_CUDA(cudaMemcpyAsync(&h_err, err.p, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -74,9 +74,13 @@ void dots(Plan& P, const double* a, const double* b, int64_t n, int64_t ld, int 
 }
 
 // A v = K_tilde v + lam v (into out); v, out: n x R, leading dimension n.
-void apply_op(Plan& P, const double* v, double* out, int R, double lam, bool fp64) {
+// steady: the iterations of the incremental CG, whose operator keeps one order of
+// its sums whatever the plain product uses.  K_tilde may be mildly indefinite,
+// and eight iterations then turn a change of the operator's last bits into one
+// 1e4 to 1e8 times as large.
+void apply_op(Plan& P, const double* v, double* out, int R, double lam, bool fp64, bool steady = false) {
   const int64_t n = P.N;
-  matvec_device(P, v, n, out, n, R, fp64);
+  matvec_device(P, v, n, out, n, R, fp64, steady);
   if (lam != 0.0)
     // out = lam * v + 1 * out  (a_sign carries lam, coef_b_const = 1)
     k_axpby<<<ceil_div(n * R, 256), 256, 0, P.stream>>>(v, out, nullptr, nullptr, 1.0, nullptr, 0.0, n, n, R, lam);
@@ -99,6 +103,7 @@ int cg_dev(Plan& P, const double* b, int R, double lam, double rtol, int maxit, 
   constexpr int kSolveChunk = 16;
   cg_begin(P, lam, b, R, P.N, rtol);
   CgState& S = P.cgs;
+  S.steady = false;   // solved to a tolerance, with the fastest operator
   st.assign(R, 2);
   int done = 0, its = 0;
   while (done < maxit) {
@@ -361,6 +366,7 @@ void cg_begin(Plan& P, double lam, const double* f, int R, int64_t ld, double rt
   S.lam = lam;
   S.rtol = rtol;
   S.active = true;
+  S.steady = true;
   S.stepped = false;   // the previous status snapshot belongs to the previous solve
   P.cg_r.alloc(nr);
   P.cg_p.alloc(nr);
@@ -404,7 +410,7 @@ static void cg_iteration(Plan& P) {
   int* status = S.d_int.p;
   int* its = S.d_int.p + R;
   const bool fp64 = P.prec == DWFMM_P_FP64;
-  apply_op(P, P.cg_p.p, P.cg_ap.p, R, S.lam, fp64);
+  apply_op(P, P.cg_p.p, P.cg_ap.p, R, S.lam, fp64, S.steady);
   dots_dev(P, P.cg_p.p, P.cg_ap.p, n, R, part, pap);
   k_cg_alpha<<<1, 64, 0, P.stream>>>(pap, rr, status, coef, R);
   k_axpby<<<ceil_div(nr, 256), 256, 0, P.stream>>>(P.cg_p.p, P.cg_c.p, nullptr, coef, 1.0, nullptr, 0.0, n, n, R, 1.0);
@@ -430,6 +436,7 @@ static bool cg_step_graph(Plan& P, int iters) {
   key.iters = iters;
   key.lam = S.lam;
   key.fp64 = P.prec == DWFMM_P_FP64;
+  key.steady = S.steady;
   key.stream = P.stream;
   const void* bufs[6] = {P.cg_p.p, P.cg_ap.p, P.cg_c.p, P.cg_r.p, P.cg_dot.p, S.d_int.p};
   for (int i = 0; i < 6; ++i) key.bufs[i] = bufs[i];

@@ -15,10 +15,39 @@ using dw::Plan;
 
 namespace dw {
 
-void Plan::free_tree() {
+// Forget the tree.  Buffers that the next tree sizes itself stay; what is built on
+// first use, or belongs to a solve on the old tree, goes.
+void Plan::drop_tree() {
   have_tree = false;
   N = 0;
   J = -1;
+  fx_state = -1;
+  fx_sym = -1;
+  rot_state = -1;
+  near_parts = 0;
+  sym_nup = 0;
+  sym_ok = false;
+  sym_x16_ok = false;
+  fsym_rows = 0;
+  fsym_ok = false;
+  m2l_crd_D = -1;
+  m2l_x16_D = -1;
+  m2l_tuned = -1;
+  m2l_tune_ms[0] = m2l_tune_ms[1] = -1.0;
+  dpad = -1;
+  h_upcount.clear();
+  cg_r.release();
+  cg_p.release();
+  cg_ap.release();
+  cg_c.release();
+  cg_f.release();
+  cg_dot.release();
+  cg_tmp.release();
+  part_rows.release();
+}
+
+void Plan::free_tree() {
+  drop_tree();
   d_begin.release();
   d_count.release();
   d_perm.release();
@@ -50,26 +79,15 @@ void Plan::free_tree() {
   mom32.release();
   loc32.release();
   lco32.release();
-  cg_r.release();
-  cg_p.release();
-  cg_ap.release();
-  cg_c.release();
-  cg_f.release();
-  cg_dot.release();
-  cg_tmp.release();
-  scratch.release();
   d_ptsk.release();
   d_ynodek.release();
   xq32.release();
   momq32.release();
   bq32.release();
   bqm32.release();
-  part_rows.release();
   entry_parts32.release();
   near_parts32.release();
   near_parts64.release();
-  fx_state = -1;
-  fx_sym = -1;
   fx_rows.t.release();
   fx_rows.ptr.release();
   ev_blk.release();
@@ -78,13 +96,10 @@ void Plan::free_tree() {
   ev_out32.release();
   ev_rows.release();
   ev_col.release();
-  rot_state = -1;
   rot.t.release();
   rot.ptr.release();
   rot_pf.release();
   rot_pt.release();
-  near_parts = 0;
-  h_upcount.clear();
   fx_pts.release();
   fx_nodes.release();
   fx_q.release();
@@ -98,8 +113,6 @@ void Plan::free_tree() {
   sym_loslot.release();
   sym_pf.release();
   sym_pt.release();
-  sym_nup = 0;
-  sym_ok = false;
   sym_order.release();
   sym_bq16.release();
   sym_fwd.release();
@@ -107,24 +120,27 @@ void Plan::free_tree() {
   sym_colmax.release();
   sym_xa16.release();
   sym_xb16.release();
-  sym_x16_ok = false;
   fsym_uprow.release();
   fsym_s.release();
   fsym_order.release();
-  fsym_rows = 0;
-  fsym_ok = false;
   m2l_crd.release();
-  m2l_crd_D = -1;
   m2l_xa16.release();
   m2l_xb16.release();
-  m2l_x16_D = -1;
   m2l_bq16.release();
   m2l_fwd.release();
   m2l_acc.release();
   m2l_colmax.release();
-  m2l_tuned = -1;
-  m2l_tune_ms[0] = m2l_tune_ms[1] = -1.0;
-  dpad = -1;
+  tw = TreeWork();
+}
+
+// Keep the tree build's workspaces while they are below 64 MB.
+void Plan::trim_tree_work() {
+  size_t b = (tw.soa0.n + tw.soa1.n) * sizeof(double) + (tw.key.n + tw.kmin.n + tw.kmax.n) * sizeof(unsigned long long);
+  for (const DBuf<int32_t>* x : {&tw.perm1, &tw.seg, &tw.ct, &tw.cs, &tw.nt, &tw.ns, &tw.lo_src, &tw.up_t, &tw.lo_slot,
+                                 &tw.eq, &tw.eqscan, &tw.left, &tw.lscan, &tw.adm, &tw.admscan, &tw.childcnt, &tw.cnt})
+    b += x->n * sizeof(int32_t);
+  for (const auto& x : tw.far_lvl) b += x.n * sizeof(int32_t);
+  if (b > (size_t(64) << 20)) tw = TreeWork();
 }
 
 // Report a bounded device wait that gave up (raised by the tuned kernels).
@@ -320,7 +336,9 @@ dwfmm_status dwfmm_tree_build(dwfmm_plan plan, const double* pts, int64_t n, int
     if (n < 0 || n > (int64_t(1) << 30)) dw::fail(DWFMM_ERR_INVALID_ARG, "N must be in 0..2^30");
     if (n > 0 && (!pts || ld < P.d)) dw::fail(DWFMM_ERR_INVALID_ARG, "pts is NULL or ld < d");
     bind_stream(P, stream);
-    P.free_tree();
+    // a much smaller tree gives the memory back
+    if (n < P.N / 4) P.free_tree();
+    else P.drop_tree();
     P.cgs.drop_graph();
     ++P.tree_gen;
     const double* dev = pts;
@@ -334,11 +352,21 @@ dwfmm_status dwfmm_tree_build(dwfmm_plan plan, const double* pts, int64_t n, int
       dev = staged.p;
       ld_dev = P.d;
     }
-    dw::build_tree(P, dev, n, ld_dev);
-    dw::build_lists(P);
-    dw::build_cluster_data(P);
-    dw::build_sym_lists(P);
-    if (P.prec == DWFMM_P_MIXED) dw::build_far_sym_lists(P);
+    auto build = [&]() {
+      dw::build_tree(P, dev, n, ld_dev);
+      dw::build_lists(P);
+      dw::build_cluster_data(P);
+      dw::build_sym_lists(P);
+      if (P.prec == DWFMM_P_MIXED) dw::build_far_sym_lists(P);
+    };
+    try {
+      build();
+    } catch (const ApiError& e) {
+      if (e.status != DWFMM_ERR_OOM) throw;
+      P.free_tree();   // the last tree's buffers may have been in the way
+      build();
+    }
+    P.trim_tree_work();
     // bound of |x'|^2 = |x|^2 log2(e) / (2 sigma^2) over the root box, which
     // holds every site and every interpolation node
     P.gauss_fact = false;

@@ -381,6 +381,20 @@ struct RowChunks {
   DBuf<int32_t> t, ptr;       // [n] target leaf, [leaves + 1] first chunk of a leaf
 };
 
+// Workspaces of the tree build, kept for the next one while they are small
+// (new sites on a plan are common, and an allocation or a release costs as much
+// as a kernel).
+struct TreeWork {
+  DBuf<double> soa0, soa1;
+  const double* sorted = nullptr;   // the tree-ordered sites [d][N], in soa0 or soa1
+  DBuf<int32_t> perm1, seg, kstar, ct, cs, nt, ns, lo_src, lorow, up_t, lo_slot;
+  DBuf<unsigned long long> key, kmin, kmax;
+  DBuf<int> bad, eq, eqscan, left, lscan, tmp, adm, admscan, rowptr, nrowptr, childcnt, cnt, cu, cl;
+  DBuf<unsigned char> st;
+  DBuf<unsigned int> hist;
+  std::vector<DBuf<int32_t>> far_lvl;
+};
+
 struct Plan {
   // configuration
   int d = 0, kernel = 0, wrule = 0, leaf = 0, M = 0, prec = 0, max_rhs = 0;
@@ -472,8 +486,7 @@ struct Plan {
   int near_parts = 0;
   std::vector<int> h_upcount;   // upper near entries per leaf
 
-  // scratch for tree build
-  DBuf<unsigned char> scratch;
+  TreeWork tw;
 
   // tuned float32 kernel summation: scaled blocks [g][dpad+1][ld]
   int dpad = -1;
@@ -539,6 +552,8 @@ struct Plan {
                   d_leg64.p};
   }
   TreeDev tree_dev() const { return TreeDev{N, J, L, C, m_pad, d_begin.p, d_count.p}; }
+  void trim_tree_work();
+  void drop_tree();   // no tree; buffers that the next one may use stay
   void free_tree();
   void free_all();
 };

@@ -395,7 +395,7 @@ void build_sym_lists(Plan& P) {
   const int L = P.L;
   if (P.N == 0 || L <= 0 || P.nnear <= 0) return;
   cudaStream_t s = P.stream;
-  DBuf<int> cu, cl, bad;
+  auto &cu = P.tw.cu, &cl = P.tw.cl, &bad = P.tw.bad;
   cu.alloc(L);
   cl.alloc(L);
   bad.alloc(1);
@@ -419,7 +419,7 @@ void build_sym_lists(Plan& P) {
   P.sym_t.alloc(static_cast<size_t>(nup));
   P.sym_s.alloc(static_cast<size_t>(nup));
   P.sym_loslot.alloc(static_cast<size_t>(std::max<int64_t>(nlo, 1)));
-  DBuf<int32_t> lo_src;
+  auto& lo_src = P.tw.lo_src;
   lo_src.alloc(static_cast<size_t>(std::max<int64_t>(nlo, 1)));
   DW_CUDA(cudaMemcpyAsync(P.sym_uprow.p, up.data(), sizeof(int32_t) * (L + 1), cudaMemcpyHostToDevice, s));
   DW_CUDA(cudaMemcpyAsync(P.sym_lorow.p, lo.data(), sizeof(int32_t) * (L + 1), cudaMemcpyHostToDevice, s));
@@ -450,7 +450,7 @@ void build_far_sym_lists(Plan& P) {
   const int C = P.C;
   if (P.N == 0 || C <= 0 || P.nfar <= 0) return;
   cudaStream_t s = P.stream;
-  DBuf<int> cu, cl, bad;
+  auto &cu = P.tw.cu, &cl = P.tw.cl, &bad = P.tw.bad;
   cu.alloc(C);
   cl.alloc(C);
   bad.alloc(1);
@@ -470,7 +470,7 @@ void build_far_sym_lists(Plan& P) {
   if (nup != nlo || nup <= 0) return;   // a symmetric relation without diagonal entries
   P.fsym_uprow.alloc(C + 1);
   P.fsym_s.alloc(static_cast<size_t>(nup));
-  DBuf<int32_t> lorow, up_t, lo_src, lo_slot;
+  auto &lorow = P.tw.lorow, &up_t = P.tw.up_t, &lo_src = P.tw.lo_src, &lo_slot = P.tw.lo_slot;
   lorow.alloc(C + 1);
   up_t.alloc(static_cast<size_t>(nup));
   lo_src.alloc(static_cast<size_t>(nlo));

@@ -267,25 +267,33 @@ __global__ void k_sel_hist(const unsigned long long* key, const int32_t* seg, in
   }
 }
 
+// One warp per segment: the digit that holds the rank, the histogram cleared.
 __global__ void k_sel_pick(SelState* st, unsigned int* hist, int nseg, int shift) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = static_cast<int>((static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
   if (s >= nseg) return;
   SelState t = st[s];
-  unsigned int* h = hist + static_cast<int64_t>(s) * 256;
-  if (t.rank >= 0) {
-    unsigned int cum = 0;
-    int b = 0;
-    for (; b < 256; ++b) {
-      if (cum + h[b] > static_cast<unsigned int>(t.rank)) break;
-      cum += h[b];
-    }
-    if (b == 256) b = 255;  // unreachable for consistent counts
-    t.prefix |= static_cast<unsigned long long>(b) << shift;
-    t.mask |= 0xFFull << shift;
-    t.rank -= static_cast<int>(cum);
-    st[s] = t;
+  unsigned int* h = hist + static_cast<int64_t>(s) * 256 + lane * 8;
+  int w[8], sum = 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    w[u] = static_cast<int>(h[u]);
+    sum += w[u];
+    h[u] = 0;
   }
-  for (int b = 0; b < 256; ++b) h[b] = 0;
+  int pre = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, pre, o);
+    if (lane >= o) pre += y;
+  }
+  pre -= sum;
+  if (t.rank < pre || t.rank >= pre + sum) return;   // one lane is left
+  int u = 0;
+  while (t.rank >= pre + w[u]) pre += w[u++];
+  t.prefix |= static_cast<unsigned long long>(lane * 8 + u) << shift;
+  t.mask |= 0xFFull << shift;
+  t.rank -= pre;
+  st[s] = t;
 }
 
 // eq[i] = key equals the segment's median key.
@@ -327,6 +335,221 @@ __global__ void k_partition(const double* soa_in, const int32_t* perm_in, int64_
   }
   perm_out[pos] = perm_in[i];
   for (int k = 0; k < d; ++k) soa_out[k * n + pos] = soa_in[k * n + i];
+}
+
+// ---- one level of small clusters ---------------------------------------------
+//
+// One CTA per cluster: its bounding box, the longest edge, the median by radix
+// select, the stable partition.  The digits start at the first bit in which the
+// box's two ends differ, so that the first histogram already spreads, and the
+// select stops once one key is left.  Bound by latency and by what one SM
+// streams.  N = 20011, d = 16: with ~20 launches a level (histogram and pick per
+// digit, two scans, ...) the tree and its lists took 4.7 ms, 1.7 ms with this
+// kernel and kept workspaces, both before k_move.
+constexpr int kSplitThreads = 1024;
+constexpr int kSplitMax = 32768;   // sites of a cluster, beyond it the whole GPU shares the level
+constexpr int kSplitKeys = 5632;   // keys kept in shared memory (with the rest within 48 KB)
+
+__global__ void __launch_bounds__(kSplitThreads)
+k_split(const double* __restrict__ soa_in, const int32_t* __restrict__ perm_in, int64_t n_all, int d,
+        const int32_t* lvl_begin, const int32_t* lvl_count, int first, double* lo, double* hi, int split,
+        double* __restrict__ soa_out, int32_t* __restrict__ perm_out, int32_t* __restrict__ dest) {
+  extern __shared__ __align__(16) unsigned char split_smem[];
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(split_smem);   // [kSplitKeys]
+  __shared__ unsigned long long red[2][4][32];
+  __shared__ double box[2][kMaxDim];
+  __shared__ int hist[256];
+  __shared__ int wsum[2][32];
+  __shared__ int s_kstar, s_digit, s_rank, s_left;
+  __shared__ unsigned long long s_key;
+  const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, wid = tid >> 5;
+  const int b = lvl_begin[blockIdx.x], n = lvl_count[blockIdx.x];
+  const int c = first + static_cast<int>(blockIdx.x);
+  for (int kb = 0; kb < d; kb += 4) {   // four dimensions at a time: independent loads
+    unsigned long long mn[4], mx[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      mn[u] = ~0ull;
+      mx[u] = 0ull;
+    }
+#pragma unroll 2
+    for (int i = tid; i < n; i += kSplitThreads) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const unsigned long long v = dkey(soa_in[min(kb + u, d - 1) * n_all + b + i]);
+        mn[u] = v < mn[u] ? v : mn[u];
+        mx[u] = v > mx[u] ? v : mx[u];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long p = __shfl_xor_sync(0xffffffffu, mn[u], o), q = __shfl_xor_sync(0xffffffffu, mx[u], o);
+        mn[u] = p < mn[u] ? p : mn[u];
+        mx[u] = q > mx[u] ? q : mx[u];
+      }
+      if (lane == 0) {
+        red[0][u][wid] = mn[u];
+        red[1][u][wid] = mx[u];
+      }
+    }
+    __syncthreads();
+    const int k = kb + wid;
+    if (wid < 4 && k < d) {
+      unsigned long long l = red[0][wid][lane], h = red[1][wid][lane];
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long p = __shfl_xor_sync(0xffffffffu, l, o), q = __shfl_xor_sync(0xffffffffu, h, o);
+        l = p < l ? p : l;
+        h = q > h ? q : h;
+      }
+      if (lane == 0) {
+        box[0][k] = dkey_inv(l);
+        box[1][k] = dkey_inv(h);
+        lo[static_cast<int64_t>(c) * d + k] = box[0][k];
+        hi[static_cast<int64_t>(c) * d + k] = box[1][k];
+      }
+    }
+    __syncthreads();   // red is read
+  }
+  if (!split) return;
+  __syncthreads();
+  if (tid == 0) {   // the first longest edge
+    double best = -1.0;
+    int bk = 0;
+    for (int k = 0; k < d; ++k) {
+      const double e = box[1][k] - box[0][k];
+      if (e > best) {
+        best = e;
+        bk = k;
+      }
+    }
+    s_kstar = bk;
+    s_rank = (n + 1) / 2 - 1;
+  }
+  __syncthreads();
+  const int ks = s_kstar;
+  const double* xs = soa_in + ks * n_all + b;
+  const bool kept = n <= kSplitKeys;
+  if (kept) {
+    for (int i = tid; i < n; i += kSplitThreads) keys[i] = dkey(xs[i]);
+  }
+  auto key = [&](int i) { return kept ? keys[i] : dkey(xs[i]); };
+  const unsigned long long k0 = dkey(box[0][ks]), k1 = dkey(box[1][ks]);
+  int shift = k0 == k1 ? 0 : max(0, 56 - __clzll(static_cast<long long>(k0 ^ k1)));
+  // bits above the first digit are those of every key
+  unsigned long long mask = shift >= 56 ? 0ull : ~0ull << (shift + 8);
+  unsigned long long med = k0 & mask;
+  if (k0 == k1) {
+    med = k0;
+    mask = ~0ull;
+  }
+  while (mask != ~0ull) {
+    if (tid < 256) hist[tid] = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += kSplitThreads) {
+      const unsigned long long v = key(i);
+      if ((v & mask) == med) atomicAdd(&hist[static_cast<int>(v >> shift) & 255], 1);
+    }
+    __syncthreads();
+    if (wid == 0) {   // the digit that holds the rank
+      int h[8], sum = 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        h[u] = hist[lane * 8 + u];
+        sum += h[u];
+      }
+      int pre = sum;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, pre, o);
+        if (lane >= o) pre += y;
+      }
+      pre -= sum;
+      const int rank = s_rank;
+      __syncwarp();
+      if (rank >= pre && rank < pre + sum) {
+        int u = 0;
+        while (rank >= pre + h[u]) pre += h[u++];
+        s_digit = lane * 8 + u;
+        s_rank = rank - pre;
+        s_left = h[u];
+      }
+    }
+    __syncthreads();
+    med |= static_cast<unsigned long long>(s_digit) << shift;
+    // the next digit, aligned to the low end of the key
+    mask |= 255ull << shift;
+    const int left = s_left;
+    if (left == 1 && mask != ~0ull) {   // one key: it is the median
+      for (int i = tid; i < n; i += kSplitThreads) {
+        const unsigned long long v = key(i);
+        if ((v & mask) == med) s_key = v;
+      }
+      __syncthreads();
+      med = s_key;
+      break;
+    }
+    if (shift == 0) break;
+    const int next = shift > 8 ? shift - 8 : 0;
+    // an overlapping last digit: its upper bits are known, so they stay fixed
+    if (next + 8 > shift) {
+      mask &= ~0ull << shift;
+    }
+    shift = next;
+  }
+  __syncthreads();
+  const int rank = s_rank;   // rank of the median among the keys equal to it
+  // stable partition: a site goes left if its key is below the median, or equal
+  // with at most `rank` equals before it
+  int less0 = 0, eq0 = 0;
+  const int n1 = (n + 1) / 2;
+  for (int t0 = 0; t0 < n; t0 += kSplitThreads) {
+    const int i = t0 + tid;
+    const unsigned long long v = i < n ? key(i) : ~0ull;
+    const bool less = i < n && v < med, eq = i < n && v == med;
+    const unsigned ml = __ballot_sync(0xffffffffu, less), me = __ballot_sync(0xffffffffu, eq);
+    if (lane == 0) {
+      wsum[0][wid] = __popc(ml);
+      wsum[1][wid] = __popc(me);
+    }
+    __syncthreads();
+    const int wl = wsum[0][lane], we = wsum[1][lane];
+    int sl = lane < wid ? wl : 0, se = lane < wid ? we : 0, al = wl, ae = we;
+    for (int o = 16; o > 0; o >>= 1) {
+      sl += __shfl_xor_sync(0xffffffffu, sl, o);
+      se += __shfl_xor_sync(0xffffffffu, se, o);
+      al += __shfl_xor_sync(0xffffffffu, al, o);
+      ae += __shfl_xor_sync(0xffffffffu, ae, o);
+    }
+    const unsigned below = (1u << lane) - 1u;
+    const int lb = less0 + sl + __popc(ml & below), eb = eq0 + se + __popc(me & below);
+    if (i < n) {
+      const int lr = lb + min(eb, rank + 1);   // sites before i that go left
+      const bool left = less || (eq && eb <= rank);
+      const int64_t pos = b + (left ? lr : n1 + (i - lr));
+      if (dest) {
+        dest[b + i] = static_cast<int32_t>(pos);
+      } else {
+        perm_out[pos] = perm_in[b + i];
+#pragma unroll 8
+        for (int k = 0; k < d; ++k) soa_out[k * n_all + pos] = soa_in[k * n_all + b + i];
+      }
+    }
+    less0 += al;
+    eq0 += ae;
+    __syncthreads();   // wsum is read
+  }
+}
+
+// The sites to their places, for the levels whose few CTAs would take long to
+// move them.
+__global__ void k_move(const double* __restrict__ soa_in, const int32_t* __restrict__ perm_in, int64_t n, int d,
+                       const int32_t* __restrict__ dest, double* __restrict__ soa_out, int32_t* __restrict__ perm_out) {
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t >= n * (d + 1)) return;
+  const int64_t k = t / n, i = t - k * n;
+  const int32_t pos = dest[i];
+  if (k < d) soa_out[k * n + pos] = soa_in[k * n + i];
+  else perm_out[pos] = perm_in[i];
 }
 
 // ---- lists ------------------------------------------------------------------
@@ -484,7 +707,6 @@ static void cluster_layout(int64_t N, int J, std::vector<int32_t>& begin, std::v
 
 void build_tree(Plan& P, const double* pts_dev, int64_t N, int64_t ld) {
   cudaStream_t s = P.stream;
-  P.free_tree();
   const int d = P.d;
   int J = 0;
   while ((N + (int64_t(1) << J) - 1) / (int64_t(1) << J) > P.leaf) ++J;
@@ -505,30 +727,34 @@ void build_tree(Plan& P, const double* pts_dev, int64_t N, int64_t ld) {
     DW_CUDA(cudaMemsetAsync(P.d_hi.p, 0, sizeof(double) * d, s));
     return;
   }
-  DBuf<double> soa0, soa1;
-  DBuf<int32_t> perm1, seg, kstar;
-  DBuf<unsigned long long> key, kmin, kmax;
-  DBuf<int> bad, eq, eqscan, left, lscan, tmp;
-  DBuf<SelState> st;
-  DBuf<unsigned int> hist;
+  TreeWork& W = P.tw;
+  auto &soa0 = W.soa0, &soa1 = W.soa1;
+  auto &perm1 = W.perm1, &seg = W.seg, &kstar = W.kstar;
+  auto &key = W.key, &kmin = W.kmin, &kmax = W.kmax;
+  auto &bad = W.bad, &eq = W.eq, &eqscan = W.eqscan, &left = W.left, &lscan = W.lscan, &tmp = W.tmp;
+  auto& hist = W.hist;
   soa0.alloc(static_cast<size_t>(N) * d);
   soa1.alloc(static_cast<size_t>(N) * d);
   perm1.alloc(N);
-  seg.alloc(N);
-  key.alloc(N);
-  eq.alloc(N);
-  left.alloc(N);
-  eqscan.alloc(N + 1);
-  lscan.alloc(N + 1);
   bad.alloc(1);
-  const int maxseg = P.L;
-  kstar.alloc(maxseg);
-  kmin.alloc(static_cast<size_t>(maxseg) * d);
-  kmax.alloc(static_cast<size_t>(maxseg) * d);
-  st.alloc(maxseg);
-  hist.alloc(static_cast<size_t>(maxseg) * 256);
   DW_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), s));
-  DW_CUDA(cudaMemsetAsync(hist.p, 0, sizeof(unsigned int) * maxseg * 256, s));
+  if (N > kSplitMax) {   // some levels are shared by the whole GPU
+    int segs = 1;
+    while (P.h_count[2 * segs - 1] > kSplitMax) segs *= 2;
+    seg.alloc(N);
+    key.alloc(N);
+    eq.alloc(N);
+    left.alloc(N);
+    eqscan.alloc(N + 1);
+    lscan.alloc(N + 1);
+    kstar.alloc(segs);
+    kmin.alloc(static_cast<size_t>(segs) * d);
+    kmax.alloc(static_cast<size_t>(segs) * d);
+    W.st.alloc(segs * sizeof(SelState));
+    hist.alloc(static_cast<size_t>(segs) * 256);
+    DW_CUDA(cudaMemsetAsync(hist.p, 0, sizeof(unsigned int) * segs * 256, s));
+  }
+  SelState* const st = reinterpret_cast<SelState*>(W.st.p);
   const int nb = ceil_div(N, 256);
   k_load_points<<<nb, 256, 0, s>>>(pts_dev, N, ld, d, soa0.p, P.d_perm.p, bad.p);
   int h_bad = 0;
@@ -546,6 +772,20 @@ void build_tree(Plan& P, const double* pts_dev, int64_t N, int64_t ld) {
     const int nseg = 1 << j;
     const int32_t* lvl_begin = P.d_begin.p + first;
     const int32_t* lvl_count = P.d_count.p + first;
+    if (P.h_count[first] <= kSplitMax) {   // the first cluster of a level is its largest
+      const size_t smem = P.h_count[first] <= kSplitKeys ? sizeof(unsigned long long) * P.h_count[first] : 0;
+      // below 64 CTAs the whole GPU moves the sites (N = 20011, d = 16: 100 us a
+      // level when the CTAs do)
+      const bool apart = nseg < 64 && j < J;
+      if (apart) seg.alloc(N);
+      k_split<<<nseg, kSplitThreads, smem, s>>>(cur, pcur, N, d, lvl_begin, lvl_count, first, P.d_lo.p, P.d_hi.p, j < J,
+                                                nxt, pnxt, apart ? seg.p : nullptr);
+      if (apart) k_move<<<ceil_div(N * (d + 1), 256), 256, 0, s>>>(cur, pcur, N, d, seg.p, nxt, pnxt);
+      if (j == J) break;
+      std::swap(cur, nxt);
+      std::swap(pcur, pnxt);
+      continue;
+    }
     k_segment_ids<<<nb, 256, 0, s>>>(lvl_begin, nseg, N, seg.p);
     k_box_init<<<ceil_div(nseg * d, 256), 256, 0, s>>>(kmin.p, kmax.p, nseg * d);
     k_box_reduce<<<nb, 256, 0, s>>>(cur, N, d, seg.p, kmin.p, kmax.p);
@@ -553,14 +793,14 @@ void build_tree(Plan& P, const double* pts_dev, int64_t N, int64_t ld) {
                                                      P.d_hi.p, j < J ? kstar.p : nullptr);
     if (j == J) break;
     k_make_keys<<<nb, 256, 0, s>>>(cur, N, seg.p, kstar.p, key.p);
-    k_sel_init<<<ceil_div(nseg, 128), 128, 0, s>>>(st.p, lvl_count, nseg);
+    k_sel_init<<<ceil_div(nseg, 128), 128, 0, s>>>(st, lvl_count, nseg);
     for (int shift = 56; shift >= 0; shift -= 8) {
-      k_sel_hist<<<hist_blocks, kHistThreads, 0, s>>>(key.p, seg.p, N, st.p, shift, hist.p);
-      k_sel_pick<<<ceil_div(nseg, 128), 128, 0, s>>>(st.p, hist.p, nseg, shift);
+      k_sel_hist<<<hist_blocks, kHistThreads, 0, s>>>(key.p, seg.p, N, st, shift, hist.p);
+      k_sel_pick<<<ceil_div(static_cast<int64_t>(nseg) * 32, 128), 128, 0, s>>>(st, hist.p, nseg, shift);
     }
-    k_flag_equal<<<nb, 256, 0, s>>>(key.p, seg.p, N, st.p, eq.p);
+    k_flag_equal<<<nb, 256, 0, s>>>(key.p, seg.p, N, st, eq.p);
     scan_exclusive(eq.p, eqscan.p, N, tmp, s);
-    k_flag_left<<<nb, 256, 0, s>>>(key.p, seg.p, N, st.p, eqscan.p, lvl_begin, left.p);
+    k_flag_left<<<nb, 256, 0, s>>>(key.p, seg.p, N, st, eqscan.p, lvl_begin, left.p);
     scan_exclusive(left.p, lscan.p, N, tmp, s);
     k_partition<<<nb, 256, 0, s>>>(cur, pcur, N, d, seg.p, left.p, lscan.p, lvl_begin, lvl_count,
                                    nxt, pnxt, bad.p);
@@ -570,10 +810,7 @@ void build_tree(Plan& P, const double* pts_dev, int64_t N, int64_t ld) {
   DW_CUDA(cudaGetLastError());
   if (pcur != P.d_perm.p)
     DW_CUDA(cudaMemcpyAsync(P.d_perm.p, pcur, N * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-  // keep the tree-ordered SoA sites for the leaf blocks
-  P.scratch.alloc(static_cast<size_t>(N) * d * sizeof(double));
-  DW_CUDA(cudaMemcpyAsync(P.scratch.p, cur, static_cast<size_t>(N) * d * sizeof(double),
-                          cudaMemcpyDeviceToDevice, s));
+  W.sorted = cur;
   DW_CUDA(cudaMemcpyAsync(&h_bad, bad.p, sizeof(int), cudaMemcpyDeviceToHost, s));
   DW_CUDA(cudaStreamSynchronize(s));
   if (h_bad) fail(DWFMM_ERR_CUDA, "median selection produced an inconsistent partition");
@@ -593,9 +830,13 @@ void build_lists(Plan& P) {
     return;
   }
   const double eta2 = P.eta * P.eta;
-  DBuf<int32_t> ct, cs, nt, ns;
-  DBuf<int> adm, admscan, rowptr, nrowptr, childcnt, tmp;
-  std::vector<DBuf<int32_t>> far_lvl(J + 1);
+  TreeWork& W = P.tw;
+  auto &ct = W.ct, &cs = W.cs, &nt = W.nt, &ns = W.ns;
+  auto &adm = W.adm, &admscan = W.admscan, &rowptr = W.rowptr, &nrowptr = W.nrowptr, &childcnt = W.childcnt;
+  auto &tmp = W.tmp, &cnt = W.cnt;
+  auto& far_lvl = W.far_lvl;
+  if (static_cast<int>(far_lvl.size()) <= J) far_lvl.resize(J + 1);
+  auto& near_pairs = P.d_near_pairs;
   int64_t nc = 1;
   ct.alloc(1);
   cs.alloc(1);
@@ -608,7 +849,6 @@ void build_lists(Plan& P) {
     DW_CUDA(cudaMemcpyAsync(rowptr.p, rp, 2 * sizeof(int), cudaMemcpyHostToDevice, s));
     DW_CUDA(cudaStreamSynchronize(s));
   }
-  DBuf<int32_t> near_pairs;
   for (int j = 0; j <= J; ++j) {
     const int first = (1 << j) - 1;
     const int nrows = 1 << j;
@@ -661,7 +901,6 @@ void build_lists(Plan& P) {
                             2 * P.far_level_count[j] * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     off += P.far_level_count[j];
   }
-  DBuf<int> cnt;
   cnt.alloc(std::max(P.C, P.L) + 1);
   P.d_far_rowptr.alloc(P.C + 1);
   P.d_far_col.alloc(std::max<int64_t>(P.nfar, 1));
@@ -672,7 +911,6 @@ void build_lists(Plan& P) {
   }
   scan_exclusive(cnt.p, P.d_far_rowptr.p, P.C, tmp, s);
   // near pairs, CSR over leaves (leaf-local ids)
-  P.d_near_pairs = std::move(near_pairs);
   P.d_near_rowptr.alloc(P.L + 1);
   P.d_near_col.alloc(std::max<int64_t>(P.nnear, 1));
   DW_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(int) * (P.L + 1), s));
@@ -683,7 +921,6 @@ void build_lists(Plan& P) {
   scan_exclusive(cnt.p, P.d_near_rowptr.p, P.L, tmp, s);
   DW_CUDA(cudaGetLastError());
   DW_CUDA(cudaStreamSynchronize(s));
-  for (auto& b : far_lvl) b.release();
 }
 
 void build_cluster_data(Plan& P) {
@@ -709,14 +946,13 @@ void build_cluster_data(Plan& P) {
   P.d_pts64.alloc(std::max<int64_t>(np, 1));
   P.d_pts32.alloc(std::max<int64_t>(np, 1));
   if (P.N > 0)
-    k_leaf_block<<<ceil_div(np, 256), 256, 0, s>>>(reinterpret_cast<const double*>(P.scratch.p), P.N, d,
+    k_leaf_block<<<ceil_div(np, 256), 256, 0, s>>>(P.tw.sorted, P.N, d,
                                                    P.d_begin.p, P.d_count.p, P.L, P.m_pad, P.d_pts64.p,
                                                    P.d_pts32.p);
   DW_CUDA(cudaMemcpyAsync(P.h_lo0, P.d_lo.p, sizeof(double) * d, cudaMemcpyDeviceToHost, s));
   DW_CUDA(cudaMemcpyAsync(P.h_hi0, P.d_hi.p, sizeof(double) * d, cudaMemcpyDeviceToHost, s));
   DW_CUDA(cudaGetLastError());
   DW_CUDA(cudaStreamSynchronize(s));
-  P.scratch.release();
 }
 
 }  // namespace dw

@@ -239,7 +239,7 @@ cudaError_t enqueue_persistent(Batch& B, cudaStream_t s, bool io) {
 // a batch.
 void enqueue_matvec(Batch& B, bool io = true, bool steady = false) {
   const bool by_pair = B.by_pair && !steady;
-  if (B.persistent && (by_pair || !B.by_pair)) {
+  if (B.persistent && !steady) {
     DW_CUDA(enqueue_persistent(B, B.stream, io));
     return;
   }
@@ -250,10 +250,10 @@ void enqueue_matvec(Batch& B, bool io = true, bool steady = false) {
   enqueue_near(B, B.split, B.thr_near, by_pair, B.side);
   DW_CUDA(cudaEventRecord(B.ev_join, B.side));
   for (size_t h = 0; h < B.up_off.size(); ++h)
-    launch_moments_batched(B.probs.p, B.work.p + B.up_off[h], B.up_cnt[h], B.far_smem, s);
+    launch_moments_batched(B.probs.p, B.work.p + B.up_off[h], B.up_cnt[h], B.far_smem, steady, s);
   enqueue_m2l(B, B.split_m2l, B.thr_m2l, s);
   for (size_t j = 0; j < B.down_off.size(); ++j)
-    launch_downward_batched(B.probs.p, B.work.p + B.down_off[j], B.down_cnt[j], B.far_smem, s);
+    launch_downward_batched(B.probs.p, B.work.p + B.down_off[j], B.down_cnt[j], B.far_smem, steady, s);
   DW_CUDA(cudaStreamWaitEvent(s, B.ev_join, 0));
   if (io)
     launch_scatter_batched(B.probs.p, B.d_leaf_off.p, B.P, B.Ltot, B.ld, *std::max_element(B.R.begin(), B.R.end()),

@@ -608,8 +608,10 @@ void check_device_error(Plan& P);
 void batch_far_attrs();
 size_t batch_far_smem(int lsum, int n, int n_pad, int nnz, int Rmax);
 size_t batch_far_need(int lsum, int n_pad);   // what the limit on index sets looks at
-void launch_moments_batched(const ProbF32* probs, const int2* work, int items, size_t smem, cudaStream_t s);
-void launch_downward_batched(const ProbF32* probs, const int2* work, int items, size_t smem, cudaStream_t s);
+void launch_moments_batched(const ProbF32* probs, const int2* work, int items, size_t smem, bool steady,
+                            cudaStream_t s);
+void launch_downward_batched(const ProbF32* probs, const int2* work, int items, size_t smem, bool steady,
+                             cudaStream_t s);
 void launch_gather_batched(const ProbF32* probs, const int* leaf_off, int P, int Ltot, int ld, float* xb,
                            cudaStream_t s);
 void launch_scatter_batched(const ProbF32* probs, const int* leaf_off, int P, int Ltot, int ld, int Rmax,

@@ -52,11 +52,9 @@ constexpr size_t far_smem(int lsum, int n, int n_pad, int nnz, int RC) {
 
 // Order of the sums.  STEADY: one thread a row of results, its terms in order,
 // and P_j by its division, then the factor sqrt(2j+1): what the conjugate
-// gradient iterations repeat bit for bit (apply_op in solve.cu); float32 always
-// runs so.  Otherwise (float64): several threads a row and the recurrence from a
-// table.
-template <typename T, bool STEADY>
-constexpr bool in_order() { return STEADY || sizeof(T) == 4; }
+// gradient iterations repeat bit for bit (apply_op in solve.cu).  Otherwise
+// several threads a row and the recurrence from a table (d = 16, 20 indices,
+// float32: 6 levels up 84 us in order, 50 us so).
 
 // p_hat_j(t) = sqrt(2j+1) P_j(2t-1), j = 1 .. deg, into row[j]; not in order: by
 // the normalised recurrence p_{j+1} = a_j u p_j - b_j p_{j-1} (a division and a
@@ -64,7 +62,7 @@ constexpr bool in_order() { return STEADY || sizeof(T) == 4; }
 template <typename T, bool STEADY>
 __device__ __forceinline__ void legendre_row(const ExpDev& e, T t, int deg, T* row) {
   const T u = T(2) * t - T(1);
-  if constexpr (in_order<T, STEADY>()) {
+  if constexpr (STEADY) {
     T pm = T(1), pc = u;
     row[1] = u * sqrt(T(3));
     for (int j = 1; j < deg; ++j) {
@@ -74,11 +72,11 @@ __device__ __forceinline__ void legendre_row(const ExpDev& e, T t, int deg, T* r
       pc = pn;
     }
   } else {
-    double prev = 1.0, cur = e.leg64[0].x * u;
+    T prev = T(1), cur = static_cast<T>(e.leg64[0].x) * u;
     row[1] = cur;
     for (int j = 1; j < deg; ++j) {
       const double2 c = e.leg64[j];
-      const double next = c.x * u * cur - c.y * prev;
+      const T next = static_cast<T>(c.x) * u * cur - static_cast<T>(c.y) * prev;
       row[j + 1] = next;
       prev = cur;
       cur = next;
@@ -130,7 +128,7 @@ struct Split {
   bool on;
   __device__ __forceinline__ explicit Split(int rows) {
     per = rows < kFarThreads ? rows : kFarThreads;
-    nsub = in_order<T, STEADY>() ? 1 : kFarThreads / per;
+    nsub = STEADY ? 1 : kFarThreads / per;
     sub = static_cast<int>(threadIdx.x) / per;
     row = static_cast<int>(threadIdx.x) - sub * per;
     on = sub < nsub;
@@ -358,35 +356,39 @@ k_downward(ExpDev e, int first, int level, int jmin, int J, int L, const int32_t
 __device__ __forceinline__ int level_of(int g) { return 31 - __clz(g + 1); }
 
 // Up to 4 right-hand sides in registers, or up to 16.
+template <bool STEADY>
 __device__ __forceinline__ void moments_item(const ProbF32& p, int c) {
   const int leaf = level_of(c) == p.J;
   if (p.R <= 4)
-    moments_body<float, 4, true>(p.e, c, leaf, p.L, p.count, p.pts, p.m_pad, p.xb, p.ynode, p.lo, p.iext, p.vinv, 0, p.R,
+    moments_body<float, 4, STEADY>(p.e, c, leaf, p.L, p.count, p.pts, p.m_pad, p.xb, p.ynode, p.lo, p.iext, p.vinv, 0, p.R,
                            p.mom);
   else
-    moments_body<float, 16, true>(p.e, c, leaf, p.L, p.count, p.pts, p.m_pad, p.xb, p.ynode, p.lo, p.iext, p.vinv, 0, p.R,
+    moments_body<float, 16, STEADY>(p.e, c, leaf, p.L, p.count, p.pts, p.m_pad, p.xb, p.ynode, p.lo, p.iext, p.vinv, 0, p.R,
                             p.mom);
 }
 
+template <bool STEADY>
 __device__ __forceinline__ void downward_item(const ProbF32& p, int c) {
   if (p.R <= 4)
-    downward_body<float, 4, true>(p.e, c, level_of(c), p.jmin, p.J, p.L, p.count, p.pts, p.m_pad, p.ynode, p.lo, p.iext,
+    downward_body<float, 4, STEADY>(p.e, c, level_of(c), p.jmin, p.J, p.L, p.count, p.pts, p.m_pad, p.ynode, p.lo, p.iext,
                             p.loc, p.lco, p.vinvt, 0, p.R, p.yfar);
   else
-    downward_body<float, 16, true>(p.e, c, level_of(c), p.jmin, p.J, p.L, p.count, p.pts, p.m_pad, p.ynode, p.lo, p.iext,
+    downward_body<float, 16, STEADY>(p.e, c, level_of(c), p.jmin, p.J, p.L, p.count, p.pts, p.m_pad, p.ynode, p.lo, p.iext,
                              p.loc, p.lco, p.vinvt, 0, p.R, p.yfar);
 }
 
+template <bool STEADY>
 __global__ void __launch_bounds__(kFarThreads)
 k_moments_batched(const ProbF32* probs, const int2* work) {
   const int2 w = work[blockIdx.x];
-  moments_item(probs[w.x], w.y);
+  moments_item<STEADY>(probs[w.x], w.y);
 }
 
+template <bool STEADY>
 __global__ void __launch_bounds__(kFarThreads)
 k_downward_batched(const ProbF32* probs, const int2* work) {
   const int2 w = work[blockIdx.x];
-  downward_item(probs[w.x], w.y);
+  downward_item<STEADY>(probs[w.x], w.y);
 }
 
 // Problem of a global leaf (binary search in the leaf offsets).
@@ -709,7 +711,7 @@ __device__ __noinline__ bool persist_barrier(const PersistArgs& pa, int ph, bool
 __device__ __forceinline__ void persist_up_items(const PersistArgs& pa, int h) {
   for (int i = static_cast<int>(blockIdx.x); i < pa.up_cnt[h]; i += static_cast<int>(gridDim.x)) {
     const int2 w = pa.work[pa.up_off[h] + i];
-    moments_item(pa.probs[w.x], w.y);
+    moments_item<false>(pa.probs[w.x], w.y);
     __syncthreads();
   }
 }
@@ -717,7 +719,7 @@ __device__ __forceinline__ void persist_up_items(const PersistArgs& pa, int h) {
 __device__ __forceinline__ void persist_down_items(const PersistArgs& pa, int j) {
   for (int i = static_cast<int>(blockIdx.x); i < pa.down_cnt[j]; i += static_cast<int>(gridDim.x)) {
     const int2 w = pa.work[pa.down_off[j] + i];
-    downward_item(pa.probs[w.x], w.y);
+    downward_item<false>(pa.probs[w.x], w.y);
     __syncthreads();
   }
 }
@@ -946,7 +948,7 @@ int far_levels_rc(Plan& P, bool up, int Rc) {
 
 template <typename T>
 int far_pass(Plan& P, bool up, int Rc, bool steady) {
-  if (steady || sizeof(T) == 4) return far_levels_rc<T, true>(P, up, Rc);
+  if (steady) return far_levels_rc<T, true>(P, up, Rc);
   return far_levels_rc<T, false>(P, up, Rc);
 }
 
@@ -1024,8 +1026,10 @@ void launch_scatter(Plan& P, double* y, int64_t ldy, int r0, int Rc, bool fp64) 
 
 void batch_far_attrs() {
   const int big = 200 * 1024;
-  DW_CUDA(cudaFuncSetAttribute(k_moments_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-  DW_CUDA(cudaFuncSetAttribute(k_downward_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  DW_CUDA(cudaFuncSetAttribute(k_moments_batched<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  DW_CUDA(cudaFuncSetAttribute(k_downward_batched<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  DW_CUDA(cudaFuncSetAttribute(k_moments_batched<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
+  DW_CUDA(cudaFuncSetAttribute(k_downward_batched<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
 }
 
 size_t batch_far_smem(int lsum, int n, int n_pad, int nnz, int Rmax) {
@@ -1038,12 +1042,16 @@ size_t batch_far_need(int lsum, int n_pad) {
   return std::max(a, b);
 }
 
-void launch_moments_batched(const ProbF32* probs, const int2* work, int items, size_t smem, cudaStream_t s) {
-  if (items > 0) k_moments_batched<<<items, kFarThreads, smem, s>>>(probs, work);
+void launch_moments_batched(const ProbF32* probs, const int2* work, int items, size_t smem, bool steady, cudaStream_t s) {
+  if (items <= 0) return;
+  if (steady) k_moments_batched<true><<<items, kFarThreads, smem, s>>>(probs, work);
+  else k_moments_batched<false><<<items, kFarThreads, smem, s>>>(probs, work);
 }
 
-void launch_downward_batched(const ProbF32* probs, const int2* work, int items, size_t smem, cudaStream_t s) {
-  if (items > 0) k_downward_batched<<<items, kFarThreads, smem, s>>>(probs, work);
+void launch_downward_batched(const ProbF32* probs, const int2* work, int items, size_t smem, bool steady, cudaStream_t s) {
+  if (items <= 0) return;
+  if (steady) k_downward_batched<true><<<items, kFarThreads, smem, s>>>(probs, work);
+  else k_downward_batched<false><<<items, kFarThreads, smem, s>>>(probs, work);
 }
 
 void launch_gather_batched(const ProbF32* probs, const int* leaf_off, int P, int Ltot, int ld, float* xb,

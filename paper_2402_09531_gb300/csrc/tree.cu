@@ -17,6 +17,7 @@
 // This file is compiled with -fmad=false so that the admissibility sums are
 // plain float64 products and adds in k order.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <utility>
 
@@ -29,8 +30,8 @@ namespace {
 constexpr unsigned long long kSign = 0x8000000000000000ull;
 
 __device__ __forceinline__ unsigned long long dkey(double x) {
-  x = x + 0.0;  // -0.0 -> +0.0
-  const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(x));
+  unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(x));
+  if (u == kSign) u = 0;   // -0.0 -> +0.0 (an addition of 0.0 would go to the float64 unit, 2 a clock)
   return (u & kSign) ? ~u : (u | kSign);
 }
 
@@ -348,7 +349,7 @@ __global__ void k_partition(const double* soa_in, const int32_t* perm_in, int64_
 // kernel and kept workspaces, both before k_move.
 constexpr int kSplitThreads = 1024;
 constexpr int kSplitMax = 32768;   // sites of a cluster, beyond it the whole GPU shares the level
-constexpr int kSplitKeys = 5632;   // keys kept in shared memory (with the rest within 48 KB)
+constexpr int kSplitKeys = 24576;  // keys kept in shared memory
 
 __global__ void __launch_bounds__(kSplitThreads)
 k_split(const double* __restrict__ soa_in, const int32_t* __restrict__ perm_in, int64_t n_all, int d,
@@ -762,6 +763,15 @@ void build_tree(Plan& P, const double* pts_dev, int64_t N, int64_t ld) {
   DW_CUDA(cudaStreamSynchronize(s));
   if (h_bad) fail(DWFMM_ERR_INVALID_ARG, "sites contain NaN or Inf");
 
+  {
+    static std::atomic<uint64_t> done{0};
+    const uint64_t bit = device_bit();
+    if (!(done.load() & bit)) {
+      DW_CUDA(cudaFuncSetAttribute(k_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   static_cast<int>(sizeof(unsigned long long)) * kSplitKeys));
+      done.fetch_or(bit);
+    }
+  }
   double* cur = soa0.p;
   double* nxt = soa1.p;
   int32_t* pcur = P.d_perm.p;

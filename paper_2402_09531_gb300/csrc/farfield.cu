@@ -37,15 +37,16 @@ __host__ __device__ constexpr int far_stride(int lsum) { return (lsum + 1) | 1; 
 template <typename T>
 __host__ __device__ constexpr int far_points(int lsum) {
   const int most = static_cast<int>(kFarTableBytes / sizeof(T)) / far_stride(lsum);
-  return most >= 128 ? 128 : most >= 64 ? 64 : 32;
+  return most >= kFarThreads ? kFarThreads : most >= 64 ? 64 : 32;
 }
 
 // Shared memory of both passes: tables, two arrays of n_pad x RC, the threads'
-// partial sums, a chunk's charges, the multi-indices.
+// partial sums (a chunk's charges in the same place), the multi-indices.  The
+// CTAs run beside the near field's, in what those leave of an SM.
 template <typename T>
 constexpr size_t far_smem(int lsum, int n, int n_pad, int nnz, int RC) {
   const int pc = far_points<T>(lsum);
-  return (static_cast<size_t>(pc) * far_stride(lsum) + (2 * static_cast<size_t>(n_pad) + kFarThreads + pc) * RC) *
+  return (static_cast<size_t>(pc) * far_stride(lsum) + (2 * static_cast<size_t>(n_pad) + kFarThreads) * RC) *
              sizeof(T) +
          static_cast<size_t>(n) * nnz * sizeof(int16_t);
 }
@@ -135,20 +136,45 @@ struct Split {
   }
 };
 
-// put(row, r, value) for every row and right-hand side; red: kFarThreads x RC.
+// dst[a][r] = load(a, r) for a < rows: every load of a thread starts before its
+// first store, which the compiler could not move them past (16 right-hand sides
+// one load after the other cost 5 us a level; d = 4, N = 12857, 16 right-hand
+// sides, float32 downward pass: 109 us, 52 us with all of them in flight).
+template <typename T, int RC, class F>
+__device__ __forceinline__ void stage(int rows, T* dst, F load) {
+  for (int a = threadIdx.x; a < rows; a += kFarThreads) {
+    T v[RC];
+#pragma unroll
+    for (int r = 0; r < RC; ++r) v[r] = load(a, r);
+#pragma unroll
+    for (int r = 0; r < RC; ++r) dst[a * RC + r] = v[r];
+  }
+}
+
+// put(row, r, value) for every row and right-hand side; red: RC x kFarThreads
+// (neighbouring threads in neighbouring banks, and neighbouring rows written
+// together).
 template <typename T, int RC, class S, class F>
-__device__ __forceinline__ void reduce(const S& s, int rows, const T (&acc)[RC], T* red, F put) {
+__device__ __forceinline__ void reduce(const S& s, const T (&acc)[RC], T* red, F put) {
+  if (s.nsub == 1) {   // the thread's sums are the row's
+    if (s.on) {
+#pragma unroll
+      for (int r = 0; r < RC; ++r) put(s.row, r, acc[r]);
+    }
+    return;
+  }
   __syncthreads();
   if (s.on) {
 #pragma unroll
-    for (int r = 0; r < RC; ++r) red[(s.sub * s.per + s.row) * RC + r] = acc[r];
+    for (int r = 0; r < RC; ++r) red[r * kFarThreads + threadIdx.x] = acc[r];
   }
   __syncthreads();
-  for (int q = threadIdx.x; q < rows * RC; q += kFarThreads) {
-    T v = red[q];
-    for (int u = 1; u < s.nsub; ++u) v += red[u * s.per * RC + q];
-    put(q / RC, q % RC, v);
-  }
+  if (s.on)
+    for (int r = s.sub; r < RC; r += s.nsub) {
+      T v = red[r * kFarThreads + s.row];
+      for (int u = 1; u < s.nsub; ++u) v += red[r * kFarThreads + u * s.per + s.row];
+      put(s.row, r, v);
+    }
 }
 
 // Moments of cluster g, then m = V^{-T} mu, for the right-hand sides r0 .. r0 +
@@ -165,8 +191,8 @@ __device__ __forceinline__ void moments_body(const ExpDev& e, int g, int leaf_mo
   T* tab = reinterpret_cast<T*>(smem_raw);     // [PC][LS]
   T* mu = tab + PC * LS;                       // [n_pad][RC]
   T* red = mu + 2 * np * RC;                   // [kFarThreads][RC]
-  T* qs = red + kFarThreads * RC;              // [PC][RC]
-  int16_t* fac = reinterpret_cast<int16_t*>(qs + PC * RC);
+  T* qs = red;                                 // [PC][RC], before the reduction
+  int16_t* fac = reinterpret_cast<int16_t*>(red + kFarThreads * RC);
   const T* lo = lo_all + static_cast<int64_t>(g) * d;
   const T* iext = iext_all + static_cast<int64_t>(g) * d;
   const int leaf = g - (L - 1);
@@ -193,9 +219,7 @@ __device__ __forceinline__ void moments_body(const ExpDev& e, int g, int leaf_mo
       const int cn = min(PC, S - cb);
       __syncthreads();
       fill_tables<T, STEADY>(e, cn, leaf_mode ? m_pad : np, lo, iext, tab, [&](int p) { return point(cb + p); });
-#pragma unroll
-      for (int r = 0; r < RC; ++r)
-        for (int p = threadIdx.x; p < cn; p += kFarThreads) qs[p * RC + r] = charge(cb + p, r);
+      stage<T, RC>(cn, qs, [&](int p, int r) { return charge(cb + p, r); });
       __syncthreads();
       if (s.on) {
         const int16_t* f = fac + (ab + s.row) * nnz;
@@ -206,7 +230,7 @@ __device__ __forceinline__ void moments_body(const ExpDev& e, int g, int leaf_mo
         }
       }
     }
-    reduce<T, RC>(s, rows, acc, red, [&](int a, int r, T v) { mu[(ab + a) * RC + r] = v; });
+    reduce<T, RC>(s, acc, red, [&](int a, int r, T v) { mu[(ab + a) * RC + r] = v; });
   }
   __syncthreads();
   // m = V^{-T} mu
@@ -222,7 +246,7 @@ __device__ __forceinline__ void moments_body(const ExpDev& e, int g, int leaf_mo
 #pragma unroll
         for (int r = 0; r < RC; ++r) acc[r] += v * mu[b * RC + r];
       }
-    reduce<T, RC>(s, rows, acc, red, [&](int a, int r, T v) {
+    reduce<T, RC>(s, acc, red, [&](int a, int r, T v) {
       mom[(static_cast<int64_t>(g) * kRC + r0 + r) * np + ab + a] = r0 + r < Rc ? v : T(0);
     });
   }
@@ -260,18 +284,15 @@ __device__ __forceinline__ void downward_body(const ExpDev& e, int g, int level,
   T* lamp = tab + PC * LS;                     // [n_pad][RC]
   T* lsm = lamp + np * RC;                     // [n_pad][RC]
   T* red = lsm + np * RC;                      // [kFarThreads][RC]
-  int16_t* fac = reinterpret_cast<int16_t*>(red + (kFarThreads + PC) * RC);
+  int16_t* fac = reinterpret_cast<int16_t*>(red + kFarThreads * RC);
   load_factors(e, fac);
-  auto row_of = [&](const T* x, int c, T* dst) {
-#pragma unroll
-    for (int r = 0; r < RC; ++r)
-      for (int a = threadIdx.x; a < n; a += kFarThreads)
-        dst[a * RC + r] = r0 + r < Rc ? x[(static_cast<int64_t>(c) * kRC + r0 + r) * np + a] : T(0);
+  auto of = [&](const T* x, int c) {
+    return [=](int a, int r) { return r0 + r < Rc ? x[(static_cast<int64_t>(c) * kRC + r0 + r) * np + a] : T(0); };
   };
-  row_of(loc, g, lsm);
+  stage<T, RC>(n, lsm, of(loc, g));
   if (level > jmin) {
     const int p = (g - 1) / 2;
-    row_of(lco, p, lamp);
+    stage<T, RC>(n, lamp, of(lco, p));
     const T* lo = lo_all + static_cast<int64_t>(p) * d;
     const T* iext = iext_all + static_cast<int64_t>(p) * d;
     const T* yn = ynode + static_cast<int64_t>(g) * d * np;
@@ -290,7 +311,7 @@ __device__ __forceinline__ void downward_body(const ExpDev& e, int g, int level,
 #pragma unroll
           for (int r = 0; r < RC; ++r) acc[r] += v * lamp[b * RC + r];
         }
-      reduce<T, RC>(s, rows, acc, red, [&](int a, int r, T v) { lsm[(ab + a) * RC + r] += v; });
+      reduce<T, RC>(s, acc, red, [&](int a, int r, T v) { lsm[(ab + a) * RC + r] += v; });
     }
   }
   __syncthreads();
@@ -307,7 +328,7 @@ __device__ __forceinline__ void downward_body(const ExpDev& e, int g, int level,
 #pragma unroll
         for (int r = 0; r < RC; ++r) acc[r] += v * lsm[b * RC + r];
       }
-    reduce<T, RC>(s, rows, acc, red, [&](int a, int r, T v) {
+    reduce<T, RC>(s, acc, red, [&](int a, int r, T v) {
       lamp[(ab + a) * RC + r] = v;
       if (level < J) lco[(static_cast<int64_t>(g) * kRC + r0 + r) * np + ab + a] = v;
     });
@@ -334,7 +355,7 @@ __device__ __forceinline__ void downward_body(const ExpDev& e, int g, int level,
 #pragma unroll
         for (int r = 0; r < RC; ++r) acc[r] += v * lamp[b * RC + r];
       }
-    reduce<T, RC>(s, rows, acc, red, [&](int i, int r, T v) {
+    reduce<T, RC>(s, acc, red, [&](int i, int r, T v) {
       if (r0 + r < Rc) yfar[(static_cast<int64_t>(leaf) * kRC + r0 + r) * m_pad + ib + i] = v;
     });
   }

@@ -229,7 +229,11 @@ __global__ void __launch_bounds__(kFT, 2) k_far_basis_tc(BasisArgs a) {
   const int cnt = (mode == 1 || (mode == 0 && !a.leaves)) ? 0 : a.count[g];
   const int K = mode == 0 ? (a.leaves ? a.m_pad : 256) : 128;
   const int tiles = mode == 2 ? a.m_pad / 128 : 1;
-  const int nchunk = K / kKC;
+  // chunks of the contraction with an entry: the others (nodes beyond n, sites
+  // beyond the leaf's) are zeros, and their products would add nothing
+  const bool pairs = mode == 0 && !a.leaves;   // two node blocks of 128 slots
+  const int cstep = pairs && n <= kKC ? 2 : 1;
+  const int nchunk = pairs ? K / kKC / cstep : max(1, ((mode == 0 ? cnt : n) + kKC - 1) / kKC);
   const int units = tiles * nchunk;
 
   // point p of the contraction (mode 0: column k; modes 1, 2: row of the tile)
@@ -347,7 +351,7 @@ __global__ void __launch_bounds__(kFT, 2) k_far_basis_tc(BasisArgs a) {
 
   // operands of unit u (tile u / nchunk, chunk u % nchunk) into stage u & 1
   auto gen = [&](int u) {
-    const int tl = u / nchunk, c = u % nchunk, st = u & 1;
+    const int tl = u / nchunk, c = u % nchunk * cstep, st = u & 1;
     if (mode == 0) fill_tab(c * kKC);
     else if (c == 0) fill_tab(tl * 128);
     __syncthreads();

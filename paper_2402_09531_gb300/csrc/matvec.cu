@@ -73,7 +73,9 @@ void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy
     const int Rc = std::min(kRC, R - r0);
     timer_begin(P, 0, s);
     P.near_parts = 0;
-    launch_gather(P, x, ldx, r0, Rc, fp64, fix, fp64 ? nullptr : P.xq32.p);
+    // the symmetric tensor-core near field reads the row layout
+    const bool xq = !fp64 && !(P.prec == DWFMM_P_MIXED && sum_padded_rc(Rc) == 16);
+    launch_gather(P, x, ldx, r0, Rc, fp64, fix, xq ? P.xq32.p : nullptr);
     timer_end(P, 0, s, 1);
     const bool rot = !fp64 && !steady && rot_ready(P, Rc);
     if (!fp64) m2l_autotune(P, Rc);   // once per tree, before the near field starts

@@ -397,7 +397,8 @@ void launch_scaled_blocks(const double* src, int64_t groups, int d, int D, int l
     k_scaled_blocks<<<ceil_div(groups * ld, 256), 256, 0, s>>>(src, groups, d, D, ld, kernel, sigma, dst);
 }
 
-// rot: each unordered pair once (rot_ready).  The charges are in P.xq32.
+// rot: each unordered pair once (rot_ready).  The charges are in P.xq32, but for
+// 9..16 right-hand sides of MIXED plans.
 bool p2p_f32_tuned(Plan& P, int Rc, bool rot, bool steady, cudaStream_t s) {
   const int D = padded_dim(P.d);
   if (D < 0) return false;
@@ -423,6 +424,8 @@ bool p2p_f32_tuned(Plan& P, int Rc, bool rot, bool steady, cudaStream_t s) {
   P.near_engine = 4;
   if (P.prec == DWFMM_P_MIXED && RC == 16 && near_sym_tc(P, D, Rc, s)) return true;
   P.near_engine = 3;
+  if (P.prec == DWFMM_P_MIXED && RC == 16)   // the gather leaves these to the kernels that read them
+    launch_interleave(P.xb32.p, P.L, P.m_pad, RC, P.xq32.p, s);
   if (P.prec == DWFMM_P_MIXED && RC == 16 &&
       sum_tc(D, P.kernel, P.d_ptsk.p, static_cast<int64_t>(D + 1) * P.m_pad, P.d_ptsk.p,
              static_cast<int64_t>(D + 1) * P.m_pad, P.xq32.p, P.L, P.bq32, P.ynear32.p,

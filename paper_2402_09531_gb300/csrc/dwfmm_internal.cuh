@@ -618,6 +618,11 @@ void launch_scatter_batched(const ProbF32* probs, const int* leaf_off, int P, in
                             const BatchParts& parts, const float* ynear, const float* yfar, cudaStream_t s);
 void launch_rot(int D, int kernel, int RC, const RotArgs& a, int chunks, cudaStream_t s);   // p2p_rot.cu
 int rot_sources_per_chunk();
+inline bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  DW_CUDA(cudaStreamIsCapturing(s, &cs));
+  return cs != cudaStreamCaptureStatusNone;
+}
 bool rot_fits(int ld, int least, int rc);   // slots, sites of the smallest leaf, padded right-hand sides
 size_t persist_rot_bytes(int D, int RC, int ld);
 // persistent batch matvec: dynamic shared memory and resident CTAs per SM

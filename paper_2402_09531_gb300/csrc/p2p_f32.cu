@@ -552,9 +552,7 @@ bool m2l_ordered_tc(Plan& P, int D, int Rc) {
 void m2l_autotune(Plan& P, int Rc) {
   if (P.prec != DWFMM_P_MIXED || Rc < 9 || Rc > 16 || P.m2l_pref >= 0 || P.m2l_tuned >= 0) return;
   if (P.jmin > P.J || P.tm.on) return;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  DW_CUDA(cudaStreamIsCapturing(P.stream, &cs));
-  if (cs != cudaStreamCaptureStatusNone) return;
+  if (capturing(P.stream)) return;
   const int D = padded_dim(P.d);
   if (D < 0 || stage_bytes(D, 16, P.n_pad) > 200 * 1024) return;
   ensure_attrs();

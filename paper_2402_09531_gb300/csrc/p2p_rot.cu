@@ -116,6 +116,7 @@ bool row_chunks(Plan& P, int per, int least, RowChunks& out) {
 // share a target; partial sums beyond 8 GB are not worth their traffic.
 bool rot_ready(Plan& P, int Rc) {
   if (sum_padded_dim(P.d) < 0 || !rot_fits(P.m_pad, kRotMinLeaf, sum_padded_rc(Rc))) return false;
+  if (P.rot_state < 0 && capturing(P.stream)) return false;   // the chunks are built outside a capture
   if (P.rot_state < 0) P.rot_state = row_chunks(P, kRotPer, kRotMinLeaf, P.rot) ? 1 : 0;
   if (P.rot_state == 0) return false;
   const size_t row = static_cast<size_t>(Rc) * round_up(P.rot.cmax, 8);

@@ -135,6 +135,7 @@ void shape(FixArgs& a, int n) {
 // sums for both sides in registers.
 bool sym_ready(Plan& P) {
   if (P.fx_sym >= 0) return P.fx_sym == 1;
+  if (capturing(P.stream)) return false;
   P.fx_sym = 0;
   if (P.m_pad > fx::kThreads || P.sym_nup <= 0) return false;
   // a warp takes 64 sources at a time; 8 such batches where that still leaves
@@ -152,6 +153,7 @@ constexpr size_t kSymMaxBytes = size_t(8) << 30;   // partial sums of the symmet
 
 bool fix_ready(Plan& P) {
   if (P.fx_state >= 0) return P.fx_state == 1;
+  if (capturing(P.stream)) return false;   // the records are built outside a capture
   P.fx_state = 0;
   if (P.d > fx::kMaxD || P.N == 0) return false;
   double longest = 0.0;

@@ -155,6 +155,10 @@ dwfmm_status dwfmm_tree_build(dwfmm_plan plan, const double* pts, int64_t n, int
  * >= N, caller's site order.  x and y must not overlap.  With device
  * pointers the call returns once the work is enqueued on `stream`; with a
  * host y it synchronises `stream` before returning.
+ * A product that the caller captured into a CUDA graph may be replayed until
+ * the next dwfmm_tree_build or dwfmm_plan_destroy on the plan, whatever other
+ * calls run in between (ordered with it): the workspaces it uses stay where
+ * they are for as long as the tree does.
  * Errors: STATE (no tree), INVALID_ARG (nrhs outside 1..max_rhs, ld < N,
  * NULL), CUDA. */
 dwfmm_status dwfmm_matvec(dwfmm_plan plan, const double* x, double* y, int32_t nrhs,

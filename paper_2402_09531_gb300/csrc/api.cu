@@ -36,6 +36,7 @@ void Plan::drop_tree() {
   m2l_tune_ms[0] = m2l_tune_ms[1] = -1.0;
   dpad = -1;
   h_upcount.clear();
+  outgrown.clear();
   cg_r.release();
   cg_p.release();
   cg_ap.release();

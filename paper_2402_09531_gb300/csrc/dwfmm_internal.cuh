@@ -15,8 +15,10 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <algorithm>
 #include <cstdint>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/dwfmm.h"
@@ -85,6 +87,12 @@ struct DBuf {
     p = nullptr;
     n = 0;
   }
+};
+
+// Workspace whose size follows a product's right-hand sides or form (Plan::grow).
+template <class T>
+struct WBuf : DBuf<T> {
+  int tree = -1;   // tree (Plan::tree_gen) whose products last held it
 };
 
 // Expansion tables shared by all clusters (device pointers).
@@ -480,7 +488,7 @@ struct Plan {
   // looked at for this tree, 0 = does not apply, 1 = chunks are built
   int rot_state = -1;
   RowChunks rot;
-  DBuf<float> rot_pf, rot_pt;
+  WBuf<float> rot_pf, rot_pt;
   // where the last near field left its sums: 0 = ynear, 1 = chunk sums in
   // sym_pf and transposed sums in sym_pt (float64), 2 = rot_pf, rot_pt (float32)
   int near_parts = 0;
@@ -495,14 +503,14 @@ struct Plan {
   DBuf<float> bq32;           // TF32 hi/lo charge blocks for the tensor-core P2P
   DBuf<float> bqm32;          // the same for the tensor-core M2L (moments at the nodes)
   DBuf<int32_t> part_rows;    // the near lists in parts
-  DBuf<float> entry_parts32;  // one sum per near entry (steady near field)
-  DBuf<float> near_parts32;   // partial near-field sums of small float32 problems
-  DBuf<double> near_parts64;  // partial near-field sums of small float64 problems (split lists)
+  WBuf<float> entry_parts32;  // one sum per near entry (steady near field)
+  WBuf<float> near_parts32;   // partial near-field sums of small float32 problems
+  WBuf<double> near_parts64;  // partial near-field sums of small float64 problems (split lists)
   // symmetric float64 near field: upper entries (T, S >= T) of the near list,
   // per-leaf rows of the upper and lower lists, slots of the lower entries,
   // forward and transposed partial sums
   DBuf<int32_t> sym_t, sym_s, sym_uprow, sym_lorow, sym_loslot;
-  DBuf<double> sym_pf, sym_pt;
+  WBuf<double> sym_pf, sym_pt;
   int64_t sym_nup = 0;
   bool sym_ok = false;
   // symmetric tensor-core near field (MIXED): target leaves by decreasing
@@ -552,6 +560,37 @@ struct Plan {
                   d_leg64.p};
   }
   TreeDev tree_dev() const { return TreeDev{N, J, L, C, m_pad, d_begin.p, d_count.p}; }
+  // Workspaces that a later product of the same tree had to outgrow.  A captured
+  // graph (the kept conjugate gradient iterations, a caller's own) may hold their
+  // addresses, so they stay allocated until the tree goes.
+  std::vector<DBuf<unsigned char>> outgrown;
+  template <class T>
+  void grow(WBuf<T>& b, size_t count) {
+    if (!b.p || count > b.n) {
+      if (b.tree != tree_gen) b.release();   // another tree's: nothing holds it
+      WBuf<T> old(std::move(b));
+      try {
+        b.alloc(count);
+      } catch (...) {
+        b = std::move(old);
+        throw;
+      }
+      if (old.p) {
+        outgrown.emplace_back();
+        outgrown.back().p = reinterpret_cast<unsigned char*>(old.p);
+        outgrown.back().n = old.n * sizeof(T);
+        old.p = nullptr;
+      }
+    }
+    b.tree = tree_gen;
+  }
+  // Columns to size such a workspace for: the kernels' next count of right-hand
+  // sides (at most what the plan takes), so that it grows once per count; fewer
+  // where `most` columns fit, never below Rc.
+  int work_cols(int Rc, int padded, size_t most) const {
+    const int c = std::max(Rc, std::min(padded, max_rhs));
+    return static_cast<size_t>(c) <= most ? c : std::max(Rc, static_cast<int>(most));
+  }
   void trim_tree_work();
   void drop_tree();   // no tree; buffers that the next one may use stay
   void free_tree();

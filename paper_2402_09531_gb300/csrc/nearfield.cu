@@ -164,7 +164,7 @@ void p2p_impl(Plan& P, int Rc, const T* pts, const T* xb, T* ynear, cudaStream_t
     return;
   }
   const int64_t stride = static_cast<int64_t>(P.L) * o_gstride;
-  P.near_parts64.alloc(static_cast<size_t>(splits) * stride);
+  P.grow(P.near_parts64, static_cast<size_t>(splits) * stride);
   T* part = reinterpret_cast<T*>(P.near_parts64.p);
   dispatch_ksum<T>(P.kernel, P.L, 0, P.d_near_rowptr.p, P.d_near_col.p, P.d, T(1.0 / P.sigma), pts, side, pts,
                    side, xb, o_gstride, P.m_pad, part, o_gstride, P.m_pad, Rc, s, splits, stride);
@@ -364,10 +364,12 @@ constexpr size_t kSymMaxBytes = size_t(8) << 30;
 
 bool near_sym(Plan& P, int Rc, cudaStream_t s) {
   if (!P.sym_ok || Rc > kSymMaxRc || P.m_pad > kThreads || P.d > 20 || P.sym_nup <= 0) return false;
-  const size_t per = static_cast<size_t>(P.sym_nup) * Rc * P.m_pad;
-  if (2 * per * sizeof(double) > kSymMaxBytes) return false;
-  P.sym_pf.alloc(per);
-  P.sym_pt.alloc(per);
+  const size_t col = static_cast<size_t>(P.sym_nup) * P.m_pad;
+  const size_t most = kSymMaxBytes / (2 * col * sizeof(double));
+  if (most < static_cast<size_t>(Rc)) return false;
+  const size_t cols = P.work_cols(Rc, Rc <= 1 ? 1 : kSymMaxRc, most);
+  P.grow(P.sym_pf, col * cols);
+  P.grow(P.sym_pt, col * cols);
   switch (P.kernel) {
     case DWFMM_K_EXP: launch_near_sym_k<DWFMM_K_EXP>(P, Rc, s); break;
     case DWFMM_K_MATERN32: launch_near_sym_k<DWFMM_K_MATERN32>(P, Rc, s); break;

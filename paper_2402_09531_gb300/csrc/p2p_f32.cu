@@ -464,7 +464,8 @@ bool p2p_f32_tuned(Plan& P, int Rc, bool rot, bool steady, cudaStream_t s) {
     a.entry_t = P.d_near_pairs.p;
     a.entry_off = P.L - 1;
     a.out_gstride = static_cast<int64_t>(Rc) * P.m_pad;
-    P.entry_parts32.alloc(static_cast<size_t>(P.nnear) * Rc * P.m_pad);
+    const size_t col = static_cast<size_t>(P.nnear) * P.m_pad;
+    P.grow(P.entry_parts32, col * P.work_cols(Rc, RC, kEntryPartsBytes / (col * sizeof(float))));
     a.out = P.entry_parts32.p;
     dispatch(D, P.kernel, RC, a, static_cast<int>(P.nnear), threads, smem, s);
     k_fold_entries<<<ceil_div(static_cast<int64_t>(P.L) * Rc * P.m_pad, 128), 128, 0, s>>>(
@@ -478,7 +479,7 @@ bool p2p_f32_tuned(Plan& P, int Rc, bool rot, bool steady, cudaStream_t s) {
     a.rowptr = P.part_rows.p;
     a.row_step = a.parts = splits;
     a.split_stride = static_cast<int64_t>(P.L) * a.out_gstride;
-    P.near_parts32.alloc(static_cast<size_t>(splits) * a.split_stride);
+    P.grow(P.near_parts32, static_cast<size_t>(splits) * a.split_stride);
     a.out = P.near_parts32.p;
     dispatch(D, P.kernel, RC, a, P.L, threads, smem, s);
     k_add_parts<<<ceil_div(static_cast<int64_t>(P.L) * Rc * P.m_pad, 256), 256, 0, s>>>(

@@ -119,11 +119,12 @@ bool rot_ready(Plan& P, int Rc) {
   if (P.rot_state < 0 && capturing(P.stream)) return false;   // the chunks are built outside a capture
   if (P.rot_state < 0) P.rot_state = row_chunks(P, kRotPer, kRotMinLeaf, P.rot) ? 1 : 0;
   if (P.rot_state == 0) return false;
-  const size_t row = static_cast<size_t>(Rc) * round_up(P.rot.cmax, 8);
-  const size_t npf = P.rot.n * row, npt = P.sym_nup * row;
-  if ((npf + npt) * sizeof(float) > kRotMaxBytes) return false;
-  P.rot_pf.alloc(npf);
-  P.rot_pt.alloc(npt);
+  const size_t row = round_up(P.rot.cmax, 8);
+  const size_t most = kRotMaxBytes / ((static_cast<size_t>(P.rot.n) + P.sym_nup) * row * sizeof(float));
+  if (most < static_cast<size_t>(Rc)) return false;
+  const size_t cols = P.work_cols(Rc, sum_padded_rc(Rc), most);
+  P.grow(P.rot_pf, P.rot.n * row * cols);
+  P.grow(P.rot_pt, P.sym_nup * row * cols);
   return true;
 }
 

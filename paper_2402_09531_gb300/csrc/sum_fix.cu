@@ -209,10 +209,13 @@ bool near_fix(Plan& P, int Rc, cudaStream_t s) {
   k_fix_charges<<<ceil_div(static_cast<int64_t>(P.L) * RC * 32, 128), 128, 0, s>>>(
       P.xb64.p, 0, P.L, P.m_pad, Rc, RC, P.fx_colmax.p, reinterpret_cast<int2*>(P.fx_q.p), P.fx_qs.p, P.fx_colscale.p,
       P.fx_flag.p);
-  const size_t npf = static_cast<size_t>(P.fx_rows.n) * Rc * P.m_pad, npt = static_cast<size_t>(P.sym_nup) * Rc * P.m_pad;
-  if (P.fx_sym == 1 && RC <= 4 && (npf + npt) * sizeof(double) <= kSymMaxBytes) {
-    P.sym_pf.alloc(npf);
-    P.sym_pt.alloc(npt);
+  size_t most = 0;   // columns of partial sums
+  if (P.fx_sym == 1 && RC <= 4)
+    most = kSymMaxBytes / ((static_cast<size_t>(P.fx_rows.n) + P.sym_nup) * P.m_pad * sizeof(double));
+  if (most >= static_cast<size_t>(Rc)) {
+    const size_t cols = P.work_cols(Rc, RC, most);
+    P.grow(P.sym_pf, P.fx_rows.n * cols * P.m_pad);
+    P.grow(P.sym_pt, P.sym_nup * cols * P.m_pad);
     FixSymArgs b{};
     b.rec = reinterpret_cast<const int4*>(P.fx_pts.p);
     b.q = reinterpret_cast<const int2*>(P.fx_q.p);
@@ -272,7 +275,7 @@ bool near_fix(Plan& P, int Rc, cudaStream_t s) {
     dispatch(P.kernel, P.d, RC, a, ctas, s);
   } else {
     const int64_t stride = static_cast<int64_t>(P.L) * a.o_gstride;
-    P.near_parts64.alloc(static_cast<size_t>(a.splits) * stride);
+    P.grow(P.near_parts64, static_cast<size_t>(a.splits) * stride);
     a.out = P.near_parts64.p;
     a.split_stride = stride;
     dispatch(P.kernel, P.d, RC, a, ctas, s);

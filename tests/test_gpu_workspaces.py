@@ -1,0 +1,44 @@
+"""Workspaces whose size follows the right-hand sides, under graphs that hold
+their addresses."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")]
+
+
+def setup(prec, n=1500, d=4, r=16, leaf=64, kernel="matern32", eta=1e9, seed=11):
+    from paper_2402_09531_gb300 import Plan
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    pts = torch.rand((n, d), dtype=torch.float64, device="cuda", generator=g)
+    x = torch.randn((r, n), dtype=torch.float64, device="cuda", generator=g)
+    p = Plan(d, kernel=kernel, gamma=np.ones(d), q=1.0, eta=eta, leaf_size=leaf, precision=prec, max_rhs=16)
+    p.tree_build(pts)
+    return p, pts, x
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "mixed"])
+@pytest.mark.parametrize("first,wide", [(1, 2), (1, 8), (4, 16)])
+def test_solve_replayed_after_a_wider_product(prec, first, wide):
+    """The kept iterations of a solve are replayed after a product (and an
+    incremental step) that needed larger workspaces."""
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        p, pts, x = setup(prec)
+        f = x[:first].contiguous()
+        got = []
+        for _ in range(2):
+            c = torch.zeros_like(f)
+            status, its, _ = p.solve(1e-1, f, c, rtol=1e-10, maxit=3000)
+            assert status == 0 and its > 32     # three runs of 16 iterations: plain, captured, replayed
+            got.append(c)
+            y = torch.empty_like(x[:wide])
+            p.matvec(x[:wide].contiguous(), y)
+            p.cg_begin(1e-1, f, rtol=1e-10)
+            p.cg_step(1)
+        q, _, _ = setup(prec)
+        c = torch.zeros_like(f)
+        q.solve(1e-1, f, c, rtol=1e-10, maxit=3000)
+        stream.synchronize()
+        assert torch.equal(got[0], got[1]) and torch.equal(got[0], c)

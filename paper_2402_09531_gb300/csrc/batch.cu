@@ -650,11 +650,10 @@ void batch_create(Batch& B, Plan* const* plans, const int32_t* nrhs, int count) 
   B.n_pad = P0.n_pad;
   B.ld = P0.m_pad;
   B.D = 0;
-  int lsum_max = 0, nnz_max = 1, Rmax = 1;
+  int lsum_max = 0, Rmax = 1;
   for (int i = 0; i < count; ++i) {
     B.D = std::max(B.D, sum_padded_dim(B.plans[i]->d));
     lsum_max = std::max(lsum_max, B.plans[i]->lsum);
-    nnz_max = std::max(nnz_max, B.plans[i]->nnz_max);
     Rmax = std::max(Rmax, B.R[i]);
   }
   B.RCmax = sum_padded_rc(Rmax);
@@ -788,7 +787,10 @@ void batch_create(Batch& B, Plan* const* plans, const int32_t* nrhs, int count) 
   }
   B.work.alloc(std::max<size_t>(w.size(), 1));
   if (!w.empty()) DW_CUDA(cudaMemcpy(B.work.p, w.data(), sizeof(int2) * w.size(), cudaMemcpyHostToDevice));
-  B.far_smem = batch_far_smem(lsum_max, B.n, B.n_pad, nnz_max, Rmax);
+  // the most that any problem's own layout takes: a larger table has fewer points
+  // in it, so the largest index set is not the one that needs most
+  for (int i = 0; i < count; ++i)
+    B.far_smem = std::max(B.far_smem, batch_far_smem(B.plans[i]->lsum, B.n, B.n_pad, B.plans[i]->nnz_max, B.R[i]));
   if (batch_far_need(lsum_max, B.n_pad) > 200 * 1024) fail(DWFMM_ERR_INVALID_ARG, "index sets too large for a batch");
   batch_far_attrs();
   ensure_sum_attrs();

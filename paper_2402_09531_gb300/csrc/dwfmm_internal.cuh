@@ -645,7 +645,7 @@ bool m2l_f32_tuned(Plan& P, int Rc, bool steady);
 void check_device_error(Plan& P);
 // batches (batch.cu uses these)
 void batch_far_attrs();
-size_t batch_far_smem(int lsum, int n, int n_pad, int nnz, int Rmax);
+size_t batch_far_smem(int lsum, int n, int n_pad, int nnz, int R);
 size_t batch_far_need(int lsum, int n_pad);   // what the limit on index sets looks at
 void launch_moments_batched(const ProbF32* probs, const int2* work, int items, size_t smem, bool steady,
                             cudaStream_t s);

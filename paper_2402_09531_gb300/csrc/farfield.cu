@@ -1053,8 +1053,9 @@ void batch_far_attrs() {
   DW_CUDA(cudaFuncSetAttribute(k_downward_batched<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
 }
 
-size_t batch_far_smem(int lsum, int n, int n_pad, int nnz, int Rmax) {
-  return far_smem<float>(lsum, n, n_pad, nnz, Rmax <= 4 ? 4 : 16);
+// One problem's shared memory in the batched passes (moments_item, downward_item).
+size_t batch_far_smem(int lsum, int n, int n_pad, int nnz, int R) {
+  return far_smem<float>(lsum, n, n_pad, nnz, R <= 4 ? 4 : 16);
 }
 
 size_t batch_far_need(int lsum, int n_pad) {

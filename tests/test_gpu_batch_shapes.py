@@ -1,0 +1,36 @@
+"""Batches whose problems need different shared memory in the passes over the
+tree.  The points that share a Legendre table halve as its rows pass 79 and
+159 values, so the problem with the larger index set takes less of it."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")]
+
+
+# degrees 0 .. q in the first dimension only: q + 1 values a table row for d = 1,
+# q + d for the others
+@pytest.mark.parametrize("q,r", [(77, (8, 8)), (77, (2, 3)), (77, (1, 9)), (78, (8, 8))])
+@pytest.mark.parametrize("engine", ["graph", "persistent"])
+def test_batch_of_index_sets_around_a_change_of_table(q, r, engine):
+    from paper_2402_09531_gb300 import Batch, Plan
+    g = torch.Generator(device="cuda").manual_seed(q)
+    plans, xs = [], []
+    for d, n, k in ((1, 3000, r[0]), (2, 2500, r[1])):
+        gamma = np.array([1.0, 1e-4])[:d]
+        pts = (2 * torch.rand((n, d), dtype=torch.float64, device="cuda", generator=g) - 1) * torch.as_tensor(
+            gamma, device="cuda")
+        p = Plan(d, kernel="exp", gamma=gamma, q=float(q), leaf_size=128, precision="fp32", max_rhs=k)
+        p.tree_build(pts)
+        assert p.info()[0] == q + 1 and p.info()[1] > 0
+        plans.append(p)
+        xs.append(torch.randn((k, n), dtype=torch.float64, device="cuda", generator=g))
+    b = Batch(plans, list(r))
+    b.set_engine(engine)
+    ys = [torch.full_like(x, float("nan")) for x in xs]
+    b.matvec(xs, ys)
+    for p, x, y in zip(plans, xs, ys):
+        want = torch.empty_like(x)
+        p.matvec(x, want)
+        assert float(torch.linalg.norm(y - want) / torch.linalg.norm(want)) <= 1e-6
+    b.close()

@@ -826,6 +826,7 @@ void batch_matvec(Batch& B, const double* const* x, double* const* y, cudaStream
     B.h_probs[i].x = x[c];
     B.h_probs[i].y = y[c];
   }
+  B.cg_host.clear();   // the iterations' operands are no longer in the table
   // the table lives in device memory; order it before the graph on the caller's stream
   DW_CUDA(cudaMemcpyAsync(B.probs.p, B.h_probs, sizeof(ProbF32) * B.P, cudaMemcpyHostToDevice, s));
   DW_CUDA(cudaEventRecord(B.ev_copy, s));

@@ -34,3 +34,36 @@ def test_batch_of_index_sets_around_a_change_of_table(q, r, engine):
         p.matvec(x, want)
         assert float(torch.linalg.norm(y - want) / torch.linalg.norm(want)) <= 1e-6
     b.close()
+
+
+def test_product_between_batched_iterations():
+    """The iterations go on with their own vectors after the batch multiplied
+    the caller's."""
+    from paper_2402_09531_gb300 import Batch, Plan
+    g = torch.Generator(device="cuda").manual_seed(5)
+    plans, fs = [], []
+    for n in (900, 1300):
+        p = Plan(4, kernel="matern32", gamma=np.ones(4), q=2.0, leaf_size=64, precision="fp32", max_rhs=2)
+        p.tree_build(torch.rand((n, 4), dtype=torch.float64, device="cuda", generator=g))
+        plans.append(p)
+        fs.append(torch.randn((2, n), dtype=torch.float64, device="cuda", generator=g))
+    b = Batch(plans, [2, 2])
+    got = []
+    for between in (False, True):
+        for p, f in zip(plans, fs):
+            p.cg_begin(1.0, f, rtol=1e-12)
+        ys = [torch.full_like(f, float("nan")) for f in fs]
+        b.matvec(fs, ys)
+        keep = [y.clone() for y in ys]
+        b.cg_step(3)
+        if between:
+            b.matvec(fs, ys)
+        b.cg_step(3)
+        cs = [torch.empty_like(f) for f in fs]
+        for p, c in zip(plans, cs):
+            p.cg_result(c)
+        torch.cuda.synchronize()
+        assert all(torch.equal(y, k) for y, k in zip(ys, keep))
+        got.append(cs)
+    assert all(torch.equal(a, c) for a, c in zip(*got))
+    b.close()

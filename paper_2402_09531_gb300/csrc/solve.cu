@@ -74,8 +74,8 @@ void dots(Plan& P, const double* a, const double* b, int64_t n, int64_t ld, int 
 }
 
 // A v = K_tilde v + lam v (into out); v, out: n x R, leading dimension n.
-// steady: the iterations of the incremental CG, whose operator keeps one order of
-// its sums whatever the plain product uses.  K_tilde may be mildly indefinite,
+// steady: the iterations of the incremental CG (and of a float64 plan's solve),
+// whose operator keeps one order of its sums whatever the plain product uses.  K_tilde may be mildly indefinite,
 // and eight iterations then turn a change of the operator's last bits into one
 // 1e4 to 1e8 times as large.
 void apply_op(Plan& P, const double* v, double* out, int R, double lam, bool fp64, bool steady = false) {
@@ -103,7 +103,10 @@ int cg_dev(Plan& P, const double* b, int R, double lam, double rtol, int maxit, 
   constexpr int kSolveChunk = 16;
   cg_begin(P, lam, b, R, P.N, rtol);
   CgState& S = P.cgs;
-  S.steady = false;   // solved to a tolerance, with the fastest operator
+  // A float64 plan's solve is the incremental CG's, iterate for iterate, so it
+  // keeps that operator's order of the sums.  The inner solves of the refinement
+  // take the fastest one: the float64 residual decides there.
+  S.steady = P.prec == DWFMM_P_FP64;
   st.assign(R, 2);
   int done = 0, its = 0;
   while (done < maxit) {

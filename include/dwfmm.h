@@ -357,8 +357,10 @@ dwfmm_status dwfmm_plan_info(dwfmm_plan plan, int64_t* n_x, int64_t* n_far, int6
 /* Which engine evaluated the near field N (Eq. (5.1)) in the plan's last
  * matvec (*engine, -1 before the first): 0 float64, one CTA per target leaf
  * over its near list; 1 float64, each unordered near pair of leaves once
- * (both in fixed point on the integer pipes, to at least float64's accuracy,
- * where d <= 16 and the sites' box is within about 22 length scales);
+ * (both with kernel values from the integer pipes, each within a relative
+ * 2^-52, and float64 sums, where d <= 16 and the diagonal of the sites' box,
+ * rounded up to a power of two, is below 22.2 sigma for the exponential, 12.8
+ * sigma for Matern-3/2, 6.7 sigma for the Gaussian);
  * 2 float32 on the CUDA cores; 3 MIXED, contraction on the tensor cores (TF32
  * hi/lo, every ordered pair); 4 MIXED, each unordered near pair once, FP16
  * hi/lo on the tensor cores with fixed-point transposed sums; 5 as 4, with

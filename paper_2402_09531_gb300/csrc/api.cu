@@ -103,10 +103,6 @@ void Plan::free_tree() {
   rot_pt.release();
   fx_pts.release();
   fx_nodes.release();
-  fx_q.release();
-  fx_qm.release();
-  fx_qs.release();
-  fx_qms.release();
   sym_t.release();
   sym_s.release();
   sym_uprow.release();
@@ -173,9 +169,6 @@ void Plan::free_all() {
   far_vt_ok = false;
   d_err.release();
   fx_table.release();
-  fx_flag.release();
-  fx_colmax.release();
-  fx_colscale.release();
   stage_in.release();
   stage_out.release();
   for (auto& r : tm.recs) {

@@ -238,18 +238,7 @@ struct PersistArgs {
 };
 
 
-namespace ks {
-// Rows of one side of a sum (ksum.cuh).
-struct Side {
-  int64_t gstride;   // elements between groups
-  int ld;            // elements between coordinate rows (or rhs rows)
-  const int32_t* count;
-  int count_off;
-  int count_const;   // used when count == nullptr
-};
-}  // namespace ks
-
-// Fixed-point float64 kernel summation (fix64.cuh, sum_fix.cuh).
+// Float64 kernel summation with fixed-point kernel values (fix64.cuh, sum_fix.cuh).
 namespace fx {
 
 struct Consts {
@@ -258,12 +247,14 @@ struct Consts {
 
 struct FixArgs {
   const int4* rec;               // point records [group][ld][2 DM], targets and sources
-  const int2* q;                 // charge limbs [group][ld][RC]
-  const double* qscale;          // [group][16]
+  const double* charge;          // rows [group][16][ld]
+  int64_t q_gstride;
   const unsigned long long* table;
   Consts c;
   const int32_t* rowptr;
   const int32_t* col;
+  const int32_t* count;          // group sizes (count[count_off + g]); nullptr -> count_const
+  int count_off, count_const;
   int first, ld, Rc;
   int passes, tp, nsub;          // passes of tp targets, threads per target
   int group_entries;             // source groups per stage (short groups), 0: chunks of one group
@@ -271,21 +262,12 @@ struct FixArgs {
   int64_t split_stride;
   double* out;                   // [group][16][ld]
   int64_t o_gstride;
-  const int* flag;               // != 0: a charge is not finite or below 2^-960, sum in float64
-  // the float64 path's view of the same data; side also holds the group sizes
-  int d;
-  double inv_sigma;
-  const double* coord;
-  ks::Side side;
-  const double* charge;
-  int64_t q_gstride;
 };
 
 // Symmetric form: each unordered pair of near leaves once (sum_fix.cuh).
 struct FixSymArgs {
   const int4* rec;               // leaf records [leaf][ld][2 DM]
-  const int2* q;                 // charge limbs [leaf][ld][RC], one scale per column
-  const double* qscale;          // [16]
+  const double* charge;          // rows [leaf][16][ld]
   const unsigned long long* table;
   Consts c;
   const int32_t* count;          // [leaf]
@@ -297,11 +279,6 @@ struct FixSymArgs {
   int batches;                   // batches of 64 sources per warp
   double* pf;                    // [chunk][Rc][ld] sums for the row's targets
   double* pt;                    // [entry][Rc][ld] sums for the entry's sources
-  const int* flag;
-  int d;
-  double inv_sigma;
-  const double* coord;           // [leaf][d][ld]
-  const double* charge;          // [leaf][16][ld]
 };
 
 void launch_fix_exp(int d, int RC, const FixArgs& a, int ctas, cudaStream_t s);
@@ -468,18 +445,15 @@ struct Plan {
   // solve workspace
   DBuf<double> cg_r, cg_p, cg_ap, cg_c, cg_f, cg_dot, cg_tmp;
 
-  // fixed-point float64 sums (sum_fix.cu): -1 = not looked at for this tree,
-  // 0 = the box or the kernel's range does not fit, 1 = records are built
+  // float64 sums with fixed-point kernel values (sum_fix.cu): -1 = not looked at
+  // for this tree, 0 = the box or the kernel's range does not fit, 1 = records are
+  // built
   int fx_state = -1;
   int fx_F = 0;
   fx::Consts fx_c{};
   double h_lo0[kMaxDim] = {0}, h_hi0[kMaxDim] = {0};   // root box
-  DBuf<int> fx_pts, fx_nodes, fx_q, fx_qm;
-  DBuf<double> fx_qs, fx_qms;
+  DBuf<int> fx_pts, fx_nodes;
   DBuf<unsigned long long> fx_table;
-  DBuf<int> fx_flag;   // near field, couplings: sum in float64 (cleared by the scatter)
-  DBuf<unsigned long long> fx_colmax;   // [16] largest |x| of each column, as bits (cleared by the scatter)
-  DBuf<double> fx_colscale;             // [16]
   // symmetric form: row chunks of the upper near entries (batches of 64
   // sources per warp), built for the tree
   int fx_sym = -1, fx_batches = 0;
@@ -613,11 +587,8 @@ void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy
                    bool steady = false);
 void ensure_workspace(Plan& P, bool fp64);
 size_t farfield_smem_need(const Plan& P, bool fp64);
-// colmax: also the columns' largest magnitudes (float64 sums in fixed point;
-// the scatter of the same pass clears them); xq: also the float32 charges
-// interleaved, [leaf][m_pad][padded rows]
-void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64, bool colmax = false,
-                   float* xq = nullptr);
+// xq: also the float32 charges interleaved, [leaf][m_pad][padded rows]
+void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64, float* xq = nullptr);
 void launch_scatter(Plan& P, double* y, int64_t ldy, int r0, int Rc, bool fp64);
 void launch_farfield(Plan& P, int Rc, bool fp64, bool steady);
 bool farfield_tc_eligible(const Plan& P);   // farfield_tc.cu
@@ -637,7 +608,7 @@ int sm_count();
 bool row_chunks(Plan& P, int per, int least, RowChunks& out);   // p2p_rot.cu
 bool rot_ready(Plan& P, int Rc);
 void near_rot(Plan& P, int D, int Rc, cudaStream_t s);
-bool fix_ready(Plan& P);                    // sum_fix.cu: fixed-point float64 sums
+bool fix_ready(Plan& P);                    // sum_fix.cu: float64 sums with fixed-point kernel values
 bool near_fix(Plan& P, int Rc, cudaStream_t s);
 bool m2l_fix(Plan& P, int Rc);
 bool p2p_f32_tuned(Plan& P, int Rc, bool rot, bool steady, cudaStream_t s);

@@ -88,7 +88,7 @@ void evaluate(Plan& P, const double* tgt, int64_t nt, int64_t ldt, const double*
   }
   for (int r0 = 0; r0 < R; r0 += kRC) {
     const int Rc = std::min(kRC, R - r0);
-    launch_gather(P, c, ldc, r0, Rc, fp64, false, fp64 ? nullptr : P.xq32.p);
+    launch_gather(P, c, ldc, r0, Rc, fp64, fp64 ? nullptr : P.xq32.p);
     if (fp64) {
       eval_f64(P, P.ev_blk.p, G, P.ev_rows.p, P.ev_col.p, splits, stride, Rc, P.ev_out64.p, s);
       k_eval_out<double><<<ceil_div(nt * Rc, 256), 256, 0, s>>>(P.ev_out64.p, splits, stride, nt, m, r0, Rc, out, ldo);

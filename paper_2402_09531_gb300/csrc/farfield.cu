@@ -820,8 +820,7 @@ __global__ void __launch_bounds__(kPersistThreads, 3) k_batch_persistent(const _
 // same values interleaved, [leaf][m_pad][rows].
 template <typename T>
 __global__ void k_gather(const double* x, int64_t ldx, int r0, int Rc, int rows, const int32_t* perm,
-                         const int32_t* begin, const int32_t* count, int L, int m_pad, T* xb, T* xq,
-                         unsigned long long* colmax) {
+                         const int32_t* begin, const int32_t* count, int L, int m_pad, T* xb, T* xq) {
   const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const int64_t total = static_cast<int64_t>(L) * rows * m_pad;
   if (t >= total) return;
@@ -834,16 +833,6 @@ __global__ void k_gather(const double* x, int64_t ldx, int r0, int Rc, int rows,
   if (r < Rc && i < count[c]) v = static_cast<T>(x[static_cast<int64_t>(r0 + r) * ldx + perm[begin[c] + i]]);
   xb[(static_cast<int64_t>(leaf) * kRC + r) * m_pad + i] = v;
   if (xq) xq[(static_cast<int64_t>(leaf) * m_pad + i) * rows + r] = v;
-  if (colmax && r < Rc) {
-    // largest magnitude of each column; lanes of a warp may lie in two rows
-    const unsigned act = __activemask();
-    unsigned long long m = static_cast<unsigned long long>(__double_as_longlong(fabs(static_cast<double>(v))));
-    const unsigned same = __match_any_sync(act, r);
-    const unsigned hi = __reduce_max_sync(same, static_cast<unsigned>(m >> 32));
-    const unsigned lo = __reduce_max_sync(same, static_cast<unsigned>(m >> 32) == hi ? static_cast<unsigned>(m) : 0u);
-    m = (static_cast<unsigned long long>(hi) << 32) | lo;
-    if ((threadIdx.x & 31) == __ffs(same) - 1 && m > colmax[r]) atomicMax(colmax + r, m);
-  }
 }
 
 // Scatter of the symmetric near fields: y = the row's chunk sums and the
@@ -856,14 +845,9 @@ template <typename T>
 __global__ void __launch_bounds__(kPartThreads)
 k_scatter_parts(double* y, int64_t ldy, int r0, int Rc, const int32_t* perm, const int32_t* begin,
                 const int32_t* count, int L, int m_pad, int ldp, const int32_t* chunk_ptr, const int32_t* lorow,
-                const int32_t* lo_slot, const T* pf, const T* pt, const T* yfar, int has_far, int* flags,
-                unsigned long long* colmax) {
+                const int32_t* lo_slot, const T* pf, const T* pt, const T* yfar, int has_far) {
   __shared__ double part[kPartThreads];
   const int tid = static_cast<int>(threadIdx.x);
-  if (blockIdx.x == 0) {   // every sum that reads them is done
-    if (flags && tid < 2) flags[tid] = 0;
-    if (colmax && tid < kRC) colmax[tid] = 0;
-  }
   const int leaf = static_cast<int>(blockIdx.x) / Rc, r = static_cast<int>(blockIdx.x) % Rc;
   const int c = L - 1 + leaf;
   const int cnt = count[c];
@@ -885,11 +869,8 @@ k_scatter_parts(double* y, int64_t ldy, int r0, int Rc, const int32_t* perm, con
 template <typename T>
 __global__ void k_scatter(double* y, int64_t ldy, int r0, int Rc, const int32_t* perm,
                           const int32_t* begin, const int32_t* count, int L, int m_pad,
-                          const T* ynear, const T* yfar, int has_far, int* flags,
-                          unsigned long long* colmax) {
+                          const T* ynear, const T* yfar, int has_far) {
   const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (flags && t < 2) flags[t] = 0;   // every sum that reads them is done
-  if (colmax && t < kRC) colmax[t] = 0;
   const int64_t total = static_cast<int64_t>(L) * Rc * m_pad;
   if (t >= total) return;
   const int i = static_cast<int>(t % m_pad);
@@ -1011,16 +992,15 @@ size_t farfield_smem_need(const Plan& P, bool fp64) {
   return std::max(a, b);
 }
 
-void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64, bool colmax, float* xq) {
+void launch_gather(Plan& P, const double* x, int64_t ldx, int r0, int Rc, bool fp64, float* xq) {
   const int rows = fp64 ? Rc : sum_padded_rc(Rc);
   const int64_t total = static_cast<int64_t>(P.L) * rows * P.m_pad;
   if (fp64)
     k_gather<double><<<ceil_div(total, 256), 256, 0, P.stream>>>(x, ldx, r0, Rc, rows, P.d_perm.p, P.d_begin.p,
-                                                                 P.d_count.p, P.L, P.m_pad, P.xb64.p, nullptr,
-                                                                 colmax ? P.fx_colmax.p : nullptr);
+                                                                 P.d_count.p, P.L, P.m_pad, P.xb64.p, nullptr);
   else
     k_gather<float><<<ceil_div(total, 256), 256, 0, P.stream>>>(x, ldx, r0, Rc, rows, P.d_perm.p, P.d_begin.p,
-                                                                P.d_count.p, P.L, P.m_pad, P.xb32.p, xq, nullptr);
+                                                                P.d_count.p, P.L, P.m_pad, P.xb32.p, xq);
   DW_CUDA(cudaGetLastError());
 }
 
@@ -1031,17 +1011,17 @@ void launch_scatter(Plan& P, double* y, int64_t ldy, int r0, int Rc, bool fp64) 
   if (P.near_parts == 1)
     k_scatter_parts<double><<<P.L * Rc, kPartThreads, 0, P.stream>>>(
         y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad, P.m_pad, P.fx_rows.ptr.p, P.sym_lorow.p,
-        P.sym_loslot.p, P.sym_pf.p, P.sym_pt.p, P.yfar64.p, has_far, P.fx_flag.p, P.fx_colmax.p);
+        P.sym_loslot.p, P.sym_pf.p, P.sym_pt.p, P.yfar64.p, has_far);
   else if (P.near_parts == 2)
     k_scatter_parts<float><<<P.L * Rc, kPartThreads, 0, P.stream>>>(
         y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad, round_up(P.rot.cmax, 8), P.rot.ptr.p, P.sym_lorow.p,
-        P.sym_loslot.p, P.rot_pf.p, P.rot_pt.p, P.yfar32.p, has_far, nullptr, nullptr);
+        P.sym_loslot.p, P.rot_pf.p, P.rot_pt.p, P.yfar32.p, has_far);
   else if (fp64)
     k_scatter<double><<<grid, 256, 0, P.stream>>>(y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad,
-                                                  P.ynear64.p, P.yfar64.p, has_far, P.fx_flag.p, P.fx_colmax.p);
+                                                  P.ynear64.p, P.yfar64.p, has_far);
   else
     k_scatter<float><<<grid, 256, 0, P.stream>>>(y, ldy, r0, Rc, P.d_perm.p, P.d_begin.p, P.d_count.p, P.L, P.m_pad,
-                                                 P.ynear32.p, P.yfar32.p, has_far, nullptr, nullptr);
+                                                 P.ynear32.p, P.yfar32.p, has_far);
   DW_CUDA(cudaGetLastError());
 }
 

@@ -1,5 +1,6 @@
-// Kernel values phi(||x - s|| / sigma) in 64-bit fixed point: the float64
-// summation of the near field and of the couplings on the integer pipes.
+// Kernel values phi(||x - s|| / sigma) by 64-bit fixed point: the float64
+// summation of the near field and of the couplings takes them from the integer
+// pipes, and the float64 unit only adds up.
 //
 // GB300's float64 unit does 2 multiply-adds a clock on an SM; a 32 x 32 + 64
 // product runs at 32 lanes a clock, adds and logic at 64 to 128 (measured).  A
@@ -15,18 +16,18 @@
 // A pair's squared distance is the exact integer
 //   T = A 2^60 + B 2^31 + C,  A = sum dh^2, B = sum dh dl, C = sum dl^2,
 // one 32 x 32 + 64 product each (no carries: A < 2^58, |B| < 2^61, C < 2^64
-// for d <= 16).  Then w = log2 of 1 / exp(...) with 57 fraction bits (boxes up
-// to w = 2^5, about 22 length scales), 2^-w by two 256-entry tables and a
-// cubic, and phi with 56 fraction bits, rounded.
+// for d <= 16).  Then w = log2 of 1 / exp(...) with 57 fraction bits, w < 2^5,
+// 2^-w by two 256-entry tables and a cubic, and phi as a float64 with all of its
+// 53 bits however small it is.
 //
-// Error of phi against 113-bit arithmetic, in units of 2^-56, over random and
-// close pairs, d = 4..16, boxes of 0.001 to 20 length scales: at most 2.0, rms
-// 0.29 to 0.49; the float64 evaluation it stands in for: at most 22, rms 1.4
-// to 5.7.
+// w < 2^5 is asked of the diagonal rounded up to a power of two (make_consts):
+// a box's diagonal may be up to 11.1 to 22.2 length scales for the exponential,
+// 6.4 to 12.8 for Matern-3/2 and 3.3 to 6.7 for the Gaussian, depending on where
+// the diagonal lies between powers of two; larger boxes keep the float64 unit.
 //
-// Charges are split alike, q = (qh 2^28 + ql) 2^(e - 55) with 2^e above the
-// largest magnitude, and a term phi q is three products; 128 terms fit the
-// 64-bit sums.  Integer sums have no rounding and no order.
+// Relative error of phi against 64-bit-mantissa arithmetic, over random and
+// close pairs, d = 1..16, boxes of 1e-7 to 22 length scales, phi down to 2^-30:
+// at most 1.09 2^-53, of which 1 is the rounding of the result.
 #pragma once
 
 #include <cstdint>
@@ -129,12 +130,24 @@ __host__ __device__ __forceinline__ u64 exp2_neg(u64 W, const u64* table, int& k
   return p - (mulhi(p, m) >> 12);
 }
 
-// phi with 56 fraction bits, rounded, from T = A 2^60 + B 2^31 + C (pairs of
-// one tree: T < 2^118), for P independent pairs side by side: one chain of
-// dependent products is too long for the warps that fit.
+// m 2^e 2^-52 for m in [2^52, 2^53].
+__host__ __device__ __forceinline__ double from_bits(u64 m, int e) {
+  const u64 b = m + (static_cast<u64>(static_cast<uint32_t>(e + 1022)) << 52);   // m carries 1 into the exponent
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double(static_cast<s64>(b));
+#else
+  double v;
+  __builtin_memcpy(&v, &b, 8);
+  return v;
+#endif
+}
+
+// phi from T = A 2^60 + B 2^31 + C (pairs of one tree: T < 2^118), for P
+// independent pairs side by side: one chain of dependent products is too long
+// for the warps that fit.
 template <int KER, int P>
-__host__ __device__ __forceinline__ void phi56(const u64 (&A)[P], const s64 (&B)[P], const u64 (&C)[P], const Consts& c,
-                                               const u64* table, u64 (&out)[P]) {
+__host__ __device__ __forceinline__ void phi64(const u64 (&A)[P], const s64 (&B)[P], const u64 (&C)[P], const Consts& c,
+                                               const u64* table, double (&out)[P]) {
   u64 W[P];
   if (KER == DWFMM_K_GAUSS) {
     // T 2^-55 in 63 bits; + 1 because the two floors may add up to -1
@@ -190,12 +203,13 @@ __host__ __device__ __forceinline__ void phi56(const u64 (&A)[P], const s64 (&B)
     int k;
     u64 e = exp2_neg(W[q], table, k);
     if (KER == DWFMM_K_MATERN32) {
-      // (1 + t) e^-t, t = w ln 2
+      // (1 + t) e^-t, t = w ln 2, 1 + t < 2^5
       const u64 t = mulhi(W[q], 0xb17217f7d1cf79acull);                   // 2^-57 (W < 2^62: no carry either)
-      e = mulhi(e, t + t + ((1ull << 58) + 1)) >> k;                      // 2^-57
-      out[q] = (e + 1) >> 1;
+      e = mulhi(e, t + t + ((1ull << 58) + 1));                           // phi 2^k 2^57, in (2^56, 2^62)
+      const int s = clz32(hi32(e)) - 1;
+      out[q] = from_bits(((e << s) + 512) >> 10, 5 - s - k);
     } else {
-      out[q] = ((e >> k) + 64) >> 7;
+      out[q] = from_bits((e + 512) >> 10, -1 - k);                        // e in (2^62, 2^63]
     }
   }
 }
@@ -263,7 +277,7 @@ inline Big big_div(unsigned __int128 n, int en, double v) {
 }
 
 // Scale of w for a box whose diagonal is below 2^(59 - F); false when w may
-// reach 2^5 (a box beyond 22 length scales).
+// reach 2^5 at that bound.
 inline bool make_consts(int kernel, double sigma, int F, Consts& c) {
   typedef unsigned __int128 u128;
   const u128 log2e = (static_cast<u128>(0xb8aa3b295c17f0bbull) << 64) | 0xbe87fed0691d3e89ull;     // 2^-127

@@ -1,8 +1,6 @@
 // Kernel summation y_i = sum_j phi(||x_i - x_j|| / sigma) q_j of one target
 // group over its list of source groups, one thread per target, sources staged
-// through shared memory in chunks: the generic kernel (nearfield.cu) and the
-// float64 path of the fixed-point kernels (sum_fix.cuh) for charges that are
-// not finite.
+// through shared memory in chunks (the generic kernel, nearfield.cu).
 #pragma once
 
 #include "dwfmm_internal.cuh"
@@ -12,6 +10,15 @@ namespace ks {
 
 constexpr int kThreads = 128;
 constexpr int kSrcChunk = 128;
+
+// Rows of one side of a sum.
+struct Side {
+  int64_t gstride;   // elements between groups
+  int ld;            // elements between coordinate rows (or rhs rows)
+  const int32_t* count;
+  int count_off;
+  int count_const;   // used when count == nullptr
+};
 
 template <typename T, int KER>
 __device__ __forceinline__ T phi_r2(T r2, T inv_sigma) {

@@ -66,7 +66,7 @@ void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy
                    bool steady) {
   if (P.N == 0 || R == 0) return;
   ensure_workspace(P, fp64);
-  const bool fix = fp64 && !steady && fix_ready(P);   // the tree's records, before the side stream forks
+  if (fp64 && !steady) (void)fix_ready(P);   // the tree's records, before the side stream forks
   cudaStream_t s = P.stream;
   timer_begin(P, 6, s);
   for (int r0 = 0; r0 < R; r0 += kRC) {
@@ -75,7 +75,7 @@ void matvec_device(Plan& P, const double* x, int64_t ldx, double* y, int64_t ldy
     P.near_parts = 0;
     // the symmetric tensor-core near field reads the row layout
     const bool xq = !fp64 && !(P.prec == DWFMM_P_MIXED && sum_padded_rc(Rc) == 16);
-    launch_gather(P, x, ldx, r0, Rc, fp64, fix, xq ? P.xq32.p : nullptr);
+    launch_gather(P, x, ldx, r0, Rc, fp64, xq ? P.xq32.p : nullptr);
     timer_end(P, 0, s, 1);
     const bool rot = !fp64 && !steady && rot_ready(P, Rc);
     if (!fp64) m2l_autotune(P, Rc);   // once per tree, before the near field starts

@@ -8,8 +8,9 @@
 // One CTA per target group, one thread per target, sources staged through
 // shared memory in chunks.  This generic kernel serves the fallback float32
 // shapes (the tuned float32 P2P lives in p2p_f32.cu) and the float64 sums that
-// the fixed-point kernels (sum_fix.cu) do not take: d > 16, boxes beyond about
-// 22 length scales.
+// the kernels with fixed-point values (sum_fix.cu) do not take: d > 16, boxes too
+// large for their length scale (fix64.cuh), evaluation at new points, and the
+// iterations of the incremental conjugate gradients.
 //
 // The float64 P2P has a symmetric form as well: phi is symmetric and so is
 // the near relation, so each unordered pair of near leaves (T, S) is

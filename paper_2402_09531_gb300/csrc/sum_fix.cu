@@ -1,6 +1,5 @@
-// Float64 near field and couplings in fixed point: the tree's records, the
-// charges' limbs, and the launches (kernels in sum_fix.cuh, format in
-// fix64.cuh).
+// Float64 near field and couplings with fixed-point kernel values: the tree's
+// records and the launches (kernels in sum_fix.cuh, format in fix64.cuh).
 #include <algorithm>
 #include <cmath>
 
@@ -28,58 +27,6 @@ __global__ void k_fix_records(const double* pts, int64_t groups, int d, int DM, 
     v = make_int2(static_cast<int>(u >> 30), static_cast<int>(u & 0x3fffffff));
   }
   rec[t] = v;
-}
-
-// Limbs [group][ld][RC] and scales [group][16] of charges [group][16][ld]
-// (rows below Rc; the others are zero): q = (qh 2^28 + ql) 2^(e - 55) with
-// |q| < 2^e over the group's row, or (colmax given: the column's largest
-// magnitude, as bits) over the column, whose scale goes to colscale too.  One
-// warp per group and row; a value outside what the format takes raises *flag.
-__global__ void k_fix_charges(const double* rows, int first, int groups, int ld, int Rc, int RC, const u64* colmax,
-                              int2* q, double* scale, double* colscale, int* flag) {
-  const int w = static_cast<int>((static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (w >= groups * RC) return;
-  const int g = first + w / RC, r = w % RC;
-  int2* qo = q + static_cast<int64_t>(g) * ld * RC + r;
-  if (r >= Rc) {
-    for (int i = lane; i < ld; i += 32) qo[static_cast<int64_t>(i) * RC] = make_int2(0, 0);
-    if (lane == 0) {
-      scale[static_cast<int64_t>(g) * kRC + r] = 0.0;
-      if (colmax && w < RC) colscale[r] = 0.0;
-    }
-    return;
-  }
-  const double* x = rows + (static_cast<int64_t>(g) * kRC + r) * ld;
-  u64 top = 0;   // magnitudes order like their bits, infinities and NaN above all
-  if (colmax) {
-    top = colmax[r];
-  } else {
-    for (int i = lane; i < ld; i += 32) {
-      const u64 v = static_cast<u64>(__double_as_longlong(fabs(x[i])));
-      top = v > top ? v : top;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const u64 v = __shfl_xor_sync(0xffffffffu, top, o);
-      top = v > top ? v : top;
-    }
-  }
-  const double mx = __longlong_as_double(static_cast<s64>(top));
-  // not finite, or so small that the scale would lose bits below the normal range
-  if (top >= 0x7ff0000000000000ull || (mx > 0.0 && mx < 0x1p-960)) {
-    if (lane == 0) atomicExch(flag, 1);
-    return;
-  }
-  const int e = mx > 0.0 ? ilogb(mx) + 1 : 0;
-  for (int i = lane; i < ld; i += 32) {
-    const s64 v = static_cast<s64>(to_units(x[i], 55 - e));
-    const s64 h = (v + (1ll << 27)) >> 28;
-    qo[static_cast<int64_t>(i) * RC] = make_int2(static_cast<int>(h), static_cast<int>(v - (h << 28)));
-  }
-  if (lane == 0) {
-    scale[static_cast<int64_t>(g) * kRC + r] = ldexp(1.0, e - 55);
-    if (colmax && w < RC) colscale[r] = ldexp(1.0, e - 55);
-  }
 }
 
 // out[g][r][i] = sum over parts of part[p][g][r][i] in part order (r < Rc).
@@ -129,9 +76,9 @@ void shape(FixArgs& a, int n) {
 
 // Chunks of the upper rows for the symmetric form; false when it does not
 // apply: leaves below a warp's width (the lanes of a turn would share a
-// target) or above 128 sites (128 terms fit the sums), or a list that is not
-// symmetric.  Up to 4 right-hand sides it is the faster form (1: 5.8 against
-// 10.3 ms at N = 65536, d = 8; 4: 7.7 against 12.1 ms); 16 would need their
+// target) or above 128 slots (twice the shared memory, half the CTAs of an SM), or a
+// list that is not symmetric.  Up to 4 right-hand sides it is the faster form (1: 5.2 against
+// 9.8 ms at N = 65536, d = 8; 4: 7.1 against 11.3 ms); 16 would need their
 // sums for both sides in registers.
 bool sym_ready(Plan& P) {
   if (P.fx_sym >= 0) return P.fx_sym == 1;
@@ -173,19 +120,6 @@ bool fix_ready(Plan& P) {
   const int64_t nl = static_cast<int64_t>(P.L) * P.m_pad, nc = static_cast<int64_t>(P.C) * P.n_pad;
   P.fx_pts.alloc(nl * 2 * DM);
   P.fx_nodes.alloc(nc * 2 * DM);
-  P.fx_q.alloc(nl * 2 * kRC);
-  P.fx_qm.alloc(nc * 2 * kRC);
-  P.fx_qs.alloc(static_cast<size_t>(P.L) * kRC);
-  P.fx_qms.alloc(static_cast<size_t>(P.C) * kRC);
-  if (!P.fx_flag.p) {
-    P.fx_flag.alloc(2);
-    DW_CUDA(cudaMemsetAsync(P.fx_flag.p, 0, 2 * sizeof(int), P.stream));
-  }
-  if (!P.fx_colmax.p) {
-    P.fx_colmax.alloc(kRC);
-    P.fx_colscale.alloc(kRC);
-    DW_CUDA(cudaMemsetAsync(P.fx_colmax.p, 0, kRC * sizeof(fx::u64), P.stream));
-  }
   if (!P.fx_table.p) {
     fx::u64 t[fx::kTable];
     fx::make_table(t);
@@ -206,9 +140,6 @@ bool near_fix(Plan& P, int Rc, cudaStream_t s) {
   P.near_parts = 0;
   if (P.fx_state != 1) return false;
   const int RC = padded_r(Rc);
-  k_fix_charges<<<ceil_div(static_cast<int64_t>(P.L) * RC * 32, 128), 128, 0, s>>>(
-      P.xb64.p, 0, P.L, P.m_pad, Rc, RC, P.fx_colmax.p, reinterpret_cast<int2*>(P.fx_q.p), P.fx_qs.p, P.fx_colscale.p,
-      P.fx_flag.p);
   size_t most = 0;   // columns of partial sums
   if (P.fx_sym == 1 && RC <= 4)
     most = kSymMaxBytes / ((static_cast<size_t>(P.fx_rows.n) + P.sym_nup) * P.m_pad * sizeof(double));
@@ -218,8 +149,7 @@ bool near_fix(Plan& P, int Rc, cudaStream_t s) {
     P.grow(P.sym_pt, P.sym_nup * cols * P.m_pad);
     FixSymArgs b{};
     b.rec = reinterpret_cast<const int4*>(P.fx_pts.p);
-    b.q = reinterpret_cast<const int2*>(P.fx_q.p);
-    b.qscale = P.fx_colscale.p;
+    b.charge = P.xb64.p;
     b.table = P.fx_table.p;
     b.c = P.fx_c;
     b.count = P.d_count.p + P.L - 1;
@@ -233,11 +163,6 @@ bool near_fix(Plan& P, int Rc, cudaStream_t s) {
     b.batches = P.fx_batches;
     b.pf = P.sym_pf.p;
     b.pt = P.sym_pt.p;
-    b.flag = P.fx_flag.p;
-    b.d = P.d;
-    b.inv_sigma = 1.0 / P.sigma;
-    b.coord = P.d_pts64.p;
-    b.charge = P.xb64.p;
     dispatch_sym(P.kernel, P.d, RC, b, P.fx_rows.n, s);
     P.near_parts = 1;
     P.near_engine = 1;
@@ -246,22 +171,17 @@ bool near_fix(Plan& P, int Rc, cudaStream_t s) {
   P.near_engine = 0;
   FixArgs a{};
   a.rec = reinterpret_cast<const int4*>(P.fx_pts.p);
-  a.q = reinterpret_cast<const int2*>(P.fx_q.p);
-  a.qscale = P.fx_qs.p;
   a.table = P.fx_table.p;
   a.c = P.fx_c;
   a.rowptr = P.d_near_rowptr.p;
   a.col = P.d_near_col.p;
   a.ld = P.m_pad;
   a.Rc = Rc;
-  a.d = P.d;
-  a.inv_sigma = 1.0 / P.sigma;
-  a.coord = P.d_pts64.p;
-  a.side = ks::Side{static_cast<int64_t>(P.d) * P.m_pad, P.m_pad, P.d_count.p, P.L - 1, 0};
+  a.count = P.d_count.p;
+  a.count_off = P.L - 1;
   a.charge = P.xb64.p;
   a.q_gstride = static_cast<int64_t>(kRC) * P.m_pad;
   a.o_gstride = a.q_gstride;
-  a.flag = P.fx_flag.p;
   int cmax = 1;
   for (int l = 0; l < P.L; ++l) cmax = std::max(cmax, P.h_count[P.L - 1 + l]);
   shape(a, cmax);
@@ -289,12 +209,8 @@ bool m2l_fix(Plan& P, int Rc) {
   if (P.fx_state != 1) return false;
   const int RC = padded_r(Rc);
   const int first = (1 << P.jmin) - 1, groups = P.C - first;
-  k_fix_charges<<<ceil_div(static_cast<int64_t>(groups) * RC * 32, 128), 128, 0, P.stream>>>(
-      P.mom64.p, first, groups, P.n_pad, Rc, RC, nullptr, reinterpret_cast<int2*>(P.fx_qm.p), P.fx_qms.p, nullptr, P.fx_flag.p + 1);
   FixArgs a{};
   a.rec = reinterpret_cast<const int4*>(P.fx_nodes.p);
-  a.q = reinterpret_cast<const int2*>(P.fx_qm.p);
-  a.qscale = P.fx_qms.p;
   a.table = P.fx_table.p;
   a.c = P.fx_c;
   a.rowptr = P.d_far_rowptr.p;
@@ -302,16 +218,12 @@ bool m2l_fix(Plan& P, int Rc) {
   a.first = first;
   a.ld = P.n_pad;
   a.Rc = Rc;
-  a.d = P.d;
-  a.inv_sigma = 1.0 / P.sigma;
-  a.coord = P.d_ynode64.p;
-  a.side = ks::Side{static_cast<int64_t>(P.d) * P.n_pad, P.n_pad, nullptr, 0, P.n};
+  a.count_const = P.n;
   a.charge = P.mom64.p;
   a.q_gstride = static_cast<int64_t>(kRC) * P.n_pad;
   a.o_gstride = a.q_gstride;
   a.out = P.loc64.p;
   a.splits = 1;
-  a.flag = P.fx_flag.p + 1;
   shape(a, P.n);
   // node sets small enough for four threads a target: whole sets per thread
   const int cap = RC > 4 ? 64 : 128;

@@ -1,42 +1,42 @@
-// Float64 kernel summation in fixed point (fix64.cuh), one translation unit
-// per kernel function (sum_fix_exp.cu, sum_fix_matern.cu, sum_fix_gauss.cu).
+// Float64 kernel summation with kernel values from the integer pipes
+// (fix64.cuh), one translation unit per kernel function (sum_fix_exp.cu,
+// sum_fix_matern.cu, sum_fix_gauss.cu).  Charges and sums are float64.
 //
 // k_fix_sum: one CTA per (target group, pass of up to 128 targets, part of the
 // list).  A thread owns one target; groups of at most 64 targets are shared by
 // several threads, which take every nsub-th source (or, for short source
-// groups, every nsub-th group).  Sources and charges are contiguous records in
-// HBM and come in by cp.async one stage ahead.  Bound by the wide products
-// (32 lanes a clock on an SM).  d = 10 Gaussian near field, N = 12289, 16
-// right-hand sides: 29.7 -> 3.1 ms; couplings of the d = 8 Matern tree at
-// N = 262144 (10 nodes a cluster): 26.7 -> 0.33 ms (a float64 warp there had
-// 10 of its 32 lanes at work).
+// groups, every nsub-th group).  Sources and charges are rows in HBM and come
+// in by cp.async one stage ahead.  Bound by the wide products (32 lanes a clock
+// on an SM) for a few right-hand sides, beyond that by the float64 unit's 2
+// multiply-adds a clock, one for each pair and side; the two share an issue port
+// (32 multiply-adds alone take a warp 512 clocks, 116 products 58, both 610).
+// d = 10 Gaussian, N = 12289, 16 right-hand sides, the whole product: 34.6 ms with
+// kernel values from the float64 unit, 5.0 ms; its 2.4e9 multiply-adds take 4.1.
+// Charges and sums in fixed point would take 3.2 ms there, but keep a term only to
+// 2^-55 of the largest one, not of itself.
 #pragma once
 
 #include <atomic>
 #include <type_traits>
 
 #include "fix64.cuh"
-#include "ksum.cuh"
 
 namespace dw {
 namespace fx {
 
-constexpr int kThreads = ks::kThreads;
+constexpr int kThreads = 128;
+constexpr int kFoldStages = 4;   // stages summed before the running sums take them
 
 template <int RC>
 constexpr int stage_cap() { return RC > 4 ? 64 : 128; }
 
-// Records: 2 * DM ints per point (limb pairs, zero beyond d); charges: RC
-// limb pairs per point.  pts_stage * DM: see fix_smem.
+// Table, two stages of records (2 DM ints per point: limb pairs, zero beyond
+// d) and charges (RC rows), running sums of RC rows.
 template <int DM, int RC>
 constexpr size_t fix_smem() {
-  return kTable * sizeof(u64) + 2 * static_cast<size_t>(stage_cap<RC>()) * (2 * DM + 2 * RC) * sizeof(int) +
+  return kTable * sizeof(u64) + 2 * static_cast<size_t>(stage_cap<RC>()) * (2 * DM * sizeof(int) + RC * sizeof(double)) +
          (RC > 4 ? static_cast<size_t>(RC) * kThreads * sizeof(double) : 0);
 }
-
-struct Limbs {
-  int h, l;
-};
 
 __device__ __forceinline__ void cp16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
@@ -56,7 +56,7 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;
 // phi of one target (limbs x) and P source records, `stride` int4 apart.
 template <int KER, int DM, int P>
 __device__ __forceinline__ void pair_phi(const int (&xh)[DM], const int (&xl)[DM], const int4* rec, int stride,
-                                         const Consts& c, const u64* table, u64 (&out)[P]) {
+                                         const Consts& c, const u64* table, double (&out)[P]) {
   u64 A[P], C[P];
   s64 B[P];
 #pragma unroll
@@ -75,22 +75,7 @@ __device__ __forceinline__ void pair_phi(const int (&xh)[DM], const int (&xl)[DM
       C[q] += static_cast<u64>(static_cast<s64>(l1) * l1);
     }
   }
-  phi56<KER, P>(A, B, C, c, table, out);
-}
-
-// (hh, m) += phi q: hh counts 2^(e - 55), m 2^(e - 83); the product of the two
-// low limbs (below 2^(e - 57), signed) is left out.
-__device__ __forceinline__ void mac(u64 p, int qh, int ql, s64& hh, s64& m) {
-  const int ph = static_cast<int>(p >> 28), pl = static_cast<int>(p) & 0xfffffff;
-  hh += static_cast<s64>(ph) * qh;
-  m += static_cast<s64>(ph) * ql;
-  m += static_cast<s64>(pl) * qh;
-}
-
-__device__ __forceinline__ double flush(s64& hh, s64& m, double scale, double acc) {
-  const s64 v = hh + ((m + (1ll << 27)) >> 28);
-  hh = m = 0;
-  return fma(static_cast<double>(v), scale, acc);
+  phi64<KER, P>(A, B, C, c, table, out);
 }
 
 template <int KER, int DM, int RC>
@@ -100,8 +85,8 @@ __global__ void __launch_bounds__(kThreads, RC > 4 ? 3 : 4) k_fix_sum(const FixA
   extern __shared__ __align__(16) unsigned char smem[];
   u64* table = reinterpret_cast<u64*>(smem);
   int4* srec = reinterpret_cast<int4*>(smem + kTable * sizeof(u64));   // [2][CAP][RV]
-  int2* sq = reinterpret_cast<int2*>(srec + 2 * CAP * RV);             // [2][CAP][RC]
-  double* sacc = reinterpret_cast<double*>(sq + 2 * CAP * RC);         // [RC][kThreads] if RC > 4
+  double* sq = reinterpret_cast<double*>(srec + 2 * CAP * RV);         // [2][RC][CAP]
+  double* sacc = sq + 2 * CAP * RC;                                    // [RC][kThreads] if RC > 4
 
   const int part = static_cast<int>(blockIdx.x) % a.splits;
   const int gp = static_cast<int>(blockIdx.x) / a.splits;
@@ -113,14 +98,6 @@ __global__ void __launch_bounds__(kThreads, RC > 4 ? 3 : 4) k_fix_sum(const FixA
   const int t0 = pass * a.tp;
   const int t_end = min(a.ld, t0 + a.tp);
   double* out = a.out + part * a.split_stride + g * a.o_gstride;
-
-  if (*a.flag) {   // a charge the format does not take (not finite, below 2^-960): float64
-    double* sc = reinterpret_cast<double*>(smem);
-    ks::ksum_targets<double, KER, DM, RC>(g, t0 + static_cast<int>(threadIdx.x), t_end, rb, re, a.col, a.d, a.inv_sigma,
-                                          a.coord, a.side, a.coord, a.side, a.charge, a.q_gstride, a.ld, out, a.ld,
-                                          a.Rc, sc, sc + DM * ks::kSrcChunk);
-    return;
-  }
 
   for (int i = threadIdx.x; i < kTable; i += kThreads) table[i] = a.table[i];
   const int sub = static_cast<int>(threadIdx.x) / a.tp;
@@ -138,73 +115,84 @@ __global__ void __launch_bounds__(kThreads, RC > 4 ? 3 : 4) k_fix_sum(const FixA
       xl[k + 1] = v.w;
     }
   }
-  s64 hh[RC], mm[RC];
-  double acc[RC > 4 ? 1 : RC];
+  // sums of a few stages, and the running sums that take them: many short sums
+  // lose less than a long one, and what is added to the running sums is little
+  double acc[RC], tot[RC > 4 ? 1 : RC];
 #pragma unroll
-  for (int r = 0; r < RC; ++r) hh[r] = mm[r] = 0;
+  for (int r = 0; r < RC; ++r) acc[r] = 0.0;
   if constexpr (RC > 4) {
 #pragma unroll
     for (int r = 0; r < RC; ++r) sacc[r * kThreads + threadIdx.x] = 0.0;
   } else {
 #pragma unroll
-    for (int r = 0; r < RC; ++r) acc[r] = 0.0;
+    for (int r = 0; r < RC; ++r) tot[r] = 0.0;
   }
-
-  // sources j and (if P = 2) j + dj of the buffer
-  auto term = [&](auto np, int buf, int j, int dj) {
-    constexpr int P = decltype(np)::value;
-    u64 p[P];
-    pair_phi<KER, DM, P>(xh, xl, srec + (buf * CAP + j) * RV, dj * RV, a.c, table, p);
-#pragma unroll
-    for (int u = 0; u < P; ++u) {
-      const int2* q = sq + (buf * CAP + j + u * dj) * RC;
-      if constexpr (RC == 1) {
-        const int2 v = q[0];
-        mac(p[u], v.x, v.y, hh[0], mm[0]);
-      } else {
-#pragma unroll
-        for (int r = 0; r < RC; r += 2) {
-          const int4 v = *reinterpret_cast<const int4*>(q + r);
-          mac(p[u], v.x, v.y, hh[r], mm[r]);
-          mac(p[u], v.z, v.w, hh[r + 1], mm[r + 1]);
-        }
-      }
-    }
-  };
-  auto terms = [&](int buf, int j0, int dj, int j1) {
-    int j = j0;
-    for (; j + dj < j1; j += 2 * dj) term(std::integral_constant<int, 2>{}, buf, j, dj);
-    if (j < j1) term(std::integral_constant<int, 1>{}, buf, j, dj);
-  };
-  auto flush_all = [&](int s) {
-    const double* sc = a.qscale + static_cast<int64_t>(s) * kRC;
+  int staged = 0;
+  auto fold = [&]() {
 #pragma unroll
     for (int r = 0; r < RC; ++r) {
-      if constexpr (RC > 4) {
-        double* p = sacc + r * kThreads + threadIdx.x;
-        *p = flush(hh[r], mm[r], sc[r], *p);
-      } else {
-        acc[r] = flush(hh[r], mm[r], sc[r], acc[r]);
-      }
+      if (r >= a.Rc) break;
+      if constexpr (RC > 4) sacc[r * kThreads + threadIdx.x] += acc[r];
+      else tot[r] += acc[r];
+      acc[r] = 0.0;
     }
   };
-  // cn slots of source group s from slot cb into buffer slots at `at`
-  auto load = [&](int buf, int at, int s, int cb, int cn) {
-    const int4* rsrc = a.rec + (static_cast<int64_t>(s) * a.ld + cb) * RV;
-    int4* rdst = srec + (buf * CAP + at) * RV;
-    for (int k = threadIdx.x; k < cn * RV; k += kThreads) cp16(rdst + k, rsrc + k);
-    const int2* qsrc = a.q + (static_cast<int64_t>(s) * a.ld + cb) * RC;
-    int2* qdst = sq + (buf * CAP + at) * RC;
-    if constexpr (RC == 1) {
-      for (int k = threadIdx.x; k < cn; k += kThreads) cp8(qdst + k, qsrc + k);
-    } else {
-      for (int k = threadIdx.x; k < cn * (RC / 2); k += kThreads) cp16(qdst + 2 * k, qsrc + 2 * k);
+
+  // P sources j, j + dj, ... of the buffer: kernel values, and their products
+  // (columns in eights, then fours, then twos up to Rc: the branches are between
+  // blocks that the compiler can interleave with the integer work)
+  auto values = [&](auto& p, int buf, int j, int dj) {
+    constexpr int P = sizeof(p) / sizeof(double);
+    pair_phi<KER, DM, P>(xh, xl, srec + (buf * CAP + j) * RV, dj * RV, a.c, table, p);
+  };
+  auto add = [&](const auto& p, int buf, int j, int dj) {
+    constexpr int P = sizeof(p) / sizeof(double);
+    const double* q = sq + buf * CAP * RC + j;
+#pragma unroll
+    for (int r = 0; r < RC; ++r) {
+      if ((r == 2 || r == 8 || r == 12) && r >= a.Rc) break;
+#pragma unroll
+      for (int u = 0; u < P; ++u) acc[r] = fma(p[u], q[r * CAP + u * dj], acc[r]);
     }
+  };
+  // two sources at a time, the next two's values on the integer pipes while the
+  // float64 unit adds the last two's
+  auto terms = [&](int buf, int j0, int dj, int j1) {
+    int j = j0;
+    if (j + dj < j1) {
+      double p[2], pn[2];
+      values(p, buf, j, dj);
+      for (j += 2 * dj; j + dj < j1; j += 2 * dj) {
+        values(pn, buf, j, dj);
+        add(p, buf, j - 2 * dj, dj);
+        p[0] = pn[0];
+        p[1] = pn[1];
+      }
+      add(p, buf, j - 2 * dj, dj);
+    }
+    if (j < j1) {
+      double p[1];
+      values(p, buf, j, dj);
+      add(p, buf, j, dj);
+    }
+  };
+  // cn slots of source group s from slot cb (rows are multiples of 8 slots)
+  auto load = [&](int buf, int s, int cb, int cn) {
+    const int4* rsrc = a.rec + (static_cast<int64_t>(s) * a.ld + cb) * RV;
+    int4* rdst = srec + buf * CAP * RV;
+    for (int k = threadIdx.x; k < cn * RV; k += kThreads) cp16(rdst + k, rsrc + k);
+    const double* qsrc = a.charge + s * a.q_gstride + cb;
+    double* qdst = sq + buf * CAP * RC;
+    for (int k = threadIdx.x; k < a.Rc * (CAP / 2); k += kThreads) {
+      const int r = k / (CAP / 2), j = k % (CAP / 2) * 2;
+      if (j < cn) cp16(qdst + r * CAP + j, qsrc + static_cast<int64_t>(r) * a.ld + j);
+    }
+    cp_commit();
   };
 
   if (a.group_entries > 0) {
     // short source groups (one size): group_entries of them a stage
-    const int n = a.side.count_const;
+    const int n = a.count_const;
     const int ge = a.group_entries;
     auto load_entries = [&](int buf, int e) {
       const int ne = min(ge, re - e);
@@ -213,10 +201,11 @@ __global__ void __launch_bounds__(kThreads, RC > 4 ? 3 : 4) k_fix_sum(const FixA
         const int en = k / per;
         cp16(srec + buf * CAP * RV + k, a.rec + static_cast<int64_t>(a.col[e + en]) * a.ld * RV + (k - en * per));
       }
-      const int perq = n * RC;
-      for (int k = threadIdx.x; k < ne * perq; k += kThreads) {
-        const int en = k / perq;
-        cp8(sq + buf * CAP * RC + k, a.q + static_cast<int64_t>(a.col[e + en]) * a.ld * RC + (k - en * perq));
+      if (static_cast<int>(threadIdx.x) < ne * n) {   // at most CAP slots
+        const int en = static_cast<int>(threadIdx.x) / n;
+        const double* qsrc = a.charge + a.col[e + en] * a.q_gstride + (static_cast<int>(threadIdx.x) - en * n);
+        double* qdst = sq + buf * CAP * RC + threadIdx.x;
+        for (int r = 0; r < a.Rc; ++r) cp8(qdst + r * CAP, qsrc + static_cast<int64_t>(r) * a.ld);
       }
       cp_commit();
     };
@@ -227,23 +216,15 @@ __global__ void __launch_bounds__(kThreads, RC > 4 ? 3 : 4) k_fix_sum(const FixA
       __syncthreads();
       if (e + ge < re) load_entries(buf ^ 1, e + ge);
       const int ne = min(ge, re - e);
-      for (int en = on ? sub : ne; en < ne; en += a.nsub) {
-        terms(buf, en * n, 1, en * n + n);
-        flush_all(a.col[e + en]);
-      }
+      for (int en = on ? sub : ne; en < ne; en += a.nsub) terms(buf, en * n, 1, en * n + n);
+      if (++staged % kFoldStages == 0) fold();
     }
   } else {
     int e = rb, cb = 0, buf = 0;
-    auto count = [&](int en) {
-      return a.side.count ? a.side.count[a.side.count_off + a.col[en]] : a.side.count_const;
-    };
+    auto count = [&](int en) { return a.count ? a.count[a.count_off + a.col[en]] : a.count_const; };
     int cnt = e < re ? count(e) : 0;
-    if (e < re) {
-      load(0, 0, a.col[e], 0, min(CAP, cnt));
-      cp_commit();
-    }
+    if (e < re) load(0, a.col[e], 0, min(CAP, cnt));
     while (e < re) {
-      const int s = a.col[e];
       const int cn = min(CAP, cnt - cb);
       int ne = e, ncb = cb + CAP, ncnt = cnt;
       if (ncb >= cnt) {
@@ -252,20 +233,16 @@ __global__ void __launch_bounds__(kThreads, RC > 4 ? 3 : 4) k_fix_sum(const FixA
       }
       cp_wait_all();
       __syncthreads();
-      if (ne < re) {
-        load(buf ^ 1, 0, a.col[ne], ncb, min(CAP, ncnt - ncb));
-        cp_commit();
-      }
-      if (on) {
-        terms(buf, sub, a.nsub, cn);
-        flush_all(s);
-      }
+      if (ne < re) load(buf ^ 1, a.col[ne], ncb, min(CAP, ncnt - ncb));
+      if (on) terms(buf, sub, a.nsub, cn);
+      if (++staged % kFoldStages == 0) fold();
       e = ne;
       cb = ncb;
       cnt = ncnt;
       buf ^= 1;
     }
   }
+  fold();
 
   if constexpr (RC > 4) {
     if (a.nsub > 1) __syncthreads();
@@ -274,7 +251,7 @@ __global__ void __launch_bounds__(kThreads, RC > 4 ? 3 : 4) k_fix_sum(const FixA
       __syncthreads();
       double* red = reinterpret_cast<double*>(srec);
 #pragma unroll
-      for (int r = 0; r < RC; ++r) red[r * kThreads + threadIdx.x] = acc[r];
+      for (int r = 0; r < RC; ++r) red[r * kThreads + threadIdx.x] = tot[r];
       sacc = red;
       __syncthreads();
     }
@@ -288,7 +265,7 @@ __global__ void __launch_bounds__(kThreads, RC > 4 ? 3 : 4) k_fix_sum(const FixA
       v = sacc[r * kThreads + threadIdx.x];
       for (int u = 1; u < a.nsub; ++u) v += sacc[r * kThreads + threadIdx.x + u * a.tp];
     } else {
-      v = acc[RC > 4 ? 0 : r];
+      v = tot[RC > 4 ? 0 : r];
     }
     out[static_cast<int64_t>(r) * a.ld + i] = v;
   }
@@ -302,15 +279,16 @@ __global__ void __launch_bounds__(kThreads, RC > 4 ? 3 : 4) k_fix_sum(const FixA
 // differ and each adds to its target's sum in shared memory without atomics,
 // while the sources' sums stay in registers.  No lane idles on a ragged leaf:
 // the turn takes exactly T's size, and the sources are a stream.  Bound by the
-// wide products.  d = 8 Matern, 1 right-hand side, N = 262144: 412 ms (float64,
-// each pair once) -> 48 ms; N = 65536: 10.3 ms with k_fix_sum, 5.8 ms here.
+// wide products, beyond 2 right-hand sides with the float64 unit close behind.
+// d = 8 Matern, 1 right-hand side, N = 262144, the whole product: 440 ms with kernel
+// values from the float64 unit (each pair once, too) -> 43.2 ms.
 template <int DM>
 constexpr int sym_stride() { return DM == 10 ? 20 : 2 * DM + 4; }   // ints, 4 mod 8: no bank conflicts
 
 template <int DM, int RC>
 constexpr size_t fix_sym_smem(int ld) {
-  return kTable * sizeof(u64) + static_cast<size_t>(ld) * (sym_stride<DM>() + 2 * RC) * sizeof(int) +
-         static_cast<size_t>(kThreads / 32) * RC * ld * (2 * sizeof(s64) + sizeof(double));
+  return kTable * sizeof(u64) + static_cast<size_t>(ld) * sym_stride<DM>() * sizeof(int) +
+         static_cast<size_t>(1 + kThreads / 32) * RC * ld * sizeof(double);
 }
 
 template <int KER, int DM, int RC>
@@ -319,10 +297,9 @@ __global__ void __launch_bounds__(kThreads) k_fix_sym(const FixSymArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int ld = a.ld;
   u64* table = reinterpret_cast<u64*>(smem);
-  longlong2* facc = reinterpret_cast<longlong2*>(table + kTable);      // [NW][RC][ld] (hh, m)
-  double* dacc = reinterpret_cast<double*>(facc + NW * RC * ld);       // [NW][RC][ld]
-  int* trec = reinterpret_cast<int*>(dacc + NW * RC * ld);             // [ld][TS]
-  int* tq = trec + ld * TS;                                            // [ld][2 RC]
+  double* facc = reinterpret_cast<double*>(table + kTable);            // [NW][RC][ld]
+  double* tq = facc + NW * RC * ld;                                    // [RC][ld]
+  int* trec = reinterpret_cast<int*>(tq + RC * ld);                    // [ld][TS]
   const int chunk = blockIdx.x;
   const int T = a.chunk_t[chunk];
   const int c = a.count[T];
@@ -330,69 +307,20 @@ __global__ void __launch_bounds__(kThreads) k_fix_sym(const FixSymArgs a) {
   const int warp = static_cast<int>(threadIdx.x) >> 5, lane = static_cast<int>(threadIdx.x) & 31;
   const int per = NW * 64 * a.batches;                                 // sources per chunk
   const int first = (chunk - a.chunk_ptr[T]) * per;
-  double* pf = a.pf + static_cast<int64_t>(chunk) * a.Rc * ld;
-
-  if (*a.flag) {   // a charge the format does not take (not finite, below 2^-960): float64
-    auto phi = [&](int g, int i, int h, int j) {
-      double r2 = 0.0;
-      for (int k = 0; k < a.d; ++k) {
-        const double df = a.coord[(static_cast<int64_t>(g) * a.d + k) * ld + i] -
-                          a.coord[(static_cast<int64_t>(h) * a.d + k) * ld + j];
-        r2 += df * df;
-      }
-      return ks::phi_r2<double, KER>(r2, a.inv_sigma);
-    };
-    const int last = min(first + per, ne * a.cmax);
-    for (int i = threadIdx.x; i < c; i += kThreads)
-      for (int r = 0; r < a.Rc; ++r) {
-        double v = 0.0;
-        for (int j = first; j < last; ++j) {
-          const int S = a.up_s[e0 + j / a.cmax], slot = j % a.cmax;
-          if (slot < a.count[S]) v += phi(T, i, S, slot) * a.charge[(static_cast<int64_t>(S) * kRC + r) * ld + slot];
-        }
-        pf[static_cast<int64_t>(r) * ld + i] = v;
-      }
-    for (int j = first + static_cast<int>(threadIdx.x); j < last; j += kThreads) {
-      const int e = e0 + j / a.cmax, slot = j % a.cmax, S = a.up_s[e];
-      if (S == T || slot >= a.count[S]) continue;
-      for (int r = 0; r < a.Rc; ++r) {
-        double v = 0.0;
-        for (int i = 0; i < c; ++i) v += phi(T, i, S, slot) * a.charge[(static_cast<int64_t>(T) * kRC + r) * ld + i];
-        a.pt[(static_cast<int64_t>(e) * a.Rc + r) * ld + slot] = v;
-      }
-    }
-    return;
-  }
 
   for (int i = threadIdx.x; i < kTable; i += kThreads) table[i] = a.table[i];
   for (int i = threadIdx.x; i < c * RV; i += kThreads)
     *reinterpret_cast<int4*>(trec + (i / RV) * TS + (i % RV) * 4) = a.rec[static_cast<int64_t>(T) * ld * RV + i];
-  for (int i = threadIdx.x; i < c * RC; i += kThreads)
-    reinterpret_cast<int2*>(tq)[i] = a.q[static_cast<int64_t>(T) * ld * RC + i];
-  for (int i = threadIdx.x; i < NW * RC * ld; i += kThreads) {
-    facc[i] = make_longlong2(0, 0);
-    dacc[i] = 0.0;
-  }
+  for (int i = threadIdx.x; i < a.Rc * ld; i += kThreads) tq[i] = a.charge[static_cast<int64_t>(T) * kRC * ld + i];
+  for (int i = threadIdx.x; i < NW * RC * ld; i += kThreads) facc[i] = 0.0;
   __syncthreads();
-  longlong2* fw = facc + warp * RC * ld;
-  double* dw = dacc + warp * RC * ld;
-  double scale[RC];
-#pragma unroll
-  for (int r = 0; r < RC; ++r) scale[r] = a.qscale[r];
-  auto drain = [&]() {   // the target sums hold at most 128 terms
-    for (int i = lane; i < RC * ld; i += 32) {
-      const longlong2 v = fw[i];
-      s64 hh = v.x, m = v.y;
-      dw[i] = flush(hh, m, a.qscale[i / ld], dw[i]);
-      fw[i] = make_longlong2(0, 0);
-    }
-    __syncwarp();
-  };
+  double* fw = facc + warp * RC * ld;
 
   for (int b = 0; b < a.batches; ++b) {
     const int base = first + (b * NW + warp) * 64;
     if (base >= ne * a.cmax) break;
-    int sh[2][DM], sl[2][DM], qh[2][RC], ql[2][RC];
+    int sh[2][DM], sl[2][DM];
+    double q[2][RC];
     int ent[2], slot[2];   // entry of the source, -1: nothing to write
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
@@ -406,31 +334,30 @@ __global__ void __launch_bounds__(kThreads) k_fix_sym(const FixSymArgs a) {
         ok = slot[u] < a.count[S];
       }
       ent[u] = ok && S != T ? e0 + en : -1;
-      const int64_t at = static_cast<int64_t>(S) * ld + (ok ? slot[u] : 0);
+      const int at = ok ? slot[u] : 0;
+      const int4* rec = a.rec + (static_cast<int64_t>(S) * ld + at) * RV;
 #pragma unroll
       for (int k = 0; k < DM; k += 2) {
-        const int4 v = a.rec[at * RV + (k >> 1)];
+        const int4 v = rec[k >> 1];
         sh[u][k] = v.x;
         sl[u][k] = v.y;
         sh[u][k + 1] = v.z;
         sl[u][k + 1] = v.w;
       }
 #pragma unroll
-      for (int r = 0; r < RC; ++r) {
-        const int2 v = ok ? a.q[at * RC + r] : make_int2(0, 0);
-        qh[u][r] = v.x;
-        ql[u][r] = v.y;
-      }
+      for (int r = 0; r < RC; ++r)
+        q[u][r] = ok && r < a.Rc ? a.charge[(static_cast<int64_t>(S) * kRC + r) * ld + at] : 0.0;
     }
-    s64 th[2][RC], tm[2][RC];
+    double tr[2][RC];
 #pragma unroll
     for (int u = 0; u < 2; ++u)
 #pragma unroll
-      for (int r = 0; r < RC; ++r) th[u][r] = tm[u][r] = 0;
+      for (int r = 0; r < RC; ++r) tr[u][r] = 0.0;
     int t = lane;
     for (int s = 0; s < c; ++s) {
-      u64 A[2] = {0, 0}, C[2] = {0, 0}, p[2];
+      u64 A[2] = {0, 0}, C[2] = {0, 0};
       s64 B[2] = {0, 0};
+      double p[2];
       const int4* rec = reinterpret_cast<const int4*>(trec + t * TS);
 #pragma unroll
       for (int k = 0; k < DM; k += 2) {
@@ -446,15 +373,16 @@ __global__ void __launch_bounds__(kThreads) k_fix_sym(const FixSymArgs a) {
           C[u] += static_cast<u64>(static_cast<s64>(l1) * l1);
         }
       }
-      phi56<KER, 2>(A, B, C, a.c, table, p);
+      phi64<KER, 2>(A, B, C, a.c, table, p);
 #pragma unroll
       for (int r = 0; r < RC; ++r) {
-        longlong2 f = fw[r * ld + t];
-        const int2 q = reinterpret_cast<const int2*>(tq)[t * RC + r];
+        if (r % 2 == 0 && r >= a.Rc) break;   // columns in twos
+        double f = fw[r * ld + t];
+        const double x = r < a.Rc ? tq[r * ld + t] : 0.0;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          mac(p[u], qh[u][r], ql[u][r], reinterpret_cast<s64&>(f.x), reinterpret_cast<s64&>(f.y));
-          mac(p[u], q.x, q.y, th[u][r], tm[u][r]);
+          f = fma(p[u], q[u][r], f);
+          tr[u][r] = fma(p[u], x, tr[u][r]);
         }
         fw[r * ld + t] = f;
       }
@@ -466,17 +394,15 @@ __global__ void __launch_bounds__(kThreads) k_fix_sym(const FixSymArgs a) {
       if (ent[u] < 0) continue;
 #pragma unroll
       for (int r = 0; r < RC; ++r)
-        if (r < a.Rc)
-          a.pt[(static_cast<int64_t>(ent[u]) * a.Rc + r) * ld + slot[u]] = flush(th[u][r], tm[u][r], scale[r], 0.0);
+        if (r < a.Rc) a.pt[(static_cast<int64_t>(ent[u]) * a.Rc + r) * ld + slot[u]] = tr[u][r];
     }
-    if (b & 1) drain();
   }
-  drain();
   __syncthreads();
+  double* pf = a.pf + static_cast<int64_t>(chunk) * a.Rc * ld;
   for (int i = threadIdx.x; i < a.Rc * ld; i += kThreads) {
-    double v = dacc[i];
+    double v = facc[i];
 #pragma unroll
-    for (int w = 1; w < NW; ++w) v += dacc[w * RC * ld + i];
+    for (int w = 1; w < NW; ++w) v += facc[w * RC * ld + i];
     pf[i] = v;
   }
 }
@@ -484,12 +410,12 @@ __global__ void __launch_bounds__(kThreads) k_fix_sym(const FixSymArgs a) {
 template <int KER, int DM, int RC>
 void launch_sym(const FixSymArgs& a, int chunks, cudaStream_t s) {
   const size_t smem = fix_sym_smem<DM, RC>(a.ld);
-  if (fix_sym_smem<DM, RC>(ks::kThreads) > 48 * 1024) {
+  if (fix_sym_smem<DM, RC>(kThreads) > 48 * 1024) {
     static std::atomic<uint64_t> done{0};
     const uint64_t bit = device_bit();
     if (!(done.load() & bit)) {
       DW_CUDA(cudaFuncSetAttribute(k_fix_sym<KER, DM, RC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   static_cast<int>(fix_sym_smem<DM, RC>(ks::kThreads))));
+                                   static_cast<int>(fix_sym_smem<DM, RC>(kThreads))));
       done.fetch_or(bit);
     }
   }

@@ -144,7 +144,8 @@ dwfmm_status dwfmm_plan_set_nodes(dwfmm_plan plan, const double* nodes, int64_t 
  * pairs; a pair at distance 0 is never admissible) and the per-cluster
  * expansion data.  `pts` (host or device) holds N x d sites, row-major with
  * leading dimension ld >= d; it is copied.  N = 0 is valid (matvec then does
- * nothing).  Replaces any previous tree.  Synchronises `stream`.
+ * nothing).  Replaces any previous tree, once the calls that use it have
+ * finished on every stream.  Synchronises `stream`.
  * Errors: INVALID_ARG (NULL, ld < d, N < 0, non-finite site), OOM, CUDA. */
 dwfmm_status dwfmm_tree_build(dwfmm_plan plan, const double* pts, int64_t n, int64_t ld,
                               void* stream);

@@ -227,7 +227,9 @@ bool is_device_pointer(const void* p) {
 }
 
 void bind_stream(Plan& P, void* stream) {
-  P.stream = static_cast<cudaStream_t>(stream);
+  const cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (P.have_tree && s != P.stream) P.several_streams = true;
+  P.stream = s;
   DW_CUDA(cudaSetDevice(P.device));
 }
 
@@ -330,6 +332,10 @@ dwfmm_status dwfmm_tree_build(dwfmm_plan plan, const double* pts, int64_t n, int
     if (n < 0 || n > (int64_t(1) << 30)) dw::fail(DWFMM_ERR_INVALID_ARG, "N must be in 0..2^30");
     if (n > 0 && (!pts || ld < P.d)) dw::fail(DWFMM_ERR_INVALID_ARG, "pts is NULL or ld < d");
     bind_stream(P, stream);
+    // the new tree is written into the old one's buffers: calls on another stream
+    // that read them come to their end first
+    if (P.several_streams) DW_CUDA(cudaDeviceSynchronize());
+    P.several_streams = false;
     // a much smaller tree gives the memory back
     if (n < P.N / 4) P.free_tree();
     else P.drop_tree();

@@ -388,6 +388,7 @@ struct Plan {
   double sigma = 1.0, q = 0.0, eta = 1.0;
   std::vector<double> gamma, w;
   cudaStream_t stream = nullptr;   // stream of the last call
+  bool several_streams = false;    // the tree has been used on more than one
   cudaStream_t side = nullptr;     // near field runs here, concurrently with the far field
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int device = 0;

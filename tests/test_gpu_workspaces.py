@@ -42,3 +42,24 @@ def test_solve_replayed_after_a_wider_product(prec, first, wide):
         q.solve(1e-1, f, c, rtol=1e-10, maxit=3000)
         stream.synchronize()
         assert torch.equal(got[0], got[1]) and torch.equal(got[0], c)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_tree_build_waits_for_products_on_other_streams(prec):
+    """New sites on another stream do not touch the tree that a product is
+    still reading."""
+    p, pts, x = setup(prec, n=60000, d=8, r=4, leaf=128, kernel="exp", eta=1.0)
+    want, y = torch.empty_like(x), torch.empty_like(x)
+    p.matvec(x, want)
+    torch.cuda.synchronize()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    other = pts.flip(0).contiguous() * 0.5
+    torch.cuda.synchronize()
+    for _ in range(3):
+        with torch.cuda.stream(a):
+            p.matvec(x, y)
+        with torch.cuda.stream(b):
+            p.tree_build(other)
+            p.tree_build(pts)
+        torch.cuda.synchronize()
+        assert torch.equal(y, want)

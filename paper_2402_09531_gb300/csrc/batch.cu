@@ -596,6 +596,16 @@ void setup_pairs(Batch& B, const PairLists& l) {
     npt += entries * row;
   }
   if (!B.by_pair) return;
+  try {
+    B.rot_pf.alloc(std::max<size_t>(npf, 1));
+    B.rot_pt.alloc(std::max<size_t>(npt, 1));
+  } catch (const ApiError& e) {   // no memory for the sums: the list kernel needs none
+    if (e.status != DWFMM_ERR_OOM) throw;
+    B.rot_pf.release();
+    B.by_pair = false;
+    for (auto& c : B.classes) c.by_pair = false;
+    return;
+  }
   auto put = [](DBuf<int32_t>& d, const std::vector<int32_t>& v) {
     d.alloc(std::max<size_t>(v.size(), 1));
     if (!v.empty()) DW_CUDA(cudaMemcpy(d.p, v.data(), v.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
@@ -607,8 +617,6 @@ void setup_pairs(Batch& B, const PairLists& l) {
   put(B.chunk_t, ct);
   put(B.chunk_ptr, cp);
   put(B.cmax_of, l.cmax_of);
-  B.rot_pf.alloc(std::max<size_t>(npf, 1));
-  B.rot_pt.alloc(std::max<size_t>(npt, 1));
   for (const auto& c : B.classes)
     for (int i = 0; c.by_pair && i < B.P; ++i)
       if (B.leaf_off[i] >= c.leaf_first && B.leaf_off[i] < c.leaf_first + c.leaf_count) {

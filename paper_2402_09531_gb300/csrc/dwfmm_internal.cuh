@@ -539,16 +539,19 @@ struct Plan {
   // graph (the kept conjugate gradient iterations, a caller's own) may hold their
   // addresses, so they stay allocated until the tree goes.
   std::vector<DBuf<unsigned char>> outgrown;
+  // False, and nothing changed, when there is no memory for it: every form with
+  // such a workspace stands beside one without.
   template <class T>
-  void grow(WBuf<T>& b, size_t count) {
+  bool grow(WBuf<T>& b, size_t count) {
     if (!b.p || count > b.n) {
       if (b.tree != tree_gen) b.release();   // another tree's: nothing holds it
       WBuf<T> old(std::move(b));
       try {
         b.alloc(count);
-      } catch (...) {
+      } catch (const ApiError& e) {
         b = std::move(old);
-        throw;
+        if (e.status != DWFMM_ERR_OOM) throw;
+        return false;
       }
       if (old.p) {
         outgrown.emplace_back();
@@ -558,6 +561,7 @@ struct Plan {
       }
     }
     b.tree = tree_gen;
+    return true;
   }
   // Columns to size such a workspace for: the kernels' next count of right-hand
   // sides (at most what the plan takes), so that it grows once per count; fewer

@@ -159,13 +159,12 @@ void p2p_impl(Plan& P, int Rc, const T* pts, const T* xb, T* ynear, cudaStream_t
     const int want = 2 * sm_count();
     if (P.L < want) splits = std::min(16, (want + P.L - 1) / P.L);
   }
-  if (splits == 1) {
+  const int64_t stride = static_cast<int64_t>(P.L) * o_gstride;
+  if (splits == 1 || !P.grow(P.near_parts64, static_cast<size_t>(splits) * stride)) {
     dispatch_ksum<T>(P.kernel, P.L, 0, P.d_near_rowptr.p, P.d_near_col.p, P.d, T(1.0 / P.sigma), pts, side,
                      pts, side, xb, o_gstride, P.m_pad, ynear, o_gstride, P.m_pad, Rc, s);
     return;
   }
-  const int64_t stride = static_cast<int64_t>(P.L) * o_gstride;
-  P.grow(P.near_parts64, static_cast<size_t>(splits) * stride);
   T* part = reinterpret_cast<T*>(P.near_parts64.p);
   dispatch_ksum<T>(P.kernel, P.L, 0, P.d_near_rowptr.p, P.d_near_col.p, P.d, T(1.0 / P.sigma), pts, side, pts,
                    side, xb, o_gstride, P.m_pad, part, o_gstride, P.m_pad, Rc, s, splits, stride);
@@ -369,8 +368,7 @@ bool near_sym(Plan& P, int Rc, cudaStream_t s) {
   const size_t most = kSymMaxBytes / (2 * col * sizeof(double));
   if (most < static_cast<size_t>(Rc)) return false;
   const size_t cols = P.work_cols(Rc, Rc <= 1 ? 1 : kSymMaxRc, most);
-  P.grow(P.sym_pf, col * cols);
-  P.grow(P.sym_pt, col * cols);
+  if (!P.grow(P.sym_pf, col * cols) || !P.grow(P.sym_pt, col * cols)) return false;
   switch (P.kernel) {
     case DWFMM_K_EXP: launch_near_sym_k<DWFMM_K_EXP>(P, Rc, s); break;
     case DWFMM_K_MATERN32: launch_near_sym_k<DWFMM_K_MATERN32>(P, Rc, s); break;

@@ -456,21 +456,22 @@ bool p2p_f32_tuned(Plan& P, int Rc, bool rot, bool steady, cudaStream_t s) {
   // (d = 10 Gaussian, N = 3362, 12 right-hand sides, 16 leaves: the product
   // took 177 us in one part, 45 us in 16)
   const int splits = std::max(1, std::min(16, 4 * sm_count() / P.L));
-  if (steady && splits > 1 &&
-      static_cast<size_t>(P.nnear) * Rc * P.m_pad * sizeof(float) <= kEntryPartsBytes) {
+  const size_t col = static_cast<size_t>(P.nnear) * P.m_pad;   // one sum per entry
+  const size_t most = kEntryPartsBytes / (col * sizeof(float));
+  const int64_t part = static_cast<int64_t>(P.L) * a.out_gstride;
+  if (steady && splits > 1 && most >= static_cast<size_t>(Rc) &&
+      P.grow(P.entry_parts32, col * P.work_cols(Rc, RC, most))) {
     // every entry's sum by itself, then in list order with the compensation
     // that one CTA per leaf would carry: the same bits, on all SMs
     // (N = 3001, d = 16: 174 us with 32 CTAs)
     a.entry_t = P.d_near_pairs.p;
     a.entry_off = P.L - 1;
     a.out_gstride = static_cast<int64_t>(Rc) * P.m_pad;
-    const size_t col = static_cast<size_t>(P.nnear) * P.m_pad;
-    P.grow(P.entry_parts32, col * P.work_cols(Rc, RC, kEntryPartsBytes / (col * sizeof(float))));
     a.out = P.entry_parts32.p;
     dispatch(D, P.kernel, RC, a, static_cast<int>(P.nnear), threads, smem, s);
     k_fold_entries<<<ceil_div(static_cast<int64_t>(P.L) * Rc * P.m_pad, 128), 128, 0, s>>>(
         P.entry_parts32.p, P.d_near_rowptr.p, P.L, P.m_pad, Rc, P.ynear32.p);
-  } else if (splits > 1 && !steady) {
+  } else if (splits > 1 && !steady && P.grow(P.near_parts32, static_cast<size_t>(splits) * part)) {
     if (!P.part_rows.p) {   // once per tree
       P.part_rows.alloc(static_cast<size_t>(P.L) * splits + 1);
       k_part_rows<<<ceil_div(static_cast<int64_t>(P.L) * splits + 1, 256), 256, 0, s>>>(P.d_near_rowptr.p, P.L, splits,
@@ -478,8 +479,7 @@ bool p2p_f32_tuned(Plan& P, int Rc, bool rot, bool steady, cudaStream_t s) {
     }
     a.rowptr = P.part_rows.p;
     a.row_step = a.parts = splits;
-    a.split_stride = static_cast<int64_t>(P.L) * a.out_gstride;
-    P.grow(P.near_parts32, static_cast<size_t>(splits) * a.split_stride);
+    a.split_stride = part;
     a.out = P.near_parts32.p;
     dispatch(D, P.kernel, RC, a, P.L, threads, smem, s);
     k_add_parts<<<ceil_div(static_cast<int64_t>(P.L) * Rc * P.m_pad, 256), 256, 0, s>>>(

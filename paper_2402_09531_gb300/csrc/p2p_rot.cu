@@ -113,7 +113,8 @@ bool row_chunks(Plan& P, int per, int least, RowChunks& out) {
 // tree's chunks on first use.  Called before the side stream forks.  Above 8
 // right-hand sides the sums of both sides leave the registers (and MIXED plans
 // have the tensor cores); leaves below 32 sites would make lanes of a turn
-// share a target; partial sums beyond 8 GB are not worth their traffic.
+// share a target; partial sums beyond 8 GB are not worth their traffic, and where
+// there is no memory for them the list kernel needs none.
 bool rot_ready(Plan& P, int Rc) {
   if (sum_padded_dim(P.d) < 0 || !rot_fits(P.m_pad, kRotMinLeaf, sum_padded_rc(Rc))) return false;
   if (P.rot_state < 0 && capturing(P.stream)) return false;   // the chunks are built outside a capture
@@ -123,9 +124,7 @@ bool rot_ready(Plan& P, int Rc) {
   const size_t most = kRotMaxBytes / ((static_cast<size_t>(P.rot.n) + P.sym_nup) * row * sizeof(float));
   if (most < static_cast<size_t>(Rc)) return false;
   const size_t cols = P.work_cols(Rc, sum_padded_rc(Rc), most);
-  P.grow(P.rot_pf, P.rot.n * row * cols);
-  P.grow(P.rot_pt, P.sym_nup * row * cols);
-  return true;
+  return P.grow(P.rot_pf, P.rot.n * row * cols) && P.grow(P.rot_pt, P.sym_nup * row * cols);
 }
 
 // pts: scaled blocks of the leaves; charges in P.xq32.

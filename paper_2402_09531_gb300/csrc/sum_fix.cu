@@ -118,8 +118,15 @@ bool fix_ready(Plan& P) {
   if (!fx::make_consts(P.kernel, P.sigma, P.fx_F, P.fx_c)) return false;
   const int DM = padded_d(P.d);
   const int64_t nl = static_cast<int64_t>(P.L) * P.m_pad, nc = static_cast<int64_t>(P.C) * P.n_pad;
-  P.fx_pts.alloc(nl * 2 * DM);
-  P.fx_nodes.alloc(nc * 2 * DM);
+  try {
+    P.fx_pts.alloc(nl * 2 * DM);
+    P.fx_nodes.alloc(nc * 2 * DM);
+  } catch (const ApiError& e) {   // no memory for the records: the float64 unit, for this tree
+    if (e.status != DWFMM_ERR_OOM) throw;
+    P.fx_pts.release();
+    P.fx_nodes.release();
+    return false;
+  }
   if (!P.fx_table.p) {
     fx::u64 t[fx::kTable];
     fx::make_table(t);
@@ -143,10 +150,9 @@ bool near_fix(Plan& P, int Rc, cudaStream_t s) {
   size_t most = 0;   // columns of partial sums
   if (P.fx_sym == 1 && RC <= 4)
     most = kSymMaxBytes / ((static_cast<size_t>(P.fx_rows.n) + P.sym_nup) * P.m_pad * sizeof(double));
-  if (most >= static_cast<size_t>(Rc)) {
-    const size_t cols = P.work_cols(Rc, RC, most);
-    P.grow(P.sym_pf, P.fx_rows.n * cols * P.m_pad);
-    P.grow(P.sym_pt, P.sym_nup * cols * P.m_pad);
+  const size_t cols = P.work_cols(Rc, RC, most);
+  if (most >= static_cast<size_t>(Rc) && P.grow(P.sym_pf, P.fx_rows.n * cols * P.m_pad) &&
+      P.grow(P.sym_pt, P.sym_nup * cols * P.m_pad)) {
     FixSymArgs b{};
     b.rec = reinterpret_cast<const int4*>(P.fx_pts.p);
     b.charge = P.xb64.p;
@@ -189,13 +195,13 @@ bool near_fix(Plan& P, int Rc, cudaStream_t s) {
   const int want = 8 * sm_count();
   a.splits = 1;
   if (P.L * a.passes < want) a.splits = std::min(16, ceil_div(want, P.L * a.passes));
+  const int64_t stride = static_cast<int64_t>(P.L) * a.o_gstride;
+  if (a.splits > 1 && !P.grow(P.near_parts64, static_cast<size_t>(a.splits) * stride)) a.splits = 1;
   const int ctas = P.L * a.passes * a.splits;
   if (a.splits == 1) {
     a.out = P.ynear64.p;
     dispatch(P.kernel, P.d, RC, a, ctas, s);
   } else {
-    const int64_t stride = static_cast<int64_t>(P.L) * a.o_gstride;
-    P.grow(P.near_parts64, static_cast<size_t>(a.splits) * stride);
     a.out = P.near_parts64.p;
     a.split_stride = stride;
     dispatch(P.kernel, P.d, RC, a, ctas, s);

@@ -63,3 +63,31 @@ def test_tree_build_waits_for_products_on_other_streams(prec):
             p.tree_build(pts)
         torch.cuda.synchronize()
         assert torch.equal(y, want)
+
+
+# partial sums of 42 MB (float32) or 84 MB (float64) a right-hand side
+@pytest.mark.parametrize("prec,r,engines", [("fp64", 4, ("fp64_list", "fp64_symmetric")), ("fp32", 8, None),
+                                            ("mixed", 8, None)])
+def test_products_without_memory_for_partial_sums(prec, r, engines):
+    """The list kernel runs where the pairs' partial sums cannot be allocated."""
+    p, pts, x = setup(prec, n=40000, d=8, leaf=128, kernel="exp")
+    want = torch.empty_like(x)
+    p.matvec(x, want)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    block = torch.empty(torch.cuda.mem_get_info()[0] - (160 << 20), dtype=torch.uint8, device="cuda")
+    y = torch.empty_like(x[:r])
+    bound = 1e-13 if prec == "fp64" else 1e-5
+    try:
+        p.matvec(x[:r].contiguous(), y)
+        torch.cuda.synchronize()
+        few = p.near_engine()
+    finally:
+        del block
+        torch.cuda.empty_cache()
+    assert float(torch.linalg.norm(y - want[:r]) / torch.linalg.norm(want[:r])) <= bound
+    y2 = torch.empty_like(y)
+    p.matvec(x[:r].contiguous(), y2)
+    assert float(torch.linalg.norm(y2 - want[:r]) / torch.linalg.norm(want[:r])) <= bound
+    if engines:
+        assert (few, p.near_engine()) == engines

@@ -156,7 +156,11 @@ dwfmm_status dwfmm_tree_build(dwfmm_plan plan, const double* pts, int64_t n, int
  * >= N, caller's site order.  x and y must not overlap.  With device
  * pointers the call returns once the work is enqueued on `stream`; with a
  * host y it synchronises `stream` before returning.
- * A product that the caller captured into a CUDA graph may be replayed until
+ * After a first product with the tree (MIXED plans: one with more than 8
+ * right-hand sides, if more than 8 are to be captured), the call may be captured
+ * into a CUDA graph with any number of right-hand sides.  Workspaces that no
+ * product outside a capture has needed are not allocated in one: the captured
+ * product may then take a slower form.  A captured product may be replayed until
  * the next dwfmm_tree_build or dwfmm_plan_destroy on the plan, whatever other
  * calls run in between (ordered with it): the workspaces it uses stay where
  * they are for as long as the tree does.

@@ -46,6 +46,12 @@ struct ApiError {
 
 inline void fail(dwfmm_status s, const std::string& m) { throw ApiError{s, m}; }
 
+inline bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  DW_CUDA(cudaStreamIsCapturing(s, &cs));
+  return cs != cudaStreamCaptureStatusNone;
+}
+
 // Device buffer with explicit lifetime (freed by the plan).
 template <class T>
 struct DBuf {
@@ -539,11 +545,13 @@ struct Plan {
   // graph (the kept conjugate gradient iterations, a caller's own) may hold their
   // addresses, so they stay allocated until the tree goes.
   std::vector<DBuf<unsigned char>> outgrown;
-  // False, and nothing changed, when there is no memory for it: every form with
-  // such a workspace stands beside one without.
+  // False, and nothing changed, when there is no memory for it or the stream is
+  // capturing (a capture can hold no allocation): every form with such a workspace
+  // stands beside one without.
   template <class T>
   bool grow(WBuf<T>& b, size_t count) {
     if (!b.p || count > b.n) {
+      if (capturing(stream)) return false;
       if (b.tree != tree_gen) b.release();   // another tree's: nothing holds it
       WBuf<T> old(std::move(b));
       try {
@@ -633,11 +641,6 @@ void launch_scatter_batched(const ProbF32* probs, const int* leaf_off, int P, in
                             const BatchParts& parts, const float* ynear, const float* yfar, cudaStream_t s);
 void launch_rot(int D, int kernel, int RC, const RotArgs& a, int chunks, cudaStream_t s);   // p2p_rot.cu
 int rot_sources_per_chunk();
-inline bool capturing(cudaStream_t s) {
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  DW_CUDA(cudaStreamIsCapturing(s, &cs));
-  return cs != cudaStreamCaptureStatusNone;
-}
 bool rot_fits(int ld, int least, int rc);   // slots, sites of the smallest leaf, padded right-hand sides
 size_t persist_rot_bytes(int D, int RC, int ld);
 // persistent batch matvec: dynamic shared memory and resident CTAs per SM

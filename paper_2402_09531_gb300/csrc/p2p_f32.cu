@@ -471,8 +471,9 @@ bool p2p_f32_tuned(Plan& P, int Rc, bool rot, bool steady, cudaStream_t s) {
     dispatch(D, P.kernel, RC, a, static_cast<int>(P.nnear), threads, smem, s);
     k_fold_entries<<<ceil_div(static_cast<int64_t>(P.L) * Rc * P.m_pad, 128), 128, 0, s>>>(
         P.entry_parts32.p, P.d_near_rowptr.p, P.L, P.m_pad, Rc, P.ynear32.p);
-  } else if (splits > 1 && !steady && P.grow(P.near_parts32, static_cast<size_t>(splits) * part)) {
-    if (!P.part_rows.p) {   // once per tree
+  } else if (splits > 1 && !steady && (P.part_rows.p || !capturing(P.stream)) &&
+             P.grow(P.near_parts32, static_cast<size_t>(splits) * part)) {
+    if (!P.part_rows.p) {   // once per tree, outside a capture
       P.part_rows.alloc(static_cast<size_t>(P.L) * splits + 1);
       k_part_rows<<<ceil_div(static_cast<int64_t>(P.L) * splits + 1, 256), 256, 0, s>>>(P.d_near_rowptr.p, P.L, splits,
                                                                                        P.part_rows.p);

@@ -91,3 +91,30 @@ def test_products_without_memory_for_partial_sums(prec, r, engines):
     assert float(torch.linalg.norm(y2 - want[:r]) / torch.linalg.norm(want[:r])) <= bound
     if engines:
         assert (few, p.near_engine()) == engines
+
+
+@pytest.mark.parametrize("prec,first,r", [("fp64", 1, 4), ("fp64", 1, 16), ("fp32", 1, 8), ("fp32", 1, 12),
+                                          ("mixed", 2, 8), ("mixed", 9, 16)])
+def test_capture_of_a_wider_product(prec, first, r):
+    """A product with more right-hand sides than any before, captured; and the
+    same graph after its workspaces grew outside."""
+    p, pts, x = setup(prec)
+    y, want = torch.empty_like(x), torch.empty_like(x)
+    p.matvec(x[:first].contiguous(), y[:first].contiguous())
+    torch.cuda.synchronize()
+    xr, yr = x[:r].contiguous(), torch.empty_like(x[:r])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        p.matvec(xr, yr)
+    yr.fill_(float("nan"))
+    graph.replay()
+    torch.cuda.synchronize()
+    got = yr.clone()
+    p.matvec(xr, want[:r])
+    bound = 1e-13 if prec == "fp64" else 1e-5
+    assert float(torch.linalg.norm(got - want[:r]) / torch.linalg.norm(want[:r])) <= bound
+    p.matvec(x, want)
+    yr.fill_(float("nan"))
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(yr, got)

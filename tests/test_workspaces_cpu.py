@@ -23,6 +23,11 @@ extern "C" cudaError_t cudaMalloc(void** p, size_t n) {
 }
 extern "C" cudaError_t cudaFree(void* p) { live.erase(p); free(p); return cudaSuccess; }
 extern "C" cudaError_t cudaGetLastError() { return cudaSuccess; }
+static bool in_capture = false;
+extern "C" cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
+  *s = in_capture ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+  return cudaSuccess;
+}
 #define CHECK(c) if (!(c)) { printf("line %d: %s\n", __LINE__, #c); return 1; }
 int main() {
   dw::Plan P;
@@ -38,6 +43,9 @@ int main() {
   CHECK(!P.grow(P.rot_pf, 800))                // no room
   CHECK(P.rot_pf.p == wide && P.rot_pf.n == 400 && live.count(wide))
   room = 1 << 20;
+  in_capture = true;
+  CHECK(!P.grow(P.rot_pf, 800) && P.grow(P.rot_pf, 400) && P.rot_pf.p == wide && live.size() == 2)
+  in_capture = false;
   P.outgrown.clear();                          // the tree goes
   ++P.tree_gen;
   CHECK(!live.count(narrow) && live.count(wide))

@@ -635,7 +635,7 @@ dwfmm_status dwfmm_cg_step(dwfmm_plan plan, int32_t iters, void* stream) {
   if (!plan) return DWFMM_ERR_INVALID_ARG;
   Plan& P = plan->P;
   return guarded(&P, [&]() -> dwfmm_status {
-    if (!P.cgs.active) dw::fail(DWFMM_ERR_STATE, "cg_step before cg_begin");
+    if (!P.cgs.active || !P.cg_p.p) dw::fail(DWFMM_ERR_STATE, "cg_step before cg_begin (since the tree was built)");
     if (iters < 0) dw::fail(DWFMM_ERR_INVALID_ARG, "iters < 0");
     bind_stream(P, stream);
     dw::cg_step(P, iters);
@@ -657,7 +657,7 @@ dwfmm_status dwfmm_cg_result(dwfmm_plan plan, double* c, int64_t ld, void* strea
   if (!plan) return DWFMM_ERR_INVALID_ARG;
   Plan& P = plan->P;
   return guarded(&P, [&]() -> dwfmm_status {
-    if (!P.cgs.active) dw::fail(DWFMM_ERR_STATE, "cg_result before cg_begin");
+    if (!P.cgs.active || !P.cg_p.p) dw::fail(DWFMM_ERR_STATE, "cg_result before cg_begin (since the tree was built)");
     if (!c || ld < P.N) dw::fail(DWFMM_ERR_INVALID_ARG, "NULL buffer or ld < N");
     bind_stream(P, stream);
     dw::cg_result(P, c, ld);

@@ -32,3 +32,23 @@ def test_incremental_iterates_are_the_solves(kernel, n, nrhs, leaf, seed):
     _, status, iters, _ = plans[1].cg_poll()
     assert np.all(status == 1) and int(iters.max()) == its
     assert torch.equal(c, inc)
+
+
+def test_iterations_after_a_new_tree_need_a_new_begin():
+    """The vectors of the iterations go with the tree: refused on the host."""
+    from paper_2402_09531_gb300 import DwfmmError, Plan
+    p = Plan(d=3, kernel="exp", gamma=np.ones(3), q=1.0, leaf_size=64, precision="fp32", max_rhs=1)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    pts = torch.rand((500, 3), dtype=torch.float64, device="cuda", generator=g)
+    f = torch.randn((1, 500), dtype=torch.float64, device="cuda", generator=g)
+    p.tree_build(pts)
+    p.cg_begin(1.0, f)
+    p.cg_step(2)
+    p.tree_build(pts)
+    for call in (lambda: p.cg_step(1), lambda: p.cg_result(torch.empty_like(f))):
+        with pytest.raises(DwfmmError) as e:
+            call()
+        assert e.value.status == 7
+    p.cg_begin(1.0, f)
+    p.cg_step(2)
+    torch.cuda.synchronize()

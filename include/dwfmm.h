@@ -336,7 +336,9 @@ dwfmm_status dwfmm_batch_set_engine(dwfmm_batch batch, int32_t engine);
  * Ap = K_tilde p of all problems as one fused batch matvec and updates all
  * problems' vectors with fused kernels; the per-column decisions are those of
  * dwfmm_cg_step (a column stops on convergence or breakdown, the others go
- * on).  Enqueued on `stream`; afterwards each plan's dwfmm_cg_poll and
+ * on).  Enqueued on `stream` (the first call on a batch with several
+ * right-hand-side classes times the shapes of its near field, synchronising the
+ * device first, unless `stream` is capturing); afterwards each plan's dwfmm_cg_poll and
  * dwfmm_cg_result read its state as after dwfmm_cg_step.  Inner products use
  * a fixed partition, so the result does not depend on timing.  Errors:
  * DWFMM_ERR_STATE if a plan has no CG begun, DWFMM_ERR_INVALID_ARG if its

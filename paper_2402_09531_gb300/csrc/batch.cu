@@ -54,6 +54,10 @@ struct Batch {
   // threads) and right-hand-side grouping, separately for the fused near
   // field and the fused couplings
   int thr_near = 0, thr_m2l = 0;
+  // the list form's own, which the CG iterations run where products evaluate
+  // each pair once (tune_list; 0: not chosen yet, the widest padded)
+  int thr_list = 0;
+  bool split_list = false;
   bool split_m2l = false;
   cudaStream_t stream = nullptr, side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_copy = nullptr;
@@ -247,7 +251,8 @@ void enqueue_matvec(Batch& B, bool io = true, bool steady = false) {
   if (io) launch_gather_batched(B.probs.p, B.d_leaf_off.p, B.P, B.Ltot, B.ld, B.xb.p, s);
   DW_CUDA(cudaEventRecord(B.ev_fork, s));
   DW_CUDA(cudaStreamWaitEvent(B.side, B.ev_fork, 0));
-  enqueue_near(B, B.split, B.thr_near, by_pair, B.side);
+  if (B.by_pair && !by_pair) enqueue_near(B, B.split_list, B.thr_list ? B.thr_list : threads_for(B.ld), false, B.side);
+  else enqueue_near(B, B.split, B.thr_near, by_pair, B.side);
   DW_CUDA(cudaEventRecord(B.ev_join, B.side));
   for (size_t h = 0; h < B.up_off.size(); ++h)
     launch_moments_batched(B.probs.p, B.work.p + B.up_off[h], B.up_cnt[h], B.far_smem, steady, s);
@@ -263,14 +268,14 @@ void enqueue_matvec(Batch& B, bool io = true, bool steady = false) {
 
 // Best of two timed runs of one launch shape of the near field (which = 0)
 // or the couplings (which = 1).
-double time_shape(Batch& B, int which, bool split, int threads) {
+double time_shape(Batch& B, int which, bool split, int threads, bool by_pair) {
   cudaEvent_t a, b;
   DW_CUDA(cudaEventCreate(&a));
   DW_CUDA(cudaEventCreate(&b));
   float best = 1e30f;
   for (int rep = 0; rep < 2; ++rep) {
     DW_CUDA(cudaEventRecord(a, B.stream));
-    if (which == 0) enqueue_near(B, split, threads, B.by_pair, B.stream);
+    if (which == 0) enqueue_near(B, split, threads, by_pair, B.stream);
     else enqueue_m2l(B, split, threads, B.stream);
     DW_CUDA(cudaEventRecord(b, B.stream));
     DW_CUDA(cudaEventSynchronize(b));
@@ -298,12 +303,12 @@ void tune_shapes(Batch& B) {
     bool bsplit = false;
     int bthr = widest;
     if (which == 0 && B.by_pair) {   // one shape: a launch per class, whole CTAs
-      best = bp = bs = time_shape(B, which, can_split, widest);
+      best = bp = bs = time_shape(B, which, can_split, widest, true);
       bsplit = can_split;
     }
     for (int thr = which == 0 && B.by_pair ? widest + 1 : 32; thr <= widest; thr = (thr * 2 > widest && thr < widest) ? widest : thr * 2) {
       for (int sp = 0; sp < (can_split ? 2 : 1); ++sp) {
-        const double ms = time_shape(B, which, sp != 0, thr);
+        const double ms = time_shape(B, which, sp != 0, thr, false);
         if (sp) bs = std::min(bs, ms);
         else bp = std::min(bp, ms);
         if (ms < best) {
@@ -325,6 +330,31 @@ void tune_shapes(Batch& B) {
   }
   B.tune_ms[0] = best_pad;
   B.tune_ms[1] = best_split;
+}
+
+// Shape of the near field's list form for the CG iterations of a batch whose
+// products evaluate each pair once: with several right-hand-side classes one
+// padded launch or one per class, whichever is faster (16 Matern problems, classes
+// of 1, 4 and 8: an iteration takes 3.6 ms with a launch per class of 64 threads,
+// 2.1 ms padded).  Timed before the first iterations, not at creation, which
+// products pay for too.  One class: the widest shape was the fastest in every
+// batch measured.
+void tune_list(Batch& B) {
+  const int widest = threads_for(B.ld);
+  B.thr_list = widest;
+  B.split_list = false;
+  if (B.classes.size() < 2) return;
+  DW_CUDA(cudaDeviceSynchronize());   // the timing runs overwrite the batch's buffers
+  double best = 1e30;
+  for (int thr = 32; thr <= widest; thr = (thr * 2 > widest && thr < widest) ? widest : thr * 2)
+    for (int sp = 0; sp < 2; ++sp) {
+      const double ms = time_shape(B, 0, sp != 0, thr, false);
+      if (ms < best) {
+        best = ms;
+        B.thr_list = thr;
+        B.split_list = sp != 0;
+      }
+    }
 }
 
 // --- persistent engine -------------------------------------------------------
@@ -1075,6 +1105,7 @@ void batch_cg_step(Batch& B, int iters, cudaStream_t s) {
   const CgPtrs* d_items = reinterpret_cast<const CgPtrs*>(B.cg_tab.p);
   const BcgSeg* d_segs = reinterpret_cast<const BcgSeg*>(B.cg_tab.p + bi);
   const int2* d_blk = reinterpret_cast<const int2*>(B.cg_tab.p + bi + bs);
+  if (B.by_pair && B.thr_list == 0 && !capturing(s)) tune_list(B);
   // `iters` iterations captured once per (iteration count, table shape) on the
   // batch's stream and replayed on the caller's
   if (iters > 0 && (!B.cg_exec || B.cg_iters != iters || B.cg_nseg != nseg || B.cg_nblk != nblk)) {

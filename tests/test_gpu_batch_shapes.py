@@ -67,3 +67,35 @@ def test_product_between_batched_iterations():
         got.append(cs)
     assert all(torch.equal(a, c) for a, c in zip(*got))
     b.close()
+
+
+@pytest.mark.parametrize("r", [(1, 3, 8), (2, 12), (16, 5)])
+def test_batched_iterations_with_several_classes(r):
+    """Iterations of a batch whose right-hand sides fall into several classes
+    (products evaluate each pair once, the iterations run the list form)."""
+    from paper_2402_09531_gb300 import Batch, Plan
+    g = torch.Generator(device="cuda").manual_seed(8)
+    plans, fs = [], []
+    for i, k in enumerate(r):
+        n = 1100 + 300 * i
+        p = Plan(4, kernel="matern32", gamma=np.ones(4), q=2.0, leaf_size=64, precision="fp32", max_rhs=k)
+        p.tree_build(torch.rand((n, 4), dtype=torch.float64, device="cuda", generator=g))
+        plans.append(p)
+        fs.append(torch.randn((k, n), dtype=torch.float64, device="cuda", generator=g))
+    b = Batch(plans, list(r))
+    got = []
+    for step in (b.cg_step, lambda it: [p.cg_step(it) for p in plans]):
+        for p, f in zip(plans, fs):
+            p.cg_begin(50.0, f, rtol=1e-12)
+        step(2)
+        step(3)
+        cs = [torch.empty_like(f) for f in fs]
+        for p, c in zip(plans, cs):
+            p.cg_result(c)
+        torch.cuda.synchronize()
+        got.append(cs)
+    # five iterations with a condition number of about 20: the float32 operator's
+    # rounding (256 2^-24 of a row's sum) enters each of them
+    for x, y in zip(*got):
+        assert float(torch.linalg.norm(x - y) / torch.linalg.norm(y)) <= 1e-4
+    b.close()

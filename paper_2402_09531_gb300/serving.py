@@ -78,11 +78,21 @@ def estimate_bytes(n: int, d: int, nrhs: int, leaf: int, n_x: int) -> int:
     n_pad = (n_x + 7) // 8 * 8
     per_site = d * 8 * 6 + 16 * 4 * 8 + 16 * 8 * 4 + nrhs * 8 * 8 + 64
     per_cluster = n_pad * 16 * 4 * 8 + n_pad * (d + 1) * 12 + d * 8 * 6
-    near_pairs = leaves * 64
-    # partial sums of the symmetric float64 near field (also run by the
-    # float64 residuals of float32 / mixed plans): 2 x upper entries x RHS x leaf
-    sym_partials = near_pairs * nrhs * leaf * 8
-    return int(n * per_site + clusters * per_cluster + near_pairs * 24 + sym_partials + (32 << 20))
+    near_pairs = leaves * min(leaves, 256)
+    upper = near_pairs // 2 + leaves
+    # columns that the workspaces are sized for (the kernels' counts)
+    cols = next((c for c in (1, 4, 8, 16) if nrhs <= c), 16)
+    # partial sums of the near fields that evaluate each pair once: float64 (also
+    # run by the float64 residuals of float32 / mixed plans) and float32, at most
+    # 8 GB each; one sum per near entry of the float32 iterations, at most 256 MB;
+    # split lists of small trees
+    partials = min(upper * (2 + leaf // 64) * cols * leaf * 8, 8 << 30)
+    partials += min(upper * (2 + leaf // 512) * cols * leaf * 4, 8 << 30)
+    partials += min(near_pairs * cols * leaf * 4, 256 << 20)
+    partials += min(16 * leaves, 2400) * leaf * 16 * 12
+    # fixed-point records of the sites and nodes (float64 sums)
+    records = 2 * 16 * 4 * (leaves * leaf + clusters * n_pad)
+    return int(n * per_site + clusters * per_cluster + near_pairs * 24 + partials + records + (64 << 20))
 
 
 @dataclass

@@ -118,3 +118,28 @@ def test_capture_of_a_wider_product(prec, first, r):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(yr, got)
+
+
+@pytest.mark.parametrize("prec,n,nrhs", [("fp64", 20000, 1), ("mixed", 20000, 4), ("fp32", 3000, 1)])
+def test_admission_estimate_covers_a_request(prec, n, nrhs):
+    """Device memory of a plan that multiplied, iterated and took a residual."""
+    from paper_2402_09531_gb300 import Plan
+    from paper_2402_09531_gb300.serving import estimate_bytes
+    d = 16
+    gamma = 2.0 ** -np.arange(d)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    pts = (2 * torch.rand((n, d), dtype=torch.float64, device="cuda", generator=g) - 1) * torch.as_tensor(gamma, device="cuda")
+    f = torch.randn((nrhs, n), dtype=torch.float64, device="cuda", generator=g)
+    c, y = torch.zeros_like(f), torch.empty_like(f)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    p = Plan(d, kernel="exp", gamma=gamma, q=6.0, leaf_size=128, precision=prec, max_rhs=nrhs)
+    p.tree_build(pts)
+    p.matvec(f, y)
+    p.cg_begin(10.0, f)
+    p.cg_step(2)
+    p.cg_result(c)
+    p.residual(10.0, f, c)
+    torch.cuda.synchronize()
+    used = before - torch.cuda.mem_get_info()[0]
+    assert used <= estimate_bytes(n, d, nrhs, 128, p.info()[0]), used
